@@ -30,6 +30,7 @@ extern "C" const void* const jacc_tab_7_64_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_7_32_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_64_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_32_out[JACC_NTILES];
+extern "C" const void* const jacc_tab_27_64_w32[JACC_NTILES];
 extern "C" const void* const jacc_tab_tb[2];
 
 namespace jacc {
@@ -129,7 +130,10 @@ static int plan_fixed(const jacc_kernel_desc& d, JParams& p) {
       if (sh >= 64 || (m[j] >> (63 - sh)) != 0) return p.fpath;  // factor must stay below 2^63
       f[j] = static_cast<i64>(m[j] << sh);
     }
-    p.fpath = JACC_FP_WIDE;
+    // weights with few bits (FP32 weights, say) take the kernel's 32-bit products
+    bool narrow = K >= 1 && K <= 31;
+    for (int j = 0; j < 4; ++j) narrow = narrow && f[j] < (static_cast<i64>(1) << 31);
+    p.fpath = narrow ? JACC_FP_W32 : JACC_FP_WIDE;
     p.fw0 = f[0];
     p.fw1 = f[1];
     p.fw2 = f[2];
@@ -202,6 +206,13 @@ int default_tile(const jacc_kernel_desc& d) {
 
 bool staged_tile(const jacc_kernel_desc& d, int t) {
   return kTiles[t].vec16 && (d.stencil == 7 || (d.stencil == 27 && d.dtype == 32));
+}
+
+// Tiles whose planes are staged by asynchronous copies, one column of
+// JACC_RING_ROWS rows per thread.
+static bool ring_tile(const jacc_kernel_desc& d, int t) {
+  (void)t;
+  return d.stencil == 27 && d.dtype == 64;
 }
 
 bool tile_valid(const jacc_kernel_desc& d, int t) {
@@ -355,14 +366,17 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   p.c3 = desc->coeffs[3];
   plan_fixed(*desc, p);
   k->block = dim3(c.bx, c.by, 1);
-  const int64_t tx = static_cast<int64_t>(c.bx) * k->vec;
+  const bool ring = ring_tile(*desc, tile);
+  const int64_t tx = static_cast<int64_t>(c.bx) * (ring ? 1 : k->vec);
+  p.zc = plane_chunk(*desc, tile);
   if (desc->stencil == 5) {
     const int64_t ty = static_cast<int64_t>(c.by) * (c.zc / 4);
     k->grid = dim3(static_cast<unsigned>((desc->nx + tx - 1) / tx), static_cast<unsigned>((desc->ny + ty - 1) / ty), 1);
   } else {
     // the staged kernels (16-byte columns: 7-point, and 27-point FP32) give each thread 2 rows
-    const int64_t ty = static_cast<int64_t>(c.by) * (staged_tile(*desc, tile) ? 2 : 1);
-    const int64_t zc = plane_chunk(*desc, tile);
+    const int64_t ty = static_cast<int64_t>(c.by) *
+                       (ring ? JACC_RING_ROWS(c.bx, c.by) : (staged_tile(*desc, tile) ? 2 : 1));
+    const int64_t zc = p.zc;
     k->grid = dim3(static_cast<unsigned>((desc->nx + tx - 1) / tx), static_cast<unsigned>((desc->ny + ty - 1) / ty),
                    static_cast<unsigned>((desc->nz + zc - 1) / zc));
   }
@@ -402,6 +416,7 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
     k->jit = true;
   } else {
     k->func = table_entry(desc->stencil, desc->dtype, tile, false);
+    if (p.fpath == JACC_FP_W32) k->func = jacc_tab_27_64_w32[tile];
     k->func_out = table_entry(desc->stencil, desc->dtype, tile, true);
     if (!k->func || !k->func_out) return fail(JACC_ERR_UNSUPPORTED, "no precompiled kernel for this descriptor");
   }

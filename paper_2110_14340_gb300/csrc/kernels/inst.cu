@@ -16,8 +16,11 @@ typedef float JT;
 #define JKERN(BX, BY, V, ZC, O) jacc_k_jacobi2d<JT, BX, BY, V, (ZC) / 4, O>
 #elif JACC_INST_STENCIL == 7
 #define JKERN(BX, BY, V, ZC, O) jacc_k_heat3d<JT, BX, BY, V, ZC, O>
+#elif JACC_INST_DTYPE == 64
+// the planes per CTA are a launch parameter: one kernel for both marches
+#define JKERN(BX, BY, V, ZC, O) jacc_k_box27<JT, BX, BY, V, 0, O, JParams>
 #else
-#define JKERN(BX, BY, V, ZC, O) jacc_k_box27<JT, BX, BY, V, ZC, O>
+#define JKERN(BX, BY, V, ZC, O) jacc_k_box27<JT, BX, BY, V, ZC, O, JParams>
 #endif
 
 #define JCAT3(a, b, c) a##b##_##c
@@ -33,3 +36,10 @@ typedef float JT;
 // store; identical to table 1 for FP32.
 extern "C" const void* const JTABNAME(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY)};
 extern "C" const void* const JTABOUT(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY_OUT)};
+
+#if JACC_INST_STENCIL == 27 && JACC_INST_DTYPE == 64
+// Table 1 for weights with 32-bit fixed-point factors (JACC_FP_W32).
+#define JENTRY_W32(id, BX, BY, VEC, ZC) \
+  (const void*)jacc_k_box27<JT, BX, BY, ((VEC) ? JVEC : 1), 0, false, JParamsW32>,
+extern "C" const void* const jacc_tab_27_64_w32[JACC_NTILES] = {JACC_TILE_LIST(JENTRY_W32)};
+#endif

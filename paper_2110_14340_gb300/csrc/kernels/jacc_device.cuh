@@ -360,17 +360,6 @@ JD void fetch_halo(const T* __restrict__ u, const P& p, i64 z, i64 bx0, i64 by0,
   }
 }
 
-// Corner halo values (needed by the 27-point stencil only): the four points
-// diagonal to the tile.  Fetched by thread (0,0) and friends; returned raw.
-template <class T, class P>
-JD T fetch_corner(const T* __restrict__ u, const P& p, i64 z, i64 xx, i64 yy) {
-  const i64 nx = p.nx, ny = p.ny, nz = p.nz;
-  z = (z + nz) % nz;
-  xx = (xx + nx) % nx;
-  yy = (yy + ny) % ny;
-  return __ldg(u + (z * ny + yy) * nx + xx);
-}
-
 // Write this thread's converted plane values and its halo share into buffer b.
 template <class T, int BX, int BY, int V, int MODE>
 JD void put_plane(Plane<typename WT<T, MODE>::type, BX, BY, V>& sm, int b, const typename WT<T, MODE>::type (&own)[V],
@@ -503,59 +492,6 @@ template <class P> JD bool heat_fold(const P& p) {
 }
 
 
-// ---------------------------------------------------------------- 27-point periodic box
-//
-// Per plane and own point: c = centre, f = the 4 in-plane faces, g = the 4
-// in-plane diagonals.  With planes z-1 (m), z (0), z+1 (n):
-//   v = w0 c0 + wf (f0 + cm + cn) + we (g0 + fm + fn) + wc (gm + gn).
-// The shared-memory plane holds plane z+1 at iteration z.  Fixed path:
-// v 2^(F+K) = sum_j fw_j * class_j exactly in 128 bits (w_j = fw_j 2^-K).
-
-template <class T, int BX, int BY, int V, int MODE>
-JD void plane_cfe(const Plane<typename WT<T, MODE>::type, BX, BY, V>& sm, int b, typename WT<T, MODE>::type (&c)[V],
-                  typename WT<T, MODE>::type (&f)[V], typename WT<T, MODE>::type (&g)[V]) {
-  typedef typename WT<T, MODE>::type W;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const W* rm = &sm.a[b][ty][V + tx * V];
-  const W* r0 = &sm.a[b][ty + 1][V + tx * V];
-  const W* rp = &sm.a[b][ty + 2][V + tx * V];
-  W m[V + 2], z[V + 2], q[V + 2];
-#pragma unroll
-  for (int e = -1; e <= V; ++e) { m[e + 1] = rm[e]; z[e + 1] = r0[e]; q[e + 1] = rp[e]; }
-#pragma unroll
-  for (int e = 0; e < V; ++e) {
-    c[e] = z[e + 1];
-    f[e] = (z[e] + z[e + 2]) + (m[e + 1] + q[e + 1]);
-    g[e] = (m[e] + m[e + 2]) + (q[e] + q[e + 2]);
-  }
-}
-
-// The four halo corners of the tile (periodic wrap), fetched by thread (0,0).
-template <class T, int BX, int BY, int V, class P>
-JD void fetch_corners(const T* __restrict__ u, const P& p, i64 z, i64 bx0, i64 by0, T (&cr)[4]) {
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    const i64 nx = p.nx, ny = p.ny, nz = p.nz;
-    const i64 zz = (z % nz + nz) % nz;
-    const i64 xl = (bx0 - 1 + nx) % nx, xr = (bx0 + BX * V) % nx;
-    const i64 yt = (by0 - 1 + ny) % ny, yb = (by0 + BY) % ny;
-    const T* pl = u + zz * nx * ny;
-    cr[0] = __ldg(pl + yt * nx + xl);
-    cr[1] = __ldg(pl + yt * nx + xr);
-    cr[2] = __ldg(pl + yb * nx + xl);
-    cr[3] = __ldg(pl + yb * nx + xr);
-  }
-}
-
-template <class T, int BX, int BY, int V, int MODE>
-JD void put_corners(Plane<typename WT<T, MODE>::type, BX, BY, V>& sm, int b, const T (&cr)[4], int F) {
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    sm.a[b][0][V - 1] = cvt_in<T, MODE>(cr[0], F);
-    sm.a[b][0][V + BX * V] = cvt_in<T, MODE>(cr[1], F);
-    sm.a[b][BY + 1][V - 1] = cvt_in<T, MODE>(cr[2], F);
-    sm.a[b][BY + 1][V + BX * V] = cvt_in<T, MODE>(cr[3], F);
-  }
-}
-
 // Sum accumulator: FP64 for FP64 data; an FP32 error-free (hi, lo) pair for
 // FP32 data, combined in FP64 once per thread.
 template <class T> struct SumAcc {
@@ -568,80 +504,6 @@ template <> struct SumAcc<float> {
   JD void add(float x) { two_sum_acc(hi, lo, x); }
   JD double total() const { return (double)hi + (double)lo; }
 };
-
-template <class T, int BX, int BY, int V, int MODE, class P>
-JD void plane_load_put(const T* __restrict__ u, const P& p, i64 z, i64 bx0, i64 by0, bool act, const T* urow,
-                       Plane<typename WT<T, MODE>::type, BX, BY, V>& sm, int b, int F) {
-  typedef typename WT<T, MODE>::type W;
-  const i64 nz = p.nz, sz = p.nx * p.ny;
-  T r[V];
-#pragma unroll
-  for (int e = 0; e < V; ++e) r[e] = T(0);
-  if (act) ldv<T, V>(urow + ((z % nz + nz) % nz) * sz, r);
-  W own[V];
-#pragma unroll
-  for (int e = 0; e < V; ++e) own[e] = cvt_in<T, MODE>(r[e], F);
-  HaloFetch<T, BX, BY, V> h;
-  fetch_halo<T, BX, BY, V>(u, p, z, bx0, by0, true, h);
-  T cr[4];
-  fetch_corners<T, BX, BY, V>(u, p, z, bx0, by0, cr);
-  put_plane<T, BX, BY, V, MODE>(sm, b, own, h, F);
-  put_corners<T, BX, BY, V, MODE>(sm, b, cr, F);
-}
-
-template <class T, int BX, int BY, int V, int ZC, int MODE, class P>
-JD void box27_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int F, SumAcc<T>& acc,
-                   Plane<typename WT<T, MODE>::type, BX, BY, V>& sm) {
-  typedef typename WT<T, MODE>::type W;
-  const i64 nx = p.nx, ny = p.ny, nz = p.nz;
-  const i64 sz = nx * ny;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const i64 bx0 = (i64)blockIdx.x * (BX * V);
-  const i64 by0 = (i64)blockIdx.y * BY;
-  const i64 x0 = bx0 + (i64)tx * V;
-  const i64 y = by0 + ty;
-  const bool act = (x0 < nx) && (y < ny);
-  const i64 z0 = (i64)blockIdx.z * ZC;
-  const i64 z1 = (z0 + ZC < nz) ? z0 + ZC : nz;
-  const T* urow = u + (y % ny) * nx + (x0 % nx);  // periodic image for overhanging threads
-  T* vrow = v + y * nx + x0;
-
-  W cm[V], fm[V], gm[V], c0[V], f0[V], g0[V];
-  int b = 0;
-  plane_load_put<T, BX, BY, V, MODE>(u, p, z0 - 1, bx0, by0, true, urow, sm, b, F);
-  __syncthreads();
-  plane_cfe<T, BX, BY, V, MODE>(sm, b, cm, fm, gm);
-  b ^= 1;
-  plane_load_put<T, BX, BY, V, MODE>(u, p, z0, bx0, by0, true, urow, sm, b, F);
-  __syncthreads();
-  plane_cfe<T, BX, BY, V, MODE>(sm, b, c0, f0, g0);
-  b ^= 1;
-  for (i64 z = z0; z < z1; ++z) {
-    plane_load_put<T, BX, BY, V, MODE>(u, p, z + 1, bx0, by0, true, urow, sm, b, F);
-    __syncthreads();
-    W cn[V], fn[V], gn[V];
-    plane_cfe<T, BX, BY, V, MODE>(sm, b, cn, fn, gn);
-    T out[V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) {
-      const W F1 = (f0[e] + cm[e]) + cn[e];
-      const W E2 = (g0[e] + fm[e]) + fn[e];
-      const W C3 = gm[e] + gn[e];
-      out[e] = ((T)p.c0 * c0[e] + (T)p.c1 * F1) + ((T)p.c2 * E2 + (T)p.c3 * C3);
-    }
-    if (act) {
-      stv<T, V>(vrow + z * sz, out);
-#pragma unroll
-      for (int e = 0; e < V; ++e) acc.add(out[e]);
-    }
-#pragma unroll
-    for (int e = 0; e < V; ++e) {
-      cm[e] = c0[e]; fm[e] = f0[e]; gm[e] = g0[e];
-      c0[e] = cn[e]; f0[e] = fn[e]; g0[e] = gn[e];
-    }
-    b ^= 1;
-  }
-}
 
 // ---------------------------------------------------------------- 27-point periodic box, native arithmetic
 //
@@ -687,19 +549,19 @@ struct Box27Fetch {
   T own[V], hrow[V], hx, cr[4];
 };
 
-template <class T, int BX, int BY, int V, int ZC, class P>
-JD void box27_body2(const T* __restrict__ u, T* __restrict__ v, const P& p, SumAcc<T>& acc, bool want_sum,
-                    Plane<T, BX, BY, V>& sm) {
+template <class T, int BX, int BY, int V, class P>
+JD void box27_body2(const T* __restrict__ u, T* __restrict__ v, const P& p, int zc, SumAcc<T>& acc, bool want_sum,
+                    Plane<T, BX, BY, V>& sm, int ys_mul = 1, int ysub = 0) {
   const i64 nx = p.nx, ny = p.ny, nz = p.nz;
   const i64 sz = nx * ny;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const i64 bx0 = (i64)blockIdx.x * (BX * V);
-  const i64 by0 = (i64)blockIdx.y * BY;
+  const i64 by0 = ((i64)blockIdx.y * ys_mul + ysub) * BY;  // a CTA may cover ys_mul tiles of BY rows
   const i64 x0 = bx0 + (i64)tx * V;
   const i64 y = by0 + ty;
   const bool act = (x0 < nx) && (y < ny);
-  const i64 z0 = (i64)blockIdx.z * ZC;
-  const i64 z1 = (z0 + ZC < nz) ? z0 + ZC : nz;
+  const i64 z0 = (i64)blockIdx.z * zc;
+  const i64 z1 = (z0 + zc < nz) ? z0 + zc : nz;
   // periodic images, once per thread (threads overhanging the grid use them too)
   const i64 xo = x0 % nx, yo = y % ny;
   const i64 own_off = yo * nx + xo;
@@ -1213,10 +1075,6 @@ JD void box27_tb_entry(const float* __restrict__ u, float* __restrict__ v, const
 
 JD i64 bits_i64(double d) { return (i64)__double_as_longlong(d); }
 JD double i64_bits(i64 q) { return __longlong_as_double(q); }
-
-// Raw 8-byte word -> fixed-point value: convert (FP64 input) or reinterpret
-// (resident fixed point).
-JD i64 fx_in(double raw, bool conv, int F) { return conv ? fx_from(raw, F) : bits_i64(raw); }
 
 // Round q * 2^-k to the nearest integer (ties up), k in [0, 62].
 JD i64 fx_round_shift(i64 q, int k) { return k ? ((q + ((i64)1 << (k - 1))) >> k) : q; }
@@ -1944,109 +1802,249 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   }
 }
 
-// ---------------------------------------------------------------- 27-point box, resident fixed point
+// ---------------------------------------------------------------- planes staged by asynchronous copies
 //
-// v 2^F = round(sum_j fw_j class_j 2^-K) from the exact 128-bit sum; the FP64
-// output is the 128-bit sum correctly rounded.  Periodic: no boundary, every
-// point is updated.  The field sum accumulates the fixed outputs exactly in
-// 128 bits per thread.
-template <int BX, int BY, int V>
-JD void fx_plane_load_put(const double* __restrict__ u, i64 nx, i64 ny, i64 nz, i64 z, i64 bx0, i64 by0,
-                          const double* urow, Plane<i64, BX, BY, V>& sm, int b, int F, bool inf) {
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const i64 zz = (z % nz + nz) % nz;
-  const double* pl = u + zz * nx * ny;
-  double r[V];
-  ldv<double, V>(urow + zz * nx * ny, r);
-  i64 w[V];
-#pragma unroll
-  for (int e = 0; e < V; ++e) w[e] = inf ? fx_from(r[e], F) : bits_i64(r[e]);
-  i64* row = &sm.a[b][ty + 1][V + tx * V];
-#pragma unroll
-  for (int e = 0; e < V; ++e) row[e] = w[e];
-  const i64 x0 = (bx0 + (i64)tx * V) % nx;
-  if (ty == 0 || ty == BY - 1) {
-    const i64 yy = ty == 0 ? (by0 - 1 + ny) % ny : (by0 + BY) % ny;
-    double h[V];
-    ldv<double, V>(pl + yy * nx + x0, h);
-#pragma unroll
-    for (int e = 0; e < V; ++e) w[e] = inf ? fx_from(h[e], F) : bits_i64(h[e]);
-    i64* hr = &sm.a[b][ty == 0 ? 0 : BY + 1][V + tx * V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) hr[e] = w[e];
-  }
-  const i64 yy = (by0 + ty) % ny;
-  if (tx == 0) sm.a[b][ty + 1][V - 1] = fx_in(__ldg(pl + yy * nx + (bx0 - 1 + nx) % nx), inf, F);
-  if (tx == BX - 1) sm.a[b][ty + 1][V + BX * V] = fx_in(__ldg(pl + yy * nx + (bx0 + BX * V) % nx), inf, F);
-  if (tx == 0 && ty == 0) {
-    const i64 xl = (bx0 - 1 + nx) % nx, xr = (bx0 + BX * V) % nx;
-    const i64 yt = (by0 - 1 + ny) % ny, yb = (by0 + BY) % ny;
-    sm.a[b][0][V - 1] = fx_in(__ldg(pl + yt * nx + xl), inf, F);
-    sm.a[b][0][V + BX * V] = fx_in(__ldg(pl + yt * nx + xr), inf, F);
-    sm.a[b][BY + 1][V - 1] = fx_in(__ldg(pl + yb * nx + xl), inf, F);
-    sm.a[b][BY + 1][V + BX * V] = fx_in(__ldg(pl + yb * nx + xr), inf, F);
-  }
+// A second way of staging planes, for the kernels whose rows need not start
+// on 16-byte boundaries or whose staged values are converted in place: every
+// thread copies its share of a plane (the tile with a one-point halo) with
+// cp.async, CH elements per copy, into a ring of S stages in shared memory;
+// one group per plane, one CTA barrier per plane.  A copy's source may be any
+// element (8- or 4-byte copies for CH = 1), so odd rows, periodic images and
+// clipped edges all come from a per-thread list of source offsets worked out
+// once, and the thread that copied an element may convert it before the
+// barrier that publishes the plane.
+//
+// Geometry: BX x BY threads; a thread owns one column of RY consecutive rows,
+// so a warp reads and writes whole rows (no bank conflicts, coalesced stores
+// at any alignment), and the y neighbours inside its rows stay in registers.
+// A stage holds R x W elements in rows of W = BX + 2 CH: column x of the tile
+// sits at slot x - bx0 + CH of row y - by0 + 1.
+template <class T, int BX, int BY, int CH> struct RingG {
+  static constexpr int NT = BX * BY;
+  static constexpr int RY = JACC_RING_ROWS(BX, BY);
+  static constexpr int TW = BX, TH = BY * RY;
+  static constexpr int W = TW + 2 * CH, R = TH + 2;
+  static constexpr int STAGE = W * R;                       // elements
+  static constexpr int NCH = W / CH, NTOT = NCH * R;        // copies per row, per plane
+  static constexpr int PER = (NTOT + NT - 1) / NT;          // copies per thread
+  static constexpr int S0 = 46080 / (STAGE * (int)sizeof(T));
+  static constexpr int S = S0 < 3 ? 3 : (S0 > 6 ? 6 : S0);  // stages, at most 45 KB
+};
+
+template <int BYTES> JD void cpa_copy(void* dst, const void* src) {
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES) : "memory");
 }
+JD void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> JD void cpa_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <bool EDGE, int BX, int BY, int V, int ZC, class P>
-JD void box27_fx_body(const double* __restrict__ u, double* __restrict__ v, const P& p, int F, int flags, s128& acc,
-                      Plane<i64, BX, BY, V>& sm) {
-  const i64 nx = p.nx, ny = p.ny, nz = p.nz;
-  const i64 sz = nx * ny;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const i64 bx0 = (i64)blockIdx.x * (BX * V);
-  const i64 by0 = (i64)blockIdx.y * BY;
-  const i64 x0 = bx0 + (i64)tx * V;
-  const i64 y = by0 + ty;
-  const bool act = (x0 < nx) && (y < ny);
-  const i64 z0 = (i64)blockIdx.z * ZC;
-  const i64 z1 = (z0 + ZC < nz) ? z0 + ZC : nz;
-  const bool inf = EDGE && (flags & JFX_IN_F64);
-  const bool outf = EDGE && (flags & JFX_OUT_F64);
-  const double* urow = u + (y % ny) * nx + (x0 % nx);  // periodic image for overhanging threads
-  double* vrow = v + y * nx + x0;
-  const i64 w0 = p.fw0, w1 = p.fw1, w2 = p.fw2, w3 = p.fw3;
-  const int K = p.fk;
-
-  i64 cm[V], fm[V], gm[V], c0[V], f0[V], g0[V];
-  int b = 0;
-  fx_plane_load_put<BX, BY, V>(u, nx, ny, nz, z0 - 1, bx0, by0, urow, sm, b, F, inf);
-  __syncthreads();
-  plane_cfe<double, BX, BY, V, JM_FIXED>(sm, b, cm, fm, gm);
-  b ^= 1;
-  fx_plane_load_put<BX, BY, V>(u, nx, ny, nz, z0, bx0, by0, urow, sm, b, F, inf);
-  __syncthreads();
-  plane_cfe<double, BX, BY, V, JM_FIXED>(sm, b, c0, f0, g0);
-  b ^= 1;
-  for (i64 z = z0; z < z1; ++z) {
-    fx_plane_load_put<BX, BY, V>(u, nx, ny, nz, z + 1, bx0, by0, urow, sm, b, F, inf);
-    __syncthreads();
-    i64 cn[V], fn[V], gn[V];
-    plane_cfe<double, BX, BY, V, JM_FIXED>(sm, b, cn, fn, gn);
-    double out[V];
+// A thread's share of every staged plane: copy i moves the CH elements at
+// offset off[i] of the plane to stage element (tid + i NT) CH; bit i of
+// `mask` is clear where there is none (past the plane, or outside a Dirichlet
+// grid, whose slots are never used).
+template <class T, int BX, int BY, int CH> struct RingPlan {
+  typedef RingG<T, BX, BY, CH> G;
+  i64 off[G::PER];
+  u32 mask;
+  JD void init(i64 nx, i64 ny, i64 bx0, i64 by0, bool periodic) {
+    const int tid = threadIdx.y * BX + threadIdx.x;
+    mask = 0;
 #pragma unroll
-    for (int e = 0; e < V; ++e) {
-      s128 a = mul_s64_u64(c0[e], (u64)w0);
-      a = add128(a, mul_s64_u64((f0[e] + cm[e]) + cn[e], (u64)w1));
-      a = add128(a, mul_s64_u64((g0[e] + fm[e]) + fn[e], (u64)w2));
-      a = add128(a, mul_s64_u64(gm[e] + gn[e], (u64)w3));
-      const i64 q = fx128_round_shift(a, K);
-      out[e] = outf ? fx128_to(a, F + K) : i64_bits(q);
-      if (act) {
-        s128 t;
-        t.lo = (u64)q;
-        t.hi = (u64)(q >> 63);
-        acc = add128(acc, t);
+    for (int i = 0; i < G::PER; ++i) {
+      const int c = tid + i * G::NT;
+      i64 x = bx0 - CH + (c % G::NCH) * CH, y = by0 - 1 + c / G::NCH;
+      bool ok = c < G::NTOT;
+      if (periodic) {
+        x = (x + nx) % nx;
+        y = (y + ny) % ny;
+      } else {
+        ok = ok && x >= 0 && x < nx && y >= 0 && y < ny;
+      }
+      off[i] = ok ? y * nx + x : 0;
+      mask |= (u32)ok << i;
+    }
+  }
+  JD void issue(T* stage, const T* plane) const {
+    const int tid = threadIdx.y * BX + threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < G::PER; ++i)
+      if ((mask >> i) & 1u) cpa_copy<CH * (int)sizeof(T)>(stage + (tid + i * G::NT) * CH, plane + off[i]);
+  }
+};
+
+// Converts this thread's share of a landed FP64 plane to fixed point in place.
+template <int BX, int BY, int CH> JD void ring_to_fixed(const RingPlan<double, BX, BY, CH>& pl, double* stage, int F) {
+  typedef RingG<double, BX, BY, CH> G;
+  const int tid = threadIdx.y * BX + threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < G::PER; ++i)
+    if ((pl.mask >> i) & 1u) {
+#pragma unroll
+      for (int e = 0; e < CH; ++e) {
+        double* w = stage + (tid + i * G::NT) * CH + e;
+        *w = i64_bits(fx_from(*w, F));
       }
     }
-    if (act) stv<double, V>(vrow + z * sz, out);
-#pragma unroll
-    for (int e = 0; e < V; ++e) {
-      cm[e] = c0[e]; fm[e] = f0[e]; gm[e] = g0[e];
-      c0[e] = cn[e]; f0[e] = fn[e]; g0[e] = gn[e];
+}
+
+// ---------------------------------------------------------------- 27-point box, resident fixed point
+//
+// v 2^F = round(sum_j fw_j class_j 2^-K) from the exact sum; the FP64 output
+// is the exact sum correctly rounded.  Periodic: no boundary, every point is
+// updated.  The field sum accumulates the fixed outputs exactly in 128 bits
+// per thread.
+//
+// The weighted sum.  JACC_FP_W32 (every fw_j below 2^31 and K in [1, 31]: the
+// weights of an FP32 program): with class_j = h_j 2^32 + l_j the sum is
+// A 2^32 + B, A = sum fw_j h_j and B = sum fw_j l_j (below 2^64, as the fw_j
+// add up to at most 2^31 (1 + 2^-20)), eight 32 x 32 -> 64-bit multiply-adds.
+// Otherwise four 64 x 64 -> 128-bit products.
+//
+// Bound by the integer ALU work (64-bit class sums and the products), no
+// longer by latency: 320 x 256 x 192, 20 sweeps, 6.21 ms with planes loaded
+// and wrapped by every thread in the sweep itself (278 thread-instructions a
+// point, 811 GB/s) against 1.42 ms (3.5 TB/s), weights of 32 bits; folded
+// kernels, 512^3, 274 GLUP/s with 32-bit and 173 with 53-bit weights.  Four
+// rows per thread share their row sums and the classes of planes z-1 and z
+// stay in registers; two rows measured 2 % slower.
+template <class P> JD i64 box27_weigh(const P& p, i64 c, i64 f, i64 e, i64 g, s128* exact) {
+  const int K = p.fk;
+  if (p.fpath == JACC_FP_W32) {
+    const int w0 = (int)p.fw0, w1 = (int)p.fw1, w2 = (int)p.fw2, w3 = (int)p.fw3;
+    u64 B = (u64)1 << (K - 1);  // the rounding half
+    B += (u64)(u32)w0 * (u32)c;
+    B += (u64)(u32)w1 * (u32)f;
+    B += (u64)(u32)w2 * (u32)e;
+    B += (u64)(u32)w3 * (u32)g;
+    i64 A = (i64)w0 * (int)(c >> 32);
+    A += (i64)w1 * (int)(f >> 32);
+    A += (i64)w2 * (int)(e >> 32);
+    A += (i64)w3 * (int)(g >> 32);
+    if (exact) {
+      B -= (u64)1 << (K - 1);
+      s128 b;
+      b.lo = B;
+      b.hi = 0;
+      *exact = add128(from_s64_shl(A, 32), b);
+      return fx128_round_shift(*exact, K);
     }
-    b ^= 1;
+    const u64 H = (u64)(A + (i64)(B >> 32));
+    return (i64)((H << (32 - K)) | ((u32)B >> K));
   }
+  s128 a = mul_s64_u64(c, (u64)p.fw0);
+  a = add128(a, mul_s64_u64(f, (u64)p.fw1));
+  a = add128(a, mul_s64_u64(e, (u64)p.fw2));
+  a = add128(a, mul_s64_u64(g, (u64)p.fw3));
+  if (exact) *exact = a;
+  return fx128_round_shift(a, K);
+}
+
+template <int BX, int BY, int CH, bool EDGE, class P>
+JD void box27_fx_body(const double* __restrict__ u, double* __restrict__ v, const P& p, const JParams& rt, int F,
+                      int flags, s128& acc, double* sm) {
+  typedef RingG<double, BX, BY, CH> G;
+  constexpr int RY = G::RY, S = G::S;
+  const i64 nx = p.nx, ny = p.ny, nz = p.nz, sz = nx * ny;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const i64 bx0 = (i64)blockIdx.x * G::TW, by0 = (i64)blockIdx.y * G::TH;
+  const i64 x0 = bx0 + tx, y0 = by0 + ty * RY;
+  const i64 z0 = (i64)blockIdx.z * rt.zc;
+  const i64 z1 = (z0 + rt.zc < nz) ? z0 + rt.zc : nz;
+  const int L = (int)(z1 - z0) + 2;  // staged planes z0-1 .. z1 (periodic images)
+  const int nrow = x0 < nx ? (int)(ny - y0 < RY ? (ny - y0 > 0 ? ny - y0 : 0) : RY) : 0;  // rows this thread writes
+  const bool inf = EDGE && (flags & JFX_IN_F64);
+  const bool outf = EDGE && (flags & JFX_OUT_F64);
+  RingPlan<double, BX, BY, CH> plan;
+  plan.init(nx, ny, bx0, by0, true);
+  i64 zi = z0 == 0 ? nz - 1 : z0 - 1;  // next plane to stage
+  int is = 0;                          // and its stage, in elements
+  int issued = 0;
+  auto issue_next = [&]() {
+    if (issued < L) plan.issue(sm + is, u + zi * sz);
+    cpa_commit();
+    ++issued;
+    zi = zi + 1 == nz ? 0 : zi + 1;
+    is = is + G::STAGE == S * G::STAGE ? 0 : is + G::STAGE;
+  };
+#pragma unroll 1
+  for (int j = 0; j < S - 1; ++j) issue_next();
+  int cs = 0;  // the stage to read, in elements
+  // own-column sums of the next staged plane: c the points, f their four
+  // in-plane faces, g the four in-plane diagonals
+  auto consume = [&](i64 (&c)[RY], i64 (&f)[RY], i64 (&g)[RY]) {
+    cpa_wait<S - 2>();
+    if constexpr (EDGE) {
+      if (inf) ring_to_fixed<BX, BY, CH>(plan, sm + cs, F);
+    }
+    __syncthreads();
+    issue_next();  // into the stage read before the barrier
+    const i64* r = reinterpret_cast<const i64*>(sm) + cs + ty * RY * G::W + CH + tx;
+    i64 m[RY + 2], s[RY + 2];
+#pragma unroll
+    for (int k = 0; k < RY + 2; ++k) {
+      m[k] = r[k * G::W];
+      s[k] = r[k * G::W - 1] + r[k * G::W + 1];
+    }
+#pragma unroll
+    for (int k = 0; k < RY; ++k) {
+      c[k] = m[k + 1];
+      f[k] = s[k + 1] + (m[k] + m[k + 2]);
+      g[k] = s[k] + s[k + 2];
+    }
+    cs = cs + G::STAGE == S * G::STAGE ? 0 : cs + G::STAGE;
+  };
+  // running classes of the output plane: pf = f(z) + c(z-1), pe = g(z) + f(z-1), pc = g(z-1)
+  i64 pf[RY], pe[RY], pc[RY];
+  double* vo = v + z0 * sz + y0 * nx + x0;
+  auto step = [&](const i64 (&c0)[RY], const i64 (&f0)[RY], const i64 (&g0)[RY], i64 (&cn)[RY], i64 (&fn)[RY],
+                  i64 (&gn)[RY]) {
+    consume(cn, fn, gn);
+    i64 rowsum = 0;  // at most four values below 2^58: exact
+#pragma unroll
+    for (int k = 0; k < RY; ++k) {
+      double o;
+      i64 q;
+      if (EDGE && outf) {
+        s128 ex;
+        q = box27_weigh(p, c0[k], pf[k] + cn[k], pe[k] + fn[k], pc[k] + gn[k], &ex);
+        o = fx128_to(ex, F + p.fk);
+      } else {
+        q = box27_weigh(p, c0[k], pf[k] + cn[k], pe[k] + fn[k], pc[k] + gn[k], nullptr);
+        o = i64_bits(q);
+      }
+      pf[k] = fn[k] + c0[k];
+      pe[k] = gn[k] + f0[k];
+      pc[k] = g0[k];
+      if (k < nrow) {
+        vo[k * nx] = o;
+        rowsum += q;
+      }
+    }
+    vo += sz;
+    s128 t;
+    t.lo = (u64)rowsum;
+    t.hi = (u64)(rowsum >> 63);
+    acc = add128(acc, t);
+  };
+  i64 ca[RY], fa[RY], ga[RY], cb[RY], fb[RY], gb[RY];
+  consume(ca, fa, ga);
+  consume(cb, fb, gb);
+#pragma unroll
+  for (int k = 0; k < RY; ++k) {
+    pf[k] = fb[k] + ca[k];
+    pe[k] = gb[k] + fa[k];
+    pc[k] = ga[k];
+  }
+  int j = 2;
+#pragma unroll 1
+  for (; j + 1 < L; j += 2) {
+    step(cb, fb, gb, ca, fa, ga);
+    step(ca, fa, ga, cb, fb, gb);
+  }
+  if (j < L) step(cb, fb, gb, ca, fa, ga);
+  cpa_wait<0>();
 }
 
 // ====================================================================== kernels
@@ -2142,9 +2140,11 @@ JD void heat3d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, con
     } else {
       double m = 0.0;
 #pragma unroll 1
-      for (int sub = 0; sub < (STAGED ? 2 : 1); ++sub)
+      for (int sub = 0; sub < (STAGED ? 2 : 1); ++sub) {
+        if (sub) __syncthreads();  // the sub-tiles share the planes
         heat3d_body<T, BX, BY, V, ZC, JM_NATIVE>(u, v, p, -1, m, *reinterpret_cast<Plane<double, BX, BY, V>*>(raw),
                                                  STAGED ? 2 : 1, sub);
+      }
       bits = dbits(m);
     }
   } else if constexpr (V == 4) {
@@ -2167,16 +2167,23 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   griddep_wait();
   double total = 0.0;
   if constexpr (sizeof(T) == 8) {
+    typedef RingG<double, BX, BY, V> G;
+    constexpr size_t SM_RING = (size_t)G::S * G::STAGE * 8, SM_PLANE = sizeof(Plane<double, BX, BY, 1>);
+    __shared__ __align__(16) unsigned char raw[SM_RING > SM_PLANE ? SM_RING : SM_PLANE];
     const int F = (maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
-    __shared__ __align__(16) unsigned char raw[sizeof(Plane<i64, BX, BY, V>)];
     if (F >= 0) {
       s128 acc;
       acc.lo = acc.hi = 0ull;
-      box27_fx_body<EDGE, BX, BY, V, ZC>(u, v, p, F, flags, acc, *reinterpret_cast<Plane<i64, BX, BY, V>*>(raw));
+      box27_fx_body<BX, BY, V, EDGE>(u, v, p, rt, F, flags, acc, reinterpret_cast<double*>(raw));
       total = fx128_to(acc, F);
     } else {
       SumAcc<T> acc;
-      box27_body2<T, BX, BY, V, ZC>(u, v, p, acc, resid != nullptr, *reinterpret_cast<Plane<double, BX, BY, V>*>(raw));
+#pragma unroll 1
+      for (int sub = 0; sub < G::RY; ++sub) {
+        __syncthreads();  // the sub-tiles share the planes
+        box27_body2<T, BX, BY, 1>(u, v, p, rt.zc, acc, resid != nullptr, *reinterpret_cast<Plane<double, BX, BY, 1>*>(raw),
+                                  G::RY, sub);
+      }
       total = acc.total();
     }
   } else if constexpr (V == 4) {
@@ -2184,7 +2191,7 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   } else {
     __shared__ Plane<T, BX, BY, V> sm;
     SumAcc<T> acc;
-    box27_body2<T, BX, BY, V, ZC>(u, v, p, acc, resid != nullptr, sm);
+    box27_body2<T, BX, BY, V>(u, v, p, ZC, acc, resid != nullptr, sm);
     total = acc.total();
   }
   block_sum_to<BX * BY>(total, resid);
@@ -2277,12 +2284,16 @@ __global__ void jacc_k_fill_skipped(double* resid, int n, int T) {
 // and, unbounded, take 124 registers (4 CTAs), so they ask for 6 (80
 // registers, 6 stages); the converting sweeps at 5 CTAs (at most 102
 // registers, from 157) take 2.40 ms for a 2-sweep sequence against 2.83.
+// For the FP64 27-point kernel with 32 x 4 threads: 4 CTAs (at most 128
+// registers); folded, 512^3: 490 us a sweep against 492 unbounded (3 CTAs)
+// and 518 at 5 (spills).
 // Every other kernel: 0, no requirement (a bound of 1 is not neutral: it
 // lets the compiler take registers for one CTA per SM, e.g. 111 instead of
 // 80 for the staged FP32 7-point kernel).
 template <int STENCIL, class T, int BX, int BY, int V, bool EDGE, bool FOLDED> struct SweepMinBlocks {
   static constexpr bool heat_staged_fp64 = STENCIL == 7 && sizeof(T) == 8 && BX == 32 && BY == 4 && V == 2;
-  static constexpr int value = heat_staged_fp64 ? (EDGE ? 5 : (FOLDED ? 7 : 6)) : 0;
+  static constexpr bool box27_fp64 = STENCIL == 27 && sizeof(T) == 8 && BX == 32 && BY == 4;
+  static constexpr int value = heat_staged_fp64 ? (EDGE ? 5 : (FOLDED ? 7 : 6)) : (box27_fp64 && !EDGE ? 4 : 0);
 };
 
 // The constant-folded last sweep of a sequence that does not convert on load
@@ -2310,8 +2321,12 @@ __global__ void __launch_bounds__(TB_BX * RY) jacc_k_box27_tb(const float* __res
                                                               JParams p, double* resid, const u64* maxword, int flags) {
   box27_tb_entry<RY, TT, ZC>(u, v, p, resid);
 }
-template <class T, int BX, int BY, int V, int ZC, bool EDGE>
-__global__ void __launch_bounds__(BX * BY) jacc_k_box27(const T* __restrict__ u, T* __restrict__ v, JParams p,
-                                                        double* resid, const u64* maxword, int flags) {
+// P = JParamsW32: the same parameter block, known to hold 32-bit factors.
+struct JParamsW32 : JParams {
+  static constexpr int fpath = JACC_FP_W32;
+};
+template <class T, int BX, int BY, int V, int ZC, bool EDGE, class P>
+__global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<27, T, BX, BY, V, EDGE, false>::value))
+    jacc_k_box27(const T* __restrict__ u, T* __restrict__ v, P p, double* resid, const u64* maxword, int flags) {
   box27_entry<T, BX, BY, V, ZC, EDGE>(u, v, p, p, resid, maxword, flags);
 }

@@ -11,6 +11,12 @@ typedef unsigned int u32;
 #define JACC_FP_SMALL 1  // 7pt, r = fb 2^-k with k <= 5: v 2^(F+k) = fa u + fb S in int64
 #define JACC_FP_WIDE 2   // 7pt / 27pt: exact 128-bit products
 #define JACC_FP_JACOBI 3 // 5pt: v 2^(F+2) = S
+#define JACC_FP_W32 4    // 27pt: every factor below 2^31 and K in [1, 31]: 32-bit factors
+
+// Rows per thread of the kernels that stage planes by asynchronous copies
+// (bx x by threads, one column each): 4, or 2 where 4 would not leave room
+// for the stages.
+#define JACC_RING_ROWS(bx, by) ((bx) * (by) > 256 ? 2 : 4)
 
 struct JParams {
   i64 nx, ny, nz;
@@ -26,7 +32,7 @@ struct JParams {
   int* status;
   i64 timeout_ns;
   int stall_plane;
-  int reserved;
+  int zc;  // planes per CTA
   // The twelve coefficient fields of the variable-coefficient 19-point
   // stencil (a0 a1 a2 a3 b0 b1 b2 c0 c1 c2 wrk1 bnd; FP32, device), set per
   // call; unused by the other stencils.
