@@ -86,17 +86,17 @@ static int plan_fixed(const jacc_kernel_desc& d, JParams& p) {
     const double r = d.coeffs[0];
     if (r == 0.0) {
       p.fpath = JACC_FP_SMALL;
-      p.fa = 1;
+      p.fm = 0;
       p.fb = 0;
       p.fk = 0;
     } else if (r > 0.0 && r <= 1.0 / 6.0) {
       uint64_t m;
       int k;
       if (dyadic(r, &m, &k)) {
+        p.fm = m << (62 - k);
         if (k <= 5) {
           p.fpath = JACC_FP_SMALL;
           p.fb = static_cast<i64>(m);
-          p.fa = (static_cast<i64>(1) << k) - 6 * static_cast<i64>(m);
           p.fk = k;
         } else {
           p.fpath = JACC_FP_WIDE;
@@ -211,8 +211,7 @@ bool staged_tile(const jacc_kernel_desc& d, int t) {
 // Tiles whose planes are staged by asynchronous copies, one column of
 // JACC_RING_ROWS rows per thread.
 static bool ring_tile(const jacc_kernel_desc& d, int t) {
-  (void)t;
-  return d.stencil == 27 && d.dtype == 64;
+  return !kTiles[t].vec16 ? d.stencil == 7 || d.stencil == 27 : d.stencil == 27 && d.dtype == 64;
 }
 
 bool tile_valid(const jacc_kernel_desc& d, int t) {
@@ -226,12 +225,34 @@ bool tile_valid(const jacc_kernel_desc& d, int t) {
   return gx < (1ll << 31) && gy <= 65535 && gz <= 65535;
 }
 
-static std::string key_of(const jacc_kernel_desc& d, int tile) {
+static std::string key_of(const jacc_kernel_desc& d, int tile, bool fit) {
   jacc_kernel_desc c = d;
   c.tile_id = tile;
   c.reserved = 0;
   if (c.tblock == 0) c.tblock = 1;
-  return std::string(reinterpret_cast<const char*>(&c), sizeof(c));
+  return std::string(reinterpret_cast<const char*>(&c), sizeof(c)) + (fit ? "f" : "t");
+}
+
+// Planes per CTA of a 3D kernel whose tile the library chose itself: at most
+// the tile's own, and few enough that the grid has at least 2.5 times the
+// CTAs that the device holds at once (no fewer than 8 planes: the two halo
+// planes of a chunk are read again).  With fewer, the last wave leaves SMs
+// idle: 301 x 253 x 199 FP64 at 64 planes (640 CTAs on 152 SMs) 65.2 us a
+// sweep, at 16 planes (2080) 55.7, at 8 (4000) 57.3; 511^3, whose grid is
+// large either way, within 3 % from 8 to 64.
+static int fitted_chunk(const Kernel& k, int zc) {
+  int dev = 0, nsm = 0, per = 6;  // a folded kernel is compiled for its chunk: 5 to 8 of them fit an SM
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      (k.func && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k.func, static_cast<int>(k.block.x * k.block.y), 0) !=
+                     cudaSuccess)) {
+    cudaGetLastError();
+    return zc;
+  }
+  const int64_t columns = static_cast<int64_t>(k.grid.x) * k.grid.y;
+  const int64_t want = (5ll * nsm * (per > 0 ? per : 1) / 2 + columns - 1) / columns;  // chunks
+  const int64_t fit = (k.desc.nz + want - 1) / want;
+  return static_cast<int>(fit >= zc ? zc : (fit < 8 ? (zc < 8 ? zc : 8) : fit));
 }
 
 // Planes per CTA of a 3D kernel.  The constant-folded variants of the staged
@@ -256,42 +277,44 @@ static std::string jit_source(const Kernel& k) {
   char buf[4096];
   const char* T = k.desc.dtype == 64 ? "double" : "float";
   const char* entry = k.desc.stencil == 5 ? "jacobi2d_entry" : (k.desc.stencil == 7 ? "heat3d_entry" : "box27_entry");
-  const int zc = k.desc.stencil == 5 ? c.zc / 4 : plane_chunk(k.desc, k.tile);
+  // the 2D march length is a template argument, the 3D one a launch parameter
+  const std::string zc = k.desc.stencil == 5 ? std::to_string(c.zc / 4) + ", " : "";
   const char* edge = k.desc.dtype == 64 ? "true" : "false";  // the converting sweeps' instantiation
   std::snprintf(buf, sizeof(buf),
                 "\nstruct JFold {\n"
                 "  static constexpr i64 nx = %lldll, ny = %lldll, nz = %lldll;\n"
                 "  static constexpr double c0 = %a, c1 = %a, c2 = %a, c3 = %a;\n"
-                "  static constexpr i64 fa = %lldll, fb = %lldll;\n"
+                "  static constexpr u64 fm = %lluull;\n"
+                "  static constexpr i64 fb = %lldll;\n"
                 "  static constexpr i64 fw0 = %lldll, fw1 = %lldll, fw2 = %lldll, fw3 = %lldll;\n"
-                "  static constexpr int fk = %d, fpath = %d;\n"
+                "  static constexpr int fk = %d, fpath = %d, zc = %d;\n"
                 "};\n"
                 "template <> struct JacobiPrefetch<JFold> { static constexpr bool value = %s; };\n"
                 "extern \"C\" __global__ void __launch_bounds__(%d, (SweepMinBlocks<%d, %s, %d, %d, %d, false, true>::value))\n"
                 "jacc_jit(const %s* __restrict__ u, "
                 "%s* __restrict__ v, JParams rt, double* resid, const u64* maxword, int flags) {\n"
                 "  const JFold f{};\n"
-                "  %s<%s, %d, %d, %d, %d, false>(u, v, f, rt, resid, maxword, flags);\n"
+                "  %s<%s, %d, %d, %d, %sfalse>(u, v, f, rt, resid, maxword, flags);\n"
                 "}\n"
                 "extern \"C\" __global__ void __launch_bounds__(%d, (SweepMinBlocks<%d, %s, %d, %d, %d, %s, true>::value))\n"
                 "jacc_jit_out(const %s* __restrict__ u, "
                 "%s* __restrict__ v, JParams rt, double* resid, const u64* maxword, int flags) {\n"
                 "  const JFold f{};\n"
-                "  %s<%s, %d, %d, %d, %d, %s>(u, v, f, rt, resid, maxword, flags);\n"
+                "  %s<%s, %d, %d, %d, %s%s>(u, v, f, rt, resid, maxword, flags);\n"
                 "}\n"
                 "extern \"C\" __global__ void __launch_bounds__(%d, (SweepMinBlocksLast<%d, %s, %d, %d, %d>::value))\n"
                 "jacc_jit_last(const %s* __restrict__ u, "
                 "%s* __restrict__ v, JParams rt, double* resid, const u64* maxword, int flags) {\n"
                 "  const JFold f{};\n"
-                "  %s<%s, %d, %d, %d, %d, %s>(u, v, f, rt, resid, maxword, JFX_OUT_F64);\n"
+                "  %s<%s, %d, %d, %d, %s%s>(u, v, f, rt, resid, maxword, JFX_OUT_F64);\n"
                 "}\n",
-                (long long)p.nx, (long long)p.ny, (long long)p.nz, p.c0, p.c1, p.c2, p.c3, (long long)p.fa,
-                (long long)p.fb, (long long)p.fw0, (long long)p.fw1, (long long)p.fw2, (long long)p.fw3, p.fk, p.fpath,
+                (long long)p.nx, (long long)p.ny, (long long)p.nz, p.c0, p.c1, p.c2, p.c3, (unsigned long long)p.fm,
+                (long long)p.fb, (long long)p.fw0, (long long)p.fw1, (long long)p.fw2, (long long)p.fw3, p.fk, p.fpath, p.zc,
                 // small (L2-resident) 2D grids: the prefetching march
                 (k.desc.stencil == 5 && k.desc.nx * k.desc.ny <= (int64_t(1) << 17)) ? "true" : "false",
-                c.bx * c.by, k.desc.stencil, T, c.bx, c.by, k.vec, T, T, entry, T, c.bx, c.by, k.vec, zc, c.bx * c.by,
-                k.desc.stencil, T, c.bx, c.by, k.vec, edge, T, T, entry, T, c.bx, c.by, k.vec, zc, edge, c.bx * c.by,
-                k.desc.stencil, T, c.bx, c.by, k.vec, T, T, entry, T, c.bx, c.by, k.vec, zc, edge);
+                c.bx * c.by, k.desc.stencil, T, c.bx, c.by, k.vec, T, T, entry, T, c.bx, c.by, k.vec, zc.c_str(), c.bx * c.by,
+                k.desc.stencil, T, c.bx, c.by, k.vec, edge, T, T, entry, T, c.bx, c.by, k.vec, zc.c_str(), edge, c.bx * c.by,
+                k.desc.stencil, T, c.bx, c.by, k.vec, T, T, entry, T, c.bx, c.by, k.vec, zc.c_str(), edge);
   return std::string(device_source()) + buf;
 }
 
@@ -332,15 +355,19 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   jacc_status st = validate(*desc);
   if (st) return st;
   int tile = desc->tile_id;
+  bool fit = false;  // the library picks the planes per CTA along with the tile
   if (desc->stencil == 19) {
     tile = 3;  // the kernel's one configuration: 32 x 4 threads, 16-byte columns, 40-plane march
   } else if (tile < 0) {
     tile = tuned_tile(*desc);
-    if (tile < 0 || !tile_valid(*desc, tile)) tile = default_tile(*desc);
+    if (tile < 0 || !tile_valid(*desc, tile)) {
+      tile = default_tile(*desc);
+      fit = (desc->stencil == 7 || desc->stencil == 27) && desc->tblock <= 1;
+    }
   }
   if (!tile_valid(*desc, tile))
     return fail(JACC_ERR_INVALID_ARG, "tile " + std::to_string(tile) + " does not fit this shape (x vector width)");
-  const std::string key = key_of(*desc, tile);
+  const std::string key = key_of(*desc, tile, fit);
   std::lock_guard<std::mutex> lock(global_mutex());
   auto it = cache().find(key);
   if (it != cache().end()) {
@@ -379,6 +406,11 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
     const int64_t zc = p.zc;
     k->grid = dim3(static_cast<unsigned>((desc->nx + tx - 1) / tx), static_cast<unsigned>((desc->ny + ty - 1) / ty),
                    static_cast<unsigned>((desc->nz + zc - 1) / zc));
+  }
+  if (fit) {
+    if (!(desc->flags & JACC_SPEC_JIT)) k->func = table_entry(desc->stencil, desc->dtype, tile, false);
+    p.zc = fitted_chunk(*k, p.zc);
+    k->grid.z = static_cast<unsigned>((desc->nz + p.zc - 1) / p.zc);
   }
   if (desc->stencil == 19) {
     var19_geometry(desc->nx, desc->ny, desc->nz, &k->grid, &k->block);

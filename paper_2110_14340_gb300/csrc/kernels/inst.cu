@@ -12,15 +12,14 @@ typedef float JT;
 #define JVEC 4
 #endif
 
+// The planes per CTA of the 3D kernels are a launch parameter: both marches of
+// a tile shape run one kernel.
 #if JACC_INST_STENCIL == 5
 #define JKERN(BX, BY, V, ZC, O) jacc_k_jacobi2d<JT, BX, BY, V, (ZC) / 4, O>
 #elif JACC_INST_STENCIL == 7
-#define JKERN(BX, BY, V, ZC, O) jacc_k_heat3d<JT, BX, BY, V, ZC, O>
-#elif JACC_INST_DTYPE == 64
-// the planes per CTA are a launch parameter: one kernel for both marches
-#define JKERN(BX, BY, V, ZC, O) jacc_k_box27<JT, BX, BY, V, 0, O, JParams>
+#define JKERN(BX, BY, V, ZC, O) jacc_k_heat3d<JT, BX, BY, V, O>
 #else
-#define JKERN(BX, BY, V, ZC, O) jacc_k_box27<JT, BX, BY, V, ZC, O, JParams>
+#define JKERN(BX, BY, V, ZC, O) jacc_k_box27<JT, BX, BY, V, O, JParams>
 #endif
 
 #define JCAT3(a, b, c) a##b##_##c
@@ -40,6 +39,6 @@ extern "C" const void* const JTABOUT(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NT
 #if JACC_INST_STENCIL == 27 && JACC_INST_DTYPE == 64
 // Table 1 for weights with 32-bit fixed-point factors (JACC_FP_W32).
 #define JENTRY_W32(id, BX, BY, VEC, ZC) \
-  (const void*)jacc_k_box27<JT, BX, BY, ((VEC) ? JVEC : 1), 0, false, JParamsW32>,
+  (const void*)jacc_k_box27<JT, BX, BY, ((VEC) ? JVEC : 1), false, JParamsW32>,
 extern "C" const void* const jacc_tab_27_64_w32[JACC_NTILES] = {JACC_TILE_LIST(JENTRY_W32)};
 #endif

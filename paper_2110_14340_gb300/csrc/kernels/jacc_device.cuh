@@ -386,13 +386,10 @@ JD void put_plane(Plane<typename WT<T, MODE>::type, BX, BY, V>& sm, int b, const
 
 // ---------------------------------------------------------------- 7-point heat
 //
-// Fixed path: with S the sum of the six faces and L = S - 6u (exact, scale F),
-//   JACC_FP_SMALL (r = fb 2^-k, k <= 5): v 2^(F+k) = fa u + fb S,  fa = 2^k - 6 fb
-//   JACC_FP_WIDE  (r = m 2^-k, m odd):   v 2^(F+k) = u 2^k + m L   (128-bit)
-// and |v - u| = r |L|, so the residual only needs max |L|.
+// Native FP64 arithmetic, and the planes of the kernels that stage nothing.
 
-template <class T, int BX, int BY, int V, int ZC, int MODE, class P>
-JD void heat3d_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int F, typename RT<T, MODE>::type& rmax,
+template <class T, int BX, int BY, int V, int MODE, class P>
+JD void heat3d_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int zc, int F, typename RT<T, MODE>::type& rmax,
                     Plane<typename WT<T, MODE>::type, BX, BY, V>& sm, int ys_mul = 1, int ysub = 0) {
   typedef typename WT<T, MODE>::type W;
   const i64 nx = p.nx, ny = p.ny, nz = p.nz;
@@ -403,8 +400,8 @@ JD void heat3d_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int 
   const i64 x0 = bx0 + (i64)tx * V;
   const i64 y = by0 + ty;
   const bool act = (x0 < nx) && (y < ny);
-  const i64 cz0 = (i64)blockIdx.z * ZC;
-  const i64 cz1 = (cz0 + ZC < nz) ? cz0 + ZC : nz;
+  const i64 cz0 = (i64)blockIdx.z * zc;
+  const i64 cz1 = (cz0 + zc < nz) ? cz0 + zc : nz;
   const T* urow = u + y * nx + x0;
   T* vrow = v + y * nx + x0;
 
@@ -480,7 +477,6 @@ JD void heat3d_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int 
   }
 }
 
-// Residual of the heat sweep from max |L|: r max|L| scaled.
 // r = fb 2^-k with 1 <= k <= 4 and fb <= 2 (r = 1/8, 1/16, ...): the
 // constant-folded staged heat kernels form v 2^F directly as
 // (fb S + (2^k - 6 fb) c + 2^(k-1)) >> k, which equals c + round(r L 2^F) bit
@@ -813,7 +809,7 @@ JD void box27s_terms(const float (*st)[Box27S<BX, BY>::W], float w0, float wf, f
 // z1 are staged (L = z1 - z0 + 2), output plane z = A(z-1) + B(z) + A(z+1)
 // is formed as P + A(z+1) with P = A(z-1) + B(z) kept in registers.  Returns
 // the thread's double-float sum of its outputs (want_sum).
-template <int BX, int BY, int ZC, class P>
+template <int BX, int BY, class P>
 JD double box27s_body(const float* __restrict__ u, float* __restrict__ v, const P& p, const JParams& rt,
                       bool want_sum) {
   typedef Box27S<BX, BY> G;
@@ -823,8 +819,8 @@ JD double box27s_body(const float* __restrict__ u, float* __restrict__ v, const 
   const int tid = ty * BX + tx;
   const bool warp0 = tid < 32;
   const i64 bx0 = (i64)blockIdx.x * G::TW, by0 = (i64)blockIdx.y * G::TH;
-  const i64 z0 = (i64)blockIdx.z * ZC;
-  const i64 z1 = (z0 + ZC < nz) ? z0 + ZC : nz;
+  const i64 z0 = (i64)blockIdx.z * p.zc;
+  const i64 z1 = (z0 + p.zc < nz) ? z0 + p.zc : nz;
   const int L = (int)(z1 - z0) + 2;
   const int weff = (int)((nx - bx0 < G::TW) ? nx - bx0 : G::TW) + 8;
   const i64 lim = rt.timeout_ns;
@@ -1306,159 +1302,49 @@ JD void jacobi_march_pf(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 
 
 // ---------------------------------------------------------------- 7-point heat, resident fixed point
 //
-// S = the six faces, L = S - 6u (exact, scale F):
-//   JACC_FP_SMALL (r = fb 2^-k): v = u + round(fb L 2^-k)      (int64)
-//   JACC_FP_WIDE  (r = m 2^-k):  v = u + round(m L 2^-k)       (128-bit product)
-// FP64 output: u + r L correctly rounded.  The residual only needs max |L|.
+// S = the six faces, L = S - 6u (exact, scale F), r = m 2^-k:
+// v = u + round(m L 2^-k), the FP64 output u + r L correctly rounded, and
+// |v - u| is the magnitude of the increment.  An intermediate sweep converts
+// nothing: every value in both buffers, the Dirichlet boundary included, is
+// in fixed point.  The first and last sweeps of a sequence (EDGE, flags
+// JFX_IN_F64 / JFX_OUT_F64) convert loads and stores.
 //
-// EDGE = false: an intermediate sweep.  Every value in both buffers, the
-// Dirichlet boundary included, is already in fixed point, so the kernel does
-// no conversion at all.  EDGE = true: the first and/or last sweep of a
-// sequence (flags JFX_IN_F64 / JFX_OUT_F64): loads convert from FP64, stores
-// convert to FP64, boundary points are converted (or copied when both).
-template <bool EDGE, int BX, int BY, int V, int ZC, class P>
-JD void heat3d_fx_body(const double* __restrict__ u, double* __restrict__ v, const P& p, int F, int flags, u64& rmax,
-                       Plane<i64, BX, BY, V>& sm) {
-  const i64 nx = p.nx, ny = p.ny, nz = p.nz;
-  const i64 sz = nx * ny;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const i64 bx0 = (i64)blockIdx.x * (BX * V);
-  const i64 by0 = (i64)blockIdx.y * BY;
-  const i64 x0 = bx0 + (i64)tx * V;
-  const i64 y = by0 + ty;
-  const bool act = (x0 < nx) && (y < ny);
-  const i64 cz0 = (i64)blockIdx.z * ZC;
-  const i64 cz1 = (cz0 + ZC < nz) ? cz0 + ZC : nz;
-  const bool inf = EDGE && (flags & JFX_IN_F64);
-  const bool outf = EDGE && (flags & JFX_OUT_F64);
-  const double* urow = u + y * nx + x0;
-  double* vrow = v + y * nx + x0;
-  // boundary point written by this sweep, from its input word
-  auto bnd_out = [&](double raw, i64 w) -> double {
-    if constexpr (!EDGE) return i64_bits(w);    // fixed in, fixed out (raw holds the same bits)
-    if (inf && outf) return raw;                // FP64 in, FP64 out: copy
-    if (outf) return fx_to(w, F);               // fixed in, FP64 out
-    return i64_bits(w);                         // FP64 in, fixed out
-  };
-  auto cvt = [&](double raw) -> i64 { return (EDGE && inf) ? fx_from(raw, F) : bits_i64(raw); };
-
-  // Boundary planes are written by the chunk that holds them.
-  if (act && (cz0 == 0 || cz1 == nz)) {
+// The increment for any r: with fm = m 2^(62-k) < 2^60 (r <= 1/6) it is
+// floor((L fm + 2^61) / 2^62).  L + 2^62 is positive (|L| < 2^61), so the
+// 96-bit product of it takes four unsigned 32 x 32 -> 64-bit multiply-adds,
+// and the fm that the bias adds to the quotient is exact and comes off at the
+// end: 12 instructions for every r, in place of a 64 x 64 -> 128-bit product
+// and a 128-bit rounding shift.
+//
+// The residual maximum of N increments: |d| as d ^ (d >> 63) (one less if
+// negative).  Its high word is at least the running maximum's only if some
+// high word of d lies outside (~t, t), so a plane usually costs two 32-bit
+// compares a point instead of a 64-bit magnitude, compare and select.
+template <int N> JD void fx_residual(const i64 (&d)[N], u64& rmax) {
+  int hi = (int)(d[0] >> 32), lo = hi;
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      if ((side == 0 && cz0 == 0) || (side == 1 && cz1 == nz)) {
-        const i64 off = side ? (nz - 1) * sz : 0;
-        double t[V];
-        ldv<double, V>(urow + off, t);
-#pragma unroll
-        for (int e = 0; e < V; ++e) t[e] = bnd_out(t[e], cvt(t[e]));
-        stv<double, V>(vrow + off, t);
-      }
-    }
+  for (int k = 1; k < N; ++k) {
+    hi = max(hi, (int)(d[k] >> 32));
+    lo = min(lo, (int)(d[k] >> 32));
   }
-  const i64 z0 = cz0 < 1 ? 1 : cz0;
-  const i64 z1 = cz1 > nz - 1 ? nz - 1 : cz1;
-  if (z0 >= z1) return;  // block-uniform
-
-  unsigned intm, bndm;
-  col_masks<V>(x0, nx, intm, bndm);
-  const bool rowb = (y == 0) || (y == ny - 1);
-  const bool yint = act && !rowb;
-  // halo sources of this thread (fixed per CTA and thread)
-  const bool has_top = (ty == 0) && (by0 >= 1) && (x0 < nx);
-  const bool has_bot = (ty == BY - 1) && (by0 + BY < ny) && (x0 < nx);
-  const double* hyp = u + (has_top ? by0 - 1 : by0 + BY) * nx + x0;
-  const bool has_xl = (tx == 0) && (bx0 >= 1) && (y < ny);
-  const bool has_xr = (tx == BX - 1) && (bx0 + BX * V < nx) && (y < ny);
-  const double* hxp = u + y * nx + (has_xl ? bx0 - 1 : bx0 + BX * V);
-
-  double rcur[V], rzn[V], rzn2[V], hy[V], hyn[V];
-  double hx = 0.0, hxn = 0.0;
-  i64 zp[V], cur[V], zn[V];
-  {
-    double t[V];
+  const int t = (int)(rmax >> 32);
+  if (hi >= t || lo <= ~t) {
 #pragma unroll
-    for (int e = 0; e < V; ++e) t[e] = rcur[e] = rzn[e] = rzn2[e] = hy[e] = hyn[e] = 0.0;
-    if (act) {
-      ldv<double, V>(urow + (z0 - 1) * sz, t);
-      ldv<double, V>(urow + z0 * sz, rcur);
-      ldv<double, V>(urow + (z0 + 1) * sz, rzn);
-      if (z0 + 2 < nz) ldv<double, V>(urow + (z0 + 2) * sz, rzn2);
+    for (int k = 0; k < N; ++k) {
+      const u64 a = (u64)(d[k] ^ (d[k] >> 63));
+      rmax = a > rmax ? a : rmax;
     }
-    if (has_top || has_bot) ldv<double, V>(hyp + z0 * sz, hy);
-    if (has_xl || has_xr) hx = __ldg(hxp + z0 * sz);
-#pragma unroll
-    for (int e = 0; e < V; ++e) { zp[e] = cvt(t[e]); cur[e] = cvt(rcur[e]); }
-  }
-  const i64 fb = p.fb, fw0 = p.fw0;
-  const int k = p.fk;
-  const bool small = p.fpath == JACC_FP_SMALL;
-  int b = 0;
-  i64 zoff = z0 * sz;
-  for (i64 z = z0; z < z1; ++z, zoff += sz) {
-#pragma unroll
-    for (int e = 0; e < V; ++e) zn[e] = cvt(rzn[e]);
-    // loads one plane ahead: own plane z+3, halo of plane z+1
-    double rn3[V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) rn3[e] = 0.0;
-    if (act && z + 3 < nz) ldv<double, V>(urow + zoff + 3 * sz, rn3);
-    if (z + 1 < z1) {
-      if (has_top || has_bot) ldv<double, V>(hyp + zoff + sz, hyn);
-      if (has_xl || has_xr) hxn = __ldg(hxp + zoff + sz);
-    }
-    // this plane into shared memory
-    i64* row = &sm.a[b][ty + 1][V + tx * V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) row[e] = cur[e];
-    if (has_top || has_bot) {
-      i64* hr = &sm.a[b][has_top ? 0 : BY + 1][V + tx * V];
-#pragma unroll
-      for (int e = 0; e < V; ++e) hr[e] = cvt(hy[e]);
-    }
-    if (has_xl) sm.a[b][ty + 1][V - 1] = cvt(hx);
-    if (has_xr) sm.a[b][ty + 1][V + BX * V] = cvt(hx);
-    __syncthreads();
-    const i64* rm = &sm.a[b][ty][V + tx * V];
-    const i64* r0 = &sm.a[b][ty + 1][V + tx * V];
-    const i64* rp = &sm.a[b][ty + 2][V + tx * V];
-    double out[V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) {
-      const bool in = yint && ((intm >> e) & 1u);
-      const i64 xl = (e == 0) ? r0[-1] : cur[e - 1];
-      const i64 xr = (e == V - 1) ? r0[V] : cur[e + 1];
-      const i64 sum = ((xl + xr) + (rm[e] + rp[e])) + (zp[e] + zn[e]);
-      const i64 L = sum - 6 * cur[e];
-      // the increment v - c in fixed point: v = c + round(r L)
-      const i64 dv = small ? fx_round_shift(fb * L, k) : fx128_round_shift(mul_s64_u64(L, (u64)fw0), k);
-      double o;
-      if (outf) {
-        if (small) o = fx_to(cur[e] * ((i64)1 << k) + fb * L, F + k);
-        else o = fx128_to(add128(from_s64_shl(cur[e], k), mul_s64_u64(L, (u64)fw0)), F + k);
-      } else {
-        o = i64_bits(cur[e] + dv);
-      }
-      out[e] = in ? o : bnd_out(rcur[e], cur[e]);
-      const u64 aL = (u64)(dv ^ (dv >> 63));  // |v - c| (one less for negative: 2^-F, below the tolerance)
-      rmax = (in && aL > rmax) ? aL : rmax;
-    }
-    if (act) stv<double, V>(vrow + zoff, out);
-#pragma unroll
-    for (int e = 0; e < V; ++e) {
-      zp[e] = cur[e];
-      cur[e] = zn[e];
-      rcur[e] = rzn[e];
-      rzn[e] = rzn2[e];
-      rzn2[e] = rn3[e];
-      hy[e] = hyn[e];
-    }
-    hx = hxn;
-    b ^= 1;
   }
 }
 
-// Residual of the heat sweep from max |L|: r max|L| scaled.
+JD i64 heat_increment(i64 L, u64 fm) {
+  const u64 b = (u64)L + (1ull << 62);
+  const u32 bl = (u32)b, bh = (u32)(b >> 32), ml = (u32)fm, mh = (u32)(fm >> 32);
+  u64 mid = (u64)bl * mh + (((u64)bl * ml) >> 32);  // < 2^61
+  mid = (u64)bh * ml + mid + (1ull << 29);          // bh < 2^31
+  const u64 hi = (u64)bh * mh + (mid >> 32);
+  return (i64)(((hi << 2) | ((u32)mid >> 30)) - fm);
+}
 
 // ---------------------------------------------------------------- 7-point heat, bulk-copy staged planes
 //
@@ -1538,7 +1424,7 @@ template <class A> struct SameT<A, A> { static constexpr bool value = true; };
 template <class T, bool FX> struct HeatAcc { typedef T type; };
 template <> struct HeatAcc<double, true> { typedef u64 type; };
 
-template <class T, int BX, int BY, int ZC, bool FX, bool EDGE, int SC, class P>
+template <class T, int BX, int BY, bool FX, bool EDGE, int SC, class P>
 JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, int F, int flags,
                     typename HeatAcc<T, FX>::type& rmax, Heat3SSmem<T, BX, BY, SC>& sm) {
   typedef Heat3S<T, BX, BY, SC> G;
@@ -1559,8 +1445,8 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
 #pragma unroll
     for (int e = 0; e < V; ++e)
       if (y0 + yy >= 1 && y0 + yy <= ny - 2 && x0 + e >= 1 && x0 + e <= nx - 2) inm |= 1u << (yy * V + e);
-  const i64 cz0 = (i64)blockIdx.z * ZC;
-  const i64 cz1 = (cz0 + ZC < nz) ? cz0 + ZC : nz;
+  const i64 cz0 = (i64)blockIdx.z * p.zc;
+  const i64 cz1 = (cz0 + p.zc < nz) ? cz0 + p.zc : nz;
   const i64 z0 = cz0 < 1 ? 1 : cz0;
   const i64 z1 = cz1 > nz - 1 ? nz - 1 : cz1;
   const bool inf = FX && EDGE && (flags & JFX_IN_F64);
@@ -1746,8 +1632,7 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
             o = outf ? fx_to(ce * ((i64)1 << k) + fb * (sum - 6 * ce), F + k) : i64_bits(vn);
           } else {
             const i64 Ld = sum - 6 * ce;
-            if (small) dv = fx_round_shift(fb * Ld, k);
-            else dv = fx128_round_shift(mul_s64_u64(Ld, (u64)fw0), k);
+            dv = heat_increment(Ld, p.fm);
             if (outf) {
               if (small) o = fx_to(ce * ((i64)1 << k) + fb * Ld, F + k);
               else o = fx128_to(add128(from_s64_shl(ce, k), mul_s64_u64(Ld, (u64)fw0)), F + k);
@@ -1889,6 +1774,208 @@ template <int BX, int BY, int CH> JD void ring_to_fixed(const RingPlan<double, B
     }
 }
 
+// ---------------------------------------------------------------- 7-point heat, planes staged by asynchronous copies
+//
+// FX: FP64 storage in the resident 64-bit fixed point (EDGE: the first and
+// last sweeps of a sequence and single launches, whose staged values the
+// copying threads convert in place); otherwise native arithmetic on T.  A
+// thread keeps its own values of planes z-1 and z in registers and reads its
+// values of plane z+1 and its neighbours in plane z from the stages; two
+// planes of look-ahead (stage j is free once step j is done, so plane j + S
+// - 2 is requested after the barrier that opens step j - 1).  Bound by the
+// integer ALU work (79 thread-instructions a point, 143 in the kernel that
+// loaded halos into registers and multiplied in 128 bits): 301 x 253 x 199,
+// r = 0.1, 90 us a sweep before, 57 now (4.2 TB/s); FP32 rows of odd length
+// 301 x 253 x 199 27.5 us.
+template <class T, int BX, int BY, int CH, bool FX, bool EDGE, class P>
+JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, int F, int flags,
+                    typename HeatAcc<T, FX>::type& rmax, T* sm) {
+  typedef RingG<T, BX, BY, CH> G;
+  typedef typename WT<T, FX ? JM_FIXED : JM_NATIVE>::type Wt;
+  constexpr int RY = G::RY, S = G::S;
+  const i64 nx = p.nx, ny = p.ny, nz = p.nz, sz = nx * ny;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const i64 bx0 = (i64)blockIdx.x * G::TW, by0 = (i64)blockIdx.y * G::TH;
+  const i64 x = bx0 + tx, y0 = by0 + ty * RY;
+  // rows this thread writes, and those whose point is interior
+  unsigned wrm = 0, inm = 0;
+#pragma unroll
+  for (int k = 0; k < RY; ++k) {
+    if (x < nx && y0 + k < ny) wrm |= 1u << k;
+    if (x >= 1 && x <= nx - 2 && y0 + k >= 1 && y0 + k <= ny - 2) inm |= 1u << k;
+  }
+  const bool fast = __all_sync(0xffffffffu, inm == (1u << RY) - 1);  // the warp holds interior points only
+  const i64 cz0 = (i64)blockIdx.z * p.zc;
+  const i64 cz1 = (cz0 + p.zc < nz) ? cz0 + p.zc : nz;
+  const i64 z0 = cz0 < 1 ? 1 : cz0;
+  const i64 z1 = cz1 > nz - 1 ? nz - 1 : cz1;
+  const bool inf = FX && EDGE && (flags & JFX_IN_F64);
+  const bool outf = FX && EDGE && (flags & JFX_OUT_F64);
+  const i64 own_off = y0 * nx + x;
+  T* vo = v + own_off;
+  // a boundary point's output from its working value (and, where FP64 goes
+  // in and out, its unchanged input at offset `at`)
+  auto bnd_out = [&](Wt w, i64 at) -> T {
+    if constexpr (FX && EDGE) {
+      if (outf) return inf ? u[at] : fx_to(w, F);
+      return i64_bits(w);
+    } else if constexpr (FX) {
+      return i64_bits(w);
+    } else {
+      return w;
+    }
+  };
+  if (z0 >= z1) {  // a chunk holding only a boundary plane (block-uniform)
+    for (i64 z = cz0; z < cz1; ++z)
+#pragma unroll
+      for (int k = 0; k < RY; ++k)
+        if ((wrm >> k) & 1u) {
+          const i64 at = own_off + z * sz + k * nx;
+          T t = u[at];
+          if constexpr (FX && EDGE) {
+            if (inf != outf) t = inf ? i64_bits(fx_from(t, F)) : fx_to(bits_i64(t), F);
+          }
+          v[at] = t;
+        }
+    return;
+  }
+  const int L = (int)(z1 - z0) + 2;  // staged planes z0-1 .. z1
+  RingPlan<T, BX, BY, CH> plan;
+  plan.init(nx, ny, bx0, by0, false);
+  const T* next = u + (z0 - 1) * sz;  // next plane to stage
+  int is = 0, issued = 0;             // its stage, in elements
+  auto issue_next = [&]() {
+    if (issued < L) plan.issue(sm + is, next);
+    cpa_commit();
+    ++issued;
+    next += sz;
+    is = is + G::STAGE == S * G::STAGE ? 0 : is + G::STAGE;
+  };
+#pragma unroll 1
+  for (int j = 0; j < S; ++j) issue_next();
+  int ns = 0;  // stage of the next plane, in elements
+  auto publish = [&]() {
+    if constexpr (FX && EDGE) {
+      if (inf) ring_to_fixed<BX, BY, CH>(plan, sm + ns, F);
+    }
+    __syncthreads();
+  };
+  const Wt* own0 = reinterpret_cast<const Wt*>(sm) + (ty * RY + 1) * G::W + CH + tx;
+  auto own = [&](int stage, Wt (&w)[RY]) {
+#pragma unroll
+    for (int k = 0; k < RY; ++k) w[k] = own0[stage + k * G::W];
+  };
+  auto store_bnd = [&](i64 z, const Wt (&w)[RY]) {
+#pragma unroll
+    for (int k = 0; k < RY; ++k)
+      if ((wrm >> k) & 1u) vo[z * sz + k * nx] = bnd_out(w[k], own_off + z * sz + k * nx);
+  };
+  Wt wa[RY], wb[RY], wc[RY];  // own values of planes z-1, z, z+1 (rotating roles)
+  cpa_wait<S - 1>();
+  publish();
+  own(ns, wa);
+  if (cz0 == 0) store_bnd(0, wa);  // boundary plane 0
+  ns += G::STAGE;
+  cpa_wait<S - 2>();
+  publish();
+  own(ns, wb);
+  int cs = ns;  // stage of the centre plane
+  ns += G::STAGE;
+  const T r = (T)p.c0;
+  constexpr bool folded = !SameT<P, JParams>::value;
+  const bool fold = folded && heat_fold(p);
+  const i64 fb = p.fb;
+  const int fk = p.fk;
+  i64 z = z0;
+  T* vz = vo + z0 * sz;
+  // output plane z from the own values of planes z-1 and z; fills zn with plane z+1's
+  auto step = [&](const Wt (&zp)[RY], const Wt (&cur)[RY], Wt (&zn)[RY]) {
+    cpa_wait<S - 3>();
+    publish();
+    issue_next();  // into the stage of plane z-1, last read before the barrier
+    own(ns, zn);
+    const Wt* c0 = own0 + cs;
+    const Wt ym = c0[-G::W], yp = c0[RY * G::W];
+    T out[RY];
+    Wt dv[RY];
+#pragma unroll
+    for (int k = 0; k < RY; ++k) {
+      const Wt xl = c0[k * G::W - 1], xr = c0[k * G::W + 1];
+      const Wt a = k == 0 ? ym : cur[k == 0 ? 0 : k - 1], b = k == RY - 1 ? yp : cur[k == RY - 1 ? k : k + 1];
+      const Wt sum = ((xl + xr) + (a + b)) + (zp[k] + zn[k]);
+      const Wt ce = cur[k];
+      if constexpr (FX) {
+        if (fold) {
+          const i64 vn = (fb * sum + ((((i64)1 << fk) - 6 * fb) * ce + ((i64)1 << (fk - 1)))) >> fk;
+          dv[k] = vn - ce;
+          out[k] = i64_bits(vn);
+        } else {
+          dv[k] = heat_increment(sum - 6 * ce, p.fm);
+          out[k] = i64_bits(ce + dv[k]);
+        }
+        if constexpr (EDGE) {
+          if (outf) {  // the exact value, rounded once
+            const i64 Ld = sum - 6 * ce;
+            if (p.fpath == JACC_FP_SMALL) out[k] = fx_to(ce * ((i64)1 << fk) + fb * Ld, F + fk);
+            else out[k] = fx128_to(add128(from_s64_shl(ce, fk), mul_s64_u64(Ld, (u64)p.fw0)), F + fk);
+          }
+        }
+      } else {
+        const T o = ce + r * (sum - T(6) * ce);
+        out[k] = o;
+        dv[k] = o - ce;
+      }
+    }
+    if (!fast) {
+#pragma unroll
+      for (int k = 0; k < RY; ++k)
+        if (!((inm >> k) & 1u)) {
+          dv[k] = Wt(0);
+          if ((wrm >> k) & 1u) out[k] = bnd_out(cur[k], own_off + z * sz + k * nx);
+        }
+    }
+    if constexpr (FX) fx_residual<RY>(dv, rmax);
+    else {
+#pragma unroll
+      for (int k = 0; k < RY; ++k) rmax = fmaxf(rmax, fabsf(dv[k]));
+    }
+    if (fast) {
+#pragma unroll
+      for (int k = 0; k < RY; ++k) vz[k * nx] = out[k];
+    } else {
+#pragma unroll
+      for (int k = 0; k < RY; ++k)
+        if ((wrm >> k) & 1u) vz[k * nx] = out[k];
+    }
+    cs = ns;
+    ns = ns + G::STAGE == S * G::STAGE ? 0 : ns + G::STAGE;
+    ++z;
+    vz += sz;
+  };
+  // three steps per iteration: the buffers' roles rotate without copies
+  const int n = L - 2;
+  int j = 0;
+#pragma unroll 1
+  for (; j + 3 <= n; j += 3) {
+    step(wa, wb, wc);
+    step(wb, wc, wa);
+    step(wc, wa, wb);
+  }
+  // plane nz-1 (the last staged one) is in the buffer that the last step filled
+  if (n - j == 0) {
+    if (cz1 == nz) store_bnd(nz - 1, wb);
+  } else {
+    step(wa, wb, wc);
+    if (n - j == 1) {
+      if (cz1 == nz) store_bnd(nz - 1, wc);
+    } else {
+      step(wb, wc, wa);
+      if (cz1 == nz) store_bnd(nz - 1, wa);
+    }
+  }
+  cpa_wait<0>();
+}
+
 // ---------------------------------------------------------------- 27-point box, resident fixed point
 //
 // v 2^F = round(sum_j fw_j class_j 2^-K) from the exact sum; the FP64 output
@@ -1941,22 +2028,30 @@ template <class P> JD i64 box27_weigh(const P& p, i64 c, i64 f, i64 e, i64 g, s1
   return fx128_round_shift(a, K);
 }
 
-template <int BX, int BY, int CH, bool EDGE, class P>
-JD void box27_fx_body(const double* __restrict__ u, double* __restrict__ v, const P& p, const JParams& rt, int F,
-                      int flags, s128& acc, double* sm) {
-  typedef RingG<double, BX, BY, CH> G;
+// The running 27-point march over staged planes, for FP64 in fixed point
+// (W = i64; EDGE as above) and for native FP32 (W = float: the definition's
+// terms in the order of box27_body2, fused field sum in `acc32`; 501 x 487 x
+// 383, rows of odd length, 447 us a sweep with planes loaded through registers
+// one step ahead, 227 here).
+template <class T, int BX, int BY, int CH, bool EDGE, class P>
+JD void box27r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, int F, int flags,
+                    bool want_sum, s128& acc, SumAcc<float>& acc32, T* sm) {
+  typedef RingG<T, BX, BY, CH> G;
+  constexpr bool FX = sizeof(T) == 8;
+  typedef typename WT<T, FX ? JM_FIXED : JM_NATIVE>::type W;
   constexpr int RY = G::RY, S = G::S;
   const i64 nx = p.nx, ny = p.ny, nz = p.nz, sz = nx * ny;
+  const int zc = p.zc;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const i64 bx0 = (i64)blockIdx.x * G::TW, by0 = (i64)blockIdx.y * G::TH;
   const i64 x0 = bx0 + tx, y0 = by0 + ty * RY;
-  const i64 z0 = (i64)blockIdx.z * rt.zc;
-  const i64 z1 = (z0 + rt.zc < nz) ? z0 + rt.zc : nz;
+  const i64 z0 = (i64)blockIdx.z * zc;
+  const i64 z1 = (z0 + zc < nz) ? z0 + zc : nz;
   const int L = (int)(z1 - z0) + 2;  // staged planes z0-1 .. z1 (periodic images)
   const int nrow = x0 < nx ? (int)(ny - y0 < RY ? (ny - y0 > 0 ? ny - y0 : 0) : RY) : 0;  // rows this thread writes
   const bool inf = EDGE && (flags & JFX_IN_F64);
   const bool outf = EDGE && (flags & JFX_OUT_F64);
-  RingPlan<double, BX, BY, CH> plan;
+  RingPlan<T, BX, BY, CH> plan;
   plan.init(nx, ny, bx0, by0, true);
   i64 zi = z0 == 0 ? nz - 1 : z0 - 1;  // next plane to stage
   int is = 0;                          // and its stage, in elements
@@ -1973,15 +2068,15 @@ JD void box27_fx_body(const double* __restrict__ u, double* __restrict__ v, cons
   int cs = 0;  // the stage to read, in elements
   // own-column sums of the next staged plane: c the points, f their four
   // in-plane faces, g the four in-plane diagonals
-  auto consume = [&](i64 (&c)[RY], i64 (&f)[RY], i64 (&g)[RY]) {
+  auto consume = [&](W (&c)[RY], W (&f)[RY], W (&g)[RY]) {
     cpa_wait<S - 2>();
-    if constexpr (EDGE) {
+    if constexpr (FX && EDGE) {
       if (inf) ring_to_fixed<BX, BY, CH>(plan, sm + cs, F);
     }
     __syncthreads();
     issue_next();  // into the stage read before the barrier
-    const i64* r = reinterpret_cast<const i64*>(sm) + cs + ty * RY * G::W + CH + tx;
-    i64 m[RY + 2], s[RY + 2];
+    const W* r = reinterpret_cast<const W*>(sm) + cs + ty * RY * G::W + CH + tx;
+    W m[RY + 2], s[RY + 2];
 #pragma unroll
     for (int k = 0; k < RY + 2; ++k) {
       m[k] = r[k * G::W];
@@ -1996,39 +2091,51 @@ JD void box27_fx_body(const double* __restrict__ u, double* __restrict__ v, cons
     cs = cs + G::STAGE == S * G::STAGE ? 0 : cs + G::STAGE;
   };
   // running classes of the output plane: pf = f(z) + c(z-1), pe = g(z) + f(z-1), pc = g(z-1)
-  i64 pf[RY], pe[RY], pc[RY];
-  double* vo = v + z0 * sz + y0 * nx + x0;
-  auto step = [&](const i64 (&c0)[RY], const i64 (&f0)[RY], const i64 (&g0)[RY], i64 (&cn)[RY], i64 (&fn)[RY],
-                  i64 (&gn)[RY]) {
+  W pf[RY], pe[RY], pc[RY];
+  const float w0 = (float)p.c0, wf = (float)p.c1, we = (float)p.c2, wc = (float)p.c3;
+  T* vo = v + z0 * sz + y0 * nx + x0;
+  auto step = [&](const W (&c0)[RY], const W (&f0)[RY], const W (&g0)[RY], W (&cn)[RY], W (&fn)[RY], W (&gn)[RY]) {
     consume(cn, fn, gn);
-    i64 rowsum = 0;  // at most four values below 2^58: exact
+    i64 rowsum = 0;  // at most four values below 2^59: exact
 #pragma unroll
     for (int k = 0; k < RY; ++k) {
-      double o;
-      i64 q;
-      if (EDGE && outf) {
-        s128 ex;
-        q = box27_weigh(p, c0[k], pf[k] + cn[k], pe[k] + fn[k], pc[k] + gn[k], &ex);
-        o = fx128_to(ex, F + p.fk);
+      const W cf = pf[k] + cn[k], ce = pe[k] + fn[k], cc = pc[k] + gn[k];
+      if constexpr (FX) {
+        double o;
+        i64 q;
+        if (EDGE && outf) {
+          s128 ex;
+          q = box27_weigh(p, c0[k], cf, ce, cc, &ex);
+          o = fx128_to(ex, F + p.fk);
+        } else {
+          q = box27_weigh(p, c0[k], cf, ce, cc, nullptr);
+          o = i64_bits(q);
+        }
+        if (k < nrow) {
+          vo[k * nx] = o;
+          rowsum += q;
+        }
       } else {
-        q = box27_weigh(p, c0[k], pf[k] + cn[k], pe[k] + fn[k], pc[k] + gn[k], nullptr);
-        o = i64_bits(q);
+        // the fused multiply-adds written out: one rounding pattern for every variant
+        const float o = __fadd_rn(fmaf(w0, c0[k], __fmul_rn(wf, cf)), fmaf(we, ce, __fmul_rn(wc, cc)));
+        if (k < nrow) {
+          vo[k * nx] = o;
+          if (want_sum) acc32.add(o);
+        }
       }
       pf[k] = fn[k] + c0[k];
       pe[k] = gn[k] + f0[k];
       pc[k] = g0[k];
-      if (k < nrow) {
-        vo[k * nx] = o;
-        rowsum += q;
-      }
     }
     vo += sz;
-    s128 t;
-    t.lo = (u64)rowsum;
-    t.hi = (u64)(rowsum >> 63);
-    acc = add128(acc, t);
+    if constexpr (FX) {
+      s128 t;
+      t.lo = (u64)rowsum;
+      t.hi = (u64)(rowsum >> 63);
+      acc = add128(acc, t);
+    }
   };
-  i64 ca[RY], fa[RY], ga[RY], cb[RY], fb[RY], gb[RY];
+  W ca[RY], fa[RY], ga[RY], cb[RY], fb[RY], gb[RY];
   consume(ca, fa, ga);
   consume(cb, fb, gb);
 #pragma unroll
@@ -2113,55 +2220,58 @@ JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, c
   block_max_to<BX * BY>(bits, resid);
 }
 
-template <class T, int BX, int BY, int V, int ZC, bool EDGE, class P>
+template <class T, int BX, int BY, int V, bool EDGE, class P>
 JD void heat3d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                      const u64* maxword, int flags) {
   griddep_wait();
   u64 bits = 0;
+  // 16-byte columns: the bulk-copy staged kernel (2 rows per thread), else
+  // the kernel staged by asynchronous copies (RingG::RY rows of one column)
+  constexpr bool STAGED = V * sizeof(T) == 16;
   if constexpr (sizeof(T) == 8) {
-    // 16-byte columns: the staged kernel (2 rows per thread, so a CTA covers
-    // 2 BY rows; the native fallback then runs two BY-row sub-tiles)
-    constexpr bool STAGED = V == 2;
-    constexpr size_t SM_PLANE = sizeof(Plane<i64, BX, BY, V>);
+    typedef RingG<double, BX, BY, V> G;
     // stage cap: 5 for the constant-folded intermediate sweeps (7 CTAs per SM,
     // SweepMinBlocks), else 6
     constexpr int SC = (!EDGE && !SameT<P, JParams>::value) ? 5 : 6;
-    constexpr size_t SM_STAGED = STAGED ? sizeof(Heat3SSmem<double, BX, BY, SC>) : 0;
-    __shared__ __align__(128) unsigned char raw[SM_PLANE > SM_STAGED ? SM_PLANE : SM_STAGED];
+    // the native path covers the CTA's rows in sub-tiles of BY rows
+    constexpr int SUBS = STAGED ? 2 : G::RY;
+    typedef Plane<double, BX, BY, V> NativePlane;
+    constexpr size_t SM_MAIN = STAGED ? sizeof(Heat3SSmem<double, BX, BY, SC>) : (size_t)G::S * G::STAGE * 8;
+    __shared__ __align__(128) unsigned char raw[sizeof(NativePlane) > SM_MAIN ? sizeof(NativePlane) : SM_MAIN];
     const int F = (maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
     if (F >= 0) {
       u64 m = 0;
       if constexpr (STAGED)
-        heat3s_body<double, BX, BY, ZC, true, EDGE, SC>(u, v, p, rt, F, flags, m,
+        heat3s_body<double, BX, BY, true, EDGE, SC>(u, v, p, rt, F, flags, m,
                                                         *reinterpret_cast<Heat3SSmem<double, BX, BY, SC>*>(raw));
       else
-        heat3d_fx_body<EDGE, BX, BY, V, ZC>(u, v, p, F, flags, m, *reinterpret_cast<Plane<i64, BX, BY, V>*>(raw));
+        heat3r_body<double, BX, BY, V, true, EDGE>(u, v, p, rt, F, flags, m, reinterpret_cast<double*>(raw));
       bits = dbits(fx_to_u(m, F));  // max |v - c| in fixed point
     } else {
       double m = 0.0;
 #pragma unroll 1
-      for (int sub = 0; sub < (STAGED ? 2 : 1); ++sub) {
+      for (int sub = 0; sub < SUBS; ++sub) {
         if (sub) __syncthreads();  // the sub-tiles share the planes
-        heat3d_body<T, BX, BY, V, ZC, JM_NATIVE>(u, v, p, -1, m, *reinterpret_cast<Plane<double, BX, BY, V>*>(raw),
-                                                 STAGED ? 2 : 1, sub);
+        heat3d_body<T, BX, BY, V, JM_NATIVE>(u, v, p, p.zc, -1, m, *reinterpret_cast<NativePlane*>(raw), SUBS, sub);
       }
       bits = dbits(m);
     }
-  } else if constexpr (V == 4) {
+  } else if constexpr (STAGED) {
     __shared__ Heat3SSmem<float, BX, BY, 6> sm;
     float m = 0.0f;
-    heat3s_body<float, BX, BY, ZC, false, false, 6>(u, v, p, rt, -1, 0, m, sm);
+    heat3s_body<float, BX, BY, false, false, 6>(u, v, p, rt, -1, 0, m, sm);
     bits = dbits((double)m);
   } else {
-    __shared__ Plane<T, BX, BY, V> sm;
-    T m = T(0);
-    heat3d_body<T, BX, BY, V, ZC, JM_NATIVE>(u, v, p, -1, m, sm);
+    typedef RingG<float, BX, BY, V> G;
+    __shared__ __align__(16) float sm[G::S * G::STAGE];
+    float m = 0.0f;
+    heat3r_body<float, BX, BY, V, false, false>(u, v, p, rt, -1, 0, m, sm);
     bits = dbits((double)m);
   }
   block_max_to<BX * BY>(bits, resid);
 }
 
-template <class T, int BX, int BY, int V, int ZC, bool EDGE, class P>
+template <class T, int BX, int BY, int V, bool EDGE, class P>
 JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                     const u64* maxword, int flags) {
   griddep_wait();
@@ -2174,24 +2284,27 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
     if (F >= 0) {
       s128 acc;
       acc.lo = acc.hi = 0ull;
-      box27_fx_body<BX, BY, V, EDGE>(u, v, p, rt, F, flags, acc, reinterpret_cast<double*>(raw));
+      SumAcc<float> none;
+      box27r_body<double, BX, BY, V, EDGE>(u, v, p, rt, F, flags, false, acc, none, reinterpret_cast<double*>(raw));
       total = fx128_to(acc, F);
     } else {
       SumAcc<T> acc;
 #pragma unroll 1
       for (int sub = 0; sub < G::RY; ++sub) {
         __syncthreads();  // the sub-tiles share the planes
-        box27_body2<T, BX, BY, 1>(u, v, p, rt.zc, acc, resid != nullptr, *reinterpret_cast<Plane<double, BX, BY, 1>*>(raw),
+        box27_body2<T, BX, BY, 1>(u, v, p, p.zc, acc, resid != nullptr, *reinterpret_cast<Plane<double, BX, BY, 1>*>(raw),
                                   G::RY, sub);
       }
       total = acc.total();
     }
   } else if constexpr (V == 4) {
-    total = box27s_body<BX, BY, ZC>(u, v, p, rt, resid != nullptr);
+    total = box27s_body<BX, BY>(u, v, p, rt, resid != nullptr);
   } else {
-    __shared__ Plane<T, BX, BY, V> sm;
-    SumAcc<T> acc;
-    box27_body2<T, BX, BY, V>(u, v, p, ZC, acc, resid != nullptr, sm);
+    typedef RingG<float, BX, BY, V> G;
+    __shared__ __align__(16) float sm[G::S * G::STAGE];
+    SumAcc<float> acc;
+    s128 none;
+    box27r_body<float, BX, BY, V, false>(u, v, p, rt, -1, 0, resid != nullptr, none, acc, sm);
     total = acc.total();
   }
   block_sum_to<BX * BY>(total, resid);
@@ -2284,16 +2397,23 @@ __global__ void jacc_k_fill_skipped(double* resid, int n, int T) {
 // and, unbounded, take 124 registers (4 CTAs), so they ask for 6 (80
 // registers, 6 stages); the converting sweeps at 5 CTAs (at most 102
 // registers, from 157) take 2.40 ms for a 2-sweep sequence against 2.83.
+// The 7-point kernels staged by asynchronous copies (scalar columns, 32 x 4
+// threads): 5 CTAs (at most 102 registers); folded, 511^3 FP64 434 us a sweep
+// against 445 unbounded (4 CTAs), 444 at 6 and 557 at 7 (spills).
 // For the FP64 27-point kernel with 32 x 4 threads: 4 CTAs (at most 128
 // registers); folded, 512^3: 490 us a sweep against 492 unbounded (3 CTAs)
 // and 518 at 5 (spills).
+// The precompiled staged FP32 27-point kernel: 7 CTAs (at most 72 registers;
+// left alone it spills at 64).
 // Every other kernel: 0, no requirement (a bound of 1 is not neutral: it
 // lets the compiler take registers for one CTA per SM, e.g. 111 instead of
 // 80 for the staged FP32 7-point kernel).
 template <int STENCIL, class T, int BX, int BY, int V, bool EDGE, bool FOLDED> struct SweepMinBlocks {
   static constexpr bool heat_staged_fp64 = STENCIL == 7 && sizeof(T) == 8 && BX == 32 && BY == 4 && V == 2;
   static constexpr bool box27_fp64 = STENCIL == 27 && sizeof(T) == 8 && BX == 32 && BY == 4;
-  static constexpr int value = heat_staged_fp64 ? (EDGE ? 5 : (FOLDED ? 7 : 6)) : (box27_fp64 && !EDGE ? 4 : 0);
+  static constexpr bool heat_ring = STENCIL == 7 && BX == 32 && BY == 4 && V == 1 && !EDGE;
+  static constexpr bool box27_fp32 = STENCIL == 27 && sizeof(T) == 4 && BX == 32 && BY == 4 && V == 4 && !FOLDED;
+  static constexpr int value = box27_fp32 ? 7 : heat_ring ? 5 : heat_staged_fp64 ? (EDGE ? 5 : (FOLDED ? 7 : 6)) : (box27_fp64 && !EDGE ? 4 : 0);
 };
 
 // The constant-folded last sweep of a sequence that does not convert on load
@@ -2310,11 +2430,11 @@ __global__ void __launch_bounds__(BX * BY) jacc_k_jacobi2d(const T* __restrict__
                                                            double* resid, const u64* maxword, int flags) {
   jacobi2d_entry<T, BX, BY, V, ZC, EDGE>(u, v, p, p, resid, maxword, flags);
 }
-template <class T, int BX, int BY, int V, int ZC, bool EDGE>
+template <class T, int BX, int BY, int V, bool EDGE>
 __global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<7, T, BX, BY, V, EDGE, false>::value))
     jacc_k_heat3d(const T* __restrict__ u, T* __restrict__ v, JParams p,
                                                          double* resid, const u64* maxword, int flags) {
-  heat3d_entry<T, BX, BY, V, ZC, EDGE>(u, v, p, p, resid, maxword, flags);
+  heat3d_entry<T, BX, BY, V, EDGE>(u, v, p, p, resid, maxword, flags);
 }
 template <int RY, int TT, int ZC>
 __global__ void __launch_bounds__(TB_BX * RY) jacc_k_box27_tb(const float* __restrict__ u, float* __restrict__ v,
@@ -2325,8 +2445,8 @@ __global__ void __launch_bounds__(TB_BX * RY) jacc_k_box27_tb(const float* __res
 struct JParamsW32 : JParams {
   static constexpr int fpath = JACC_FP_W32;
 };
-template <class T, int BX, int BY, int V, int ZC, bool EDGE, class P>
+template <class T, int BX, int BY, int V, bool EDGE, class P>
 __global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<27, T, BX, BY, V, EDGE, false>::value))
     jacc_k_box27(const T* __restrict__ u, T* __restrict__ v, P p, double* resid, const u64* maxword, int flags) {
-  box27_entry<T, BX, BY, V, ZC, EDGE>(u, v, p, p, resid, maxword, flags);
+  box27_entry<T, BX, BY, V, EDGE>(u, v, p, p, resid, maxword, flags);
 }

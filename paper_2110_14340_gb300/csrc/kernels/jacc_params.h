@@ -8,7 +8,7 @@ typedef unsigned int u32;
 
 // Fixed-point path selector (JParams::fpath).
 #define JACC_FP_NONE 0   // native arithmetic only
-#define JACC_FP_SMALL 1  // 7pt, r = fb 2^-k with k <= 5: v 2^(F+k) = fa u + fb S in int64
+#define JACC_FP_SMALL 1  // 7pt, r = fb 2^-k with k <= 5: the FP64 output in 64 bits
 #define JACC_FP_WIDE 2   // 7pt / 27pt: exact 128-bit products
 #define JACC_FP_JACOBI 3 // 5pt: v 2^(F+2) = S
 #define JACC_FP_W32 4    // 27pt: every factor below 2^31 and K in [1, 31]: 32-bit factors
@@ -21,7 +21,8 @@ typedef unsigned int u32;
 struct JParams {
   i64 nx, ny, nz;
   double c0, c1, c2, c3;   // coefficients for the native path: 7pt r; 27pt w0, wf, we, wc
-  i64 fa, fb;              // JACC_FP_SMALL factors
+  u64 fm;                  // 7pt: r 2^62
+  i64 fb;                  // JACC_FP_SMALL: r = fb 2^-fk
   i64 fw0, fw1, fw2, fw3;  // JACC_FP_WIDE factors (7pt: fw0 = odd mantissa of r)
   int fk;                  // extra fraction bits of the fixed-point result
   int fpath;               // JACC_FP_*

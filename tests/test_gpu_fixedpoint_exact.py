@@ -85,3 +85,43 @@ def test_box27_f64_equals_integer_arithmetic(coeffs, shape, tile, jit):
     assert np.array_equal(g, as_f64(exact, F + K))
     # the field sum: exact per thread, then FP64 additions of the threads' parts
     assert np.max(np.abs(gs - np.array(sums))) <= 1e-12 * float(np.sum(np.abs(u)))
+
+
+def heat_sum(q):
+    c = q[1:-1, 1:-1, 1:-1]
+    return (q[1:-1, 1:-1, :-2] + q[1:-1, 1:-1, 2:] + q[1:-1, :-2, 1:-1] + q[1:-1, 2:, 1:-1] + q[:-2, 1:-1, 1:-1]
+            + q[2:, 1:-1, 1:-1] - 6 * c)
+
+
+@pytest.mark.parametrize("r", [0.125, 0.0625, 3 / 64, 0.1, 1 / 6, 0.003, 0.0])
+@pytest.mark.parametrize("shape", [(3, 3, 3), (5, 17, 33), (9, 18, 64), (17, 16, 31), (4, 35, 97)])
+@pytest.mark.parametrize("tile,jit", [(-1, False), (0, False), (3, False), (22, False), (-1, True)])
+def test_heat3d_f64_equals_integer_arithmetic(r, shape, tile, jit):
+    nz, ny, nx = shape
+    if tile == 3 and nx % 2:
+        tile = 2
+    u = 2.0 * inputs.uniform64(32, nx * ny * nz).reshape(shape) - 1.0
+    F = frac_bits(u)
+    w, k2 = weights([r])
+    k = jacc.Kernel(jacc.STENCIL_7PT, jacc.F64, nx, ny, nz, coeffs=(r,), tile_id=tile, jit=jit)
+    assert k.info()["fixed_point"]
+    inner = (slice(1, -1),) * 3
+    q = to_fixed(u, F)
+    resids = []
+    for n in range(1, 5):
+        exact = q * (1 << k2)
+        exact[inner] = exact[inner] + w[0] * heat_sum(q)
+        new = np.vectorize(lambda x: round_up(x, k2), otypes=[object])(exact)
+        d = new - q
+        resids.append(max(int(x) if x >= 0 else -int(x) - 1 for x in d[inner].ravel()))
+        if n in (1, 2, 4):
+            g, gr = run(k, u, n)
+            want = as_f64(exact, F + k2)
+            if n == 1:  # a single sweep copies the boundary
+                edge = np.ones(shape, bool)
+                edge[inner] = False
+                want[edge] = u[edge]
+            assert np.array_equal(g, want)
+            assert np.array_equal(gr, as_f64(np.array(resids, dtype=object), F))
+        q = new
+    assert k.status() == 0
