@@ -177,14 +177,18 @@ extern "C" jacc_status jacc_costmodel_train(jacc_costmodel h, const float* x_dev
                                0.999f, 1e-8f, nullptr, q),
                       "MLP Adam step");
   };
-  // Capture a block of steps as one graph and replay it.
-  const int K = epochs < 64 ? epochs : 64;
+  // Capture a block of steps as one graph and replay it; a run of few steps is
+  // launched directly (capturing and instantiating 64 steps costs the host
+  // more than launching 128 of them).
+  const int K = 64;
   cudaStream_t cap = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  st = cuda_check(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "cudaStreamCreate");
-  if (!st) st = cuda_check(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
-  if (!st) {
+  const bool graphed = epochs > 2 * K;
+  if (graphed) st = cuda_check(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "cudaStreamCreate");
+  if (!st && graphed)
+    st = cuda_check(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
+  if (!st && graphed) {
     jacc_status est = ok();
     for (int k = 0; k < K && !est; ++k) est = step(cap, k == K - 1 ? loss_dev : nullptr);
     cudaError_t ce = cudaStreamEndCapture(cap, &graph);
@@ -192,7 +196,7 @@ extern "C" jacc_status jacc_costmodel_train(jacc_costmodel h, const float* x_dev
     if (!st) st = cuda_check(cudaGraphInstantiate(&exec, graph, 0), "cudaGraphInstantiate");
   }
   int done = 0;
-  while (!st && done + K <= epochs) {
+  while (!st && graphed && done + K <= epochs) {
     st = cuda_check(cudaGraphLaunch(exec, s), "cudaGraphLaunch(train)");
     done += K;
   }
