@@ -62,6 +62,7 @@ struct Kernel {
   int smem = 0;                 // dynamic shared memory per CTA of `func`
   int tblock = 1;
   int cluster_nc = 0;           // JACC_SPEC_CLUSTER: CTAs of the cluster-resident sweep launch
+  int until_nc = -1;            // CTAs of the cluster that runs jacc_sweep_until (0: none fits, -1: not asked yet)
   int refcount = 0;
   u64* scratch = nullptr;       // max-abs word for direct launches (device)
   std::map<GraphKey, SweepGraph> graphs;

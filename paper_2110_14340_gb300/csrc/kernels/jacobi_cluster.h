@@ -13,6 +13,12 @@ struct JClusterArgs {
   long long pitch;   // shared-memory row pitch in words (set by the launcher)
   int nsweeps;
   int native;        // 1: native FP64 arithmetic (JACC_ARITH_NATIVE)
+  // sweeps until a tolerance: at most nsweeps sweeps from u = u_out; the two
+  // buffers (res and oth are worked out from the count)
+  double* u_out;     // u0
+  double* keep;      // u1: also keeps the start of the running chunk
+  double tol;
+  int* status;       // receives the count and the result buffer
 };
 
 // 1 and the cluster size (16 or 8) if both fields of an nx x ny grid fit in
@@ -20,3 +26,5 @@ struct JClusterArgs {
 int jacobi_cluster_plan(long long nx, long long ny, int* nc_out);
 // One launch of one cluster of nc CTAs running all a.nsweeps sweeps.
 cudaError_t launch_jacobi_cluster(JClusterArgs a, int nc, cudaStream_t s);
+// The same until a residual is at most a.tol, a.nsweeps sweeps at most.
+cudaError_t launch_jacobi_cluster_until(JClusterArgs a, int nc, cudaStream_t s);
