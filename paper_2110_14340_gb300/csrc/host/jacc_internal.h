@@ -40,7 +40,7 @@ using GraphKey = std::tuple<const void*, const void*, int32_t, const double*>;
 struct UntilGraph {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
-  u64* scratch = nullptr;  // [0] max-abs word, [1] residual slot, [2] sweep counter, [3] spare residual slot
+  u64* scratch = nullptr;  // [0] max-abs word, [1] residual slot, [2] sweep counter and stop word, [3] spare slot
 };
 using UntilKey = std::tuple<const void*, const void*, int32_t, double, const double*, const int32_t*>;
 
@@ -59,6 +59,8 @@ struct Kernel {
   const void* func_last = nullptr;  // constant-folded FP64 last sweep that converts only on store (or null)
   cudaLibrary_t lib = nullptr;  // NVRTC module, if jit
   dim3 grid, block;
+  dim3 grid_out, block_out;     // geometry of func_out and func_last
+  int fam = 0;                  // JACC_FAM_*
   int smem = 0;                 // dynamic shared memory per CTA of `func`
   int tblock = 1;
   int cluster_nc = 0;           // JACC_SPEC_CLUSTER: CTAs of the cluster-resident sweep launch
@@ -95,8 +97,9 @@ cudaError_t launch_until_final(const int* counter, int* status, int recompute, c
 
 // Launch one sweep of `k` (no validation).  maxword may be null.  flags:
 // JFX_* bits (first sweep of a sequence reads FP64, last writes FP64).
+// stop (device, nullable): the kernel returns at once if it finds it set.
 cudaError_t launch_sweep_kernel(const Kernel& k, const void* u, void* v, double* resid, const u64* maxword, int flags,
-                                cudaStream_t s);
+                                cudaStream_t s, const int* stop = nullptr);
 constexpr int kFxIn = 1, kFxOut = 2;  // JFX_IN_F64, JFX_OUT_F64
 // Default limit of one bounded device wait (staged kernels): 2 s.
 constexpr int64_t kDefaultTimeoutNs = 2000000000;
@@ -121,8 +124,6 @@ std::mutex& global_mutex();
 // Tile validity for a descriptor (vector width and grid limits) and the
 // default tile; the autotuner's remembered pick for a shape (-1 if none).
 bool tile_valid(const jacc_kernel_desc& d, int t);
-// Tiles that run a bulk-copy staged kernel (2 rows per thread).
-bool staged_tile(const jacc_kernel_desc& d, int t);
 int default_tile(const jacc_kernel_desc& d);
 int tuned_tile(const jacc_kernel_desc& d);
 void remember_tile(const jacc_kernel_desc& d, int tile);

@@ -31,6 +31,13 @@ extern "C" const void* const jacc_tab_7_32_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_64_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_32_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_64_w32[JACC_NTILES];
+extern "C" const void* const jacc_tab_5_64_lib[6][2];
+extern "C" const void* const jacc_tab_5_32_lib[6][2];
+extern "C" const void* const jacc_tab_7_64_lib[6][2];
+extern "C" const void* const jacc_tab_7_32_lib[6][2];
+extern "C" const void* const jacc_tab_27_64_lib[6][2];
+extern "C" const void* const jacc_tab_27_64_lib_w32[6][2];
+extern "C" const void* const jacc_tab_27_32_lib[6][2];
 extern "C" const void* const jacc_tab_tb[2];
 
 namespace jacc {
@@ -183,35 +190,76 @@ static jacc_status validate(const jacc_kernel_desc& d) {
   return ok();
 }
 
-// The default tile, from the autotuner's timing tables on GB300 (5/7/27-point,
-// FP32 and FP64, sides 256-1024), by size class.  3D: 32 x 4 threads with
-// 16-byte columns; a 64-plane march (tile 3) when it still yields at least
-// 1024 CTAs, else a 16-plane march (tile 1) for more CTAs on small grids.
-// 2D: 128 x 2 threads, 16-byte columns, 16-row march (tile 17) from 2^19
-// points; 64 x 4 threads, scalar columns, 4-row march (tile 8) below, where
-// the grid lives in L2 and more, shorter CTAs hide latency better.  Scalar
-// 3D variants (2, 0) when nx is not a multiple of the vector width.
+// The library's own kernel (entry `row` of its table), or null.
+static const void* lib_entry(const jacc_kernel_desc& d, const JParams& p, int row, bool vec) {
+  const bool f64 = d.dtype == 64;
+  if (d.stencil == 5) return (f64 ? jacc_tab_5_64_lib : jacc_tab_5_32_lib)[row][vec];
+  if (d.stencil == 7) return (f64 ? jacc_tab_7_64_lib : jacc_tab_7_32_lib)[row][vec];
+  if (!f64) return jacc_tab_27_32_lib[row][vec];
+  return (p.fpath == JACC_FP_W32 ? jacc_tab_27_64_lib_w32 : jacc_tab_27_64_lib)[row][vec];
+}
+
+// The default tile: 32 x 4 threads, 16-byte columns where nx allows.  2D: they
+// pay from 2^18 points on (4096^2 FP64: 50.0 us a sweep, 62.5 with scalar
+// columns); below, more, narrower strips hide latency better (300^2: 2.04 us).
+// 3D: the long march where it yields at least 1024 CTAs.
 int default_tile(const jacc_kernel_desc& d) {
   const int V = d.dtype == 64 ? 2 : 4;
   const bool vec_ok = (d.nx % V) == 0;
-  if (d.stencil == 5) {
-    if (d.nx * d.ny < (int64_t(1) << 19)) return 8;
-    return vec_ok ? 17 : 16;
-  }
+  if (d.stencil == 5) return vec_ok && d.nx * d.ny >= (int64_t(1) << 18) ? 3 : 2;
   const int64_t w = 32 * (vec_ok ? V : 1);  // columns of a 32 x 4 tile
   const int64_t ctas_long = ((d.nx + w - 1) / w) * ((d.ny + 7) / 8) * ((d.nz + 63) / 64);
   if (ctas_long >= 1024) return vec_ok ? 3 : 2;
   return vec_ok ? 1 : 0;
 }
 
-bool staged_tile(const jacc_kernel_desc& d, int t) {
-  return kTiles[t].vec16 && (d.stencil == 7 || (d.stencil == 27 && d.dtype == 32));
+// The kernel family of the library's own choice.  7-point grids that live in
+// L2 need no staging (us a sweep without / with the ring: FP32 64^3 1.8 / 3.3,
+// 128^3 4.2 / 4.9, 160^3 9.9 / 10.4, 216^3 18.0 / 16.0; FP64 64^3 3.1 / 5.4,
+// 128^3 9.9 / 10.4, 160^3 20.9 / 19.5; scalar columns FP32 81^3 3.7 / 4.1,
+// 97^3 5.5 / 4.8, FP64 97^3 8.8 / 9.1, 129^3 16.9 / 12.8).  Folded kernels of
+// fields that stream from HBM stage by bulk copies (bulk / ring: 7-point FP64
+// 512^3 361 / 398, 320^3 98 / 95; FP32 512^3 164 / 189, 400^3 92 / 92; 27-point
+// FP32 768^3 577 / 610, 512^3 195 / 179), of the precompiled ones only the FP32
+// 7-point kernel (512^3 164 / 170); the rest asynchronous copies (precompiled,
+// ring / bulk: 7-point FP64 512^3 396 / 480, 27-point FP32 768^3 604 / 748).
+static int default_family(const jacc_kernel_desc& d, int tile) {
+  if (d.tblock > 1 || d.stencil == 19) return JACC_FAM_TABLE;
+  if (d.stencil == 5) return JACC_FAM_STRIP;
+  const bool vec = kTiles[tile].vec16, f64 = d.dtype == 64;
+  const int64_t n = d.nx * d.ny * d.nz;
+  if (d.stencil == 7) {
+    const int64_t direct = vec ? (f64 ? int64_t(1) << 21 : int64_t(1) << 22) : (f64 ? int64_t(1) << 20 : int64_t(5) << 17);
+    if (n <= direct) return JACC_FAM_DIRECT;
+  }
+  const bool bulk = d.stencil == 7 ? n * (f64 ? 8 : 4) >= (int64_t(1) << 28) : !f64 && n * 4 >= (int64_t(1) << 30);
+  const bool pays = (d.flags & JACC_SPEC_JIT) || (d.stencil == 7 && !f64);
+  return tile == 3 && bulk && pays ? JACC_FAM_BULK : JACC_FAM_RING;
 }
 
-// Tiles whose planes are staged by asynchronous copies, one column of
-// JACC_RING_ROWS rows per thread.
-static bool ring_tile(const jacc_kernel_desc& d, int t) {
-  return !kTiles[t].vec16 ? d.stencil == 7 || d.stencil == 27 : d.stencil == 27 && d.dtype == 64;
+// What a CTA of kernel family `fam` covers per plane (columns, rows), and how
+// many planes (3D) or rows per thread row (2D) it marches.
+struct CtaTile {
+  int64_t cols, rows, march;
+};
+static CtaTile cta_tile(const jacc_kernel_desc& d, int tile, int fam, bool edge, int zc) {
+  const TileCfg& c = kTiles[tile];
+  const int V = c.vec16 ? (d.dtype == 64 ? 2 : 4) : 1;
+  if (d.stencil == 5)
+    return fam == JACC_FAM_STRIP || V == 1 ? CtaTile{static_cast<int64_t>(c.bx / 32) * 30 * V, c.by, zc}
+                                 : CtaTile{static_cast<int64_t>(c.bx) * V, c.by, zc};
+  const bool f64 = d.dtype == 64;
+  if (d.stencil == 7 && !edge && (fam == JACC_FAM_DIRECT || (fam == JACC_FAM_TABLE && JACC_DIRECT_TILE(c.bx, c.by, V))))
+    return CtaTile{static_cast<int64_t>(32) * V, 8, JACC_DIRECT_PLANES};
+  // one column of JACC_RING_ROWS rows per thread
+  if ((d.stencil == 27 && f64) || (V == 1 && (f64 || fam == JACC_FAM_RING))) return CtaTile{c.bx, c.by * JACC_RING_ROWS(c.bx, c.by), zc};
+  if (V == 1) return CtaTile{c.bx, c.by, zc};               // FP32 table tiles of scalar columns
+  return CtaTile{static_cast<int64_t>(c.bx) * V, c.by * 2, zc};  // a 16-byte column of two rows
+}
+static dim3 cta_grid(const jacc_kernel_desc& d, const CtaTile& t) {
+  auto up = [](int64_t a, int64_t b) { return static_cast<unsigned>((a + b - 1) / b); };
+  if (d.stencil == 5) return dim3(up(d.nx, t.cols), up(d.ny, t.rows * t.march), 1);
+  return dim3(up(d.nx, t.cols), up(d.ny, t.rows), up(d.nz, t.march));
 }
 
 bool tile_valid(const jacc_kernel_desc& d, int t) {
@@ -233,10 +281,10 @@ static std::string key_of(const jacc_kernel_desc& d, int tile, bool fit) {
   return std::string(reinterpret_cast<const char*>(&c), sizeof(c)) + (fit ? "f" : "t");
 }
 
-// Planes per CTA of a 3D kernel whose tile the library chose itself: at most
+// Planes per CTA (3D) or rows per warp (2D) of a kernel whose tile the library
+// chose itself.  3D: at most
 // the tile's own, and few enough that the grid has at least 2.5 times the
-// CTAs that the device holds at once (no fewer than 8 planes: the two halo
-// planes of a chunk are read again).  With fewer, the last wave leaves SMs
+// CTAs that the device holds at once.  With fewer, the last wave leaves SMs
 // idle: 301 x 253 x 199 FP64 at 64 planes (640 CTAs on 152 SMs) 65.2 us a
 // sweep, at 16 planes (2080) 55.7, at 8 (4000) 57.3; 511^3, whose grid is
 // large either way, within 3 % from 8 to 64.
@@ -249,38 +297,58 @@ static int fitted_chunk(const Kernel& k, int zc) {
     cudaGetLastError();
     return zc;
   }
-  const int64_t columns = static_cast<int64_t>(k.grid.x) * k.grid.y;
-  const int64_t want = (5ll * nsm * (per > 0 ? per : 1) / 2 + columns - 1) / columns;  // chunks
+  const int64_t slots = static_cast<int64_t>(nsm) * (per > 0 ? per : 1);
+  if (k.desc.stencil == 5) {
+    // rows per warp, 2 to the tile's own: a strip's start-up (three rows of
+    // loads before the first result) costs more than an unfilled wave, so 0.6
+    // of the slots are enough (1000^2 FP64: 4.42 us a sweep at 8 rows, 544
+    // CTAs; 4.87 at 4, 5.2 at 16)
+    const int64_t rows = 10ll * k.grid.x * k.desc.ny / (6ll * slots * k.block.y);
+    return static_cast<int>(rows >= zc ? zc : (rows < 2 ? 2 : rows));
+  }
+  const int64_t columns = static_cast<int64_t>(k.grid_out.x) * k.grid_out.y;
+  const int64_t want = (5 * slots / 2 + columns - 1) / columns;  // chunks
   const int64_t fit = (k.desc.nz + want - 1) / want;
-  return static_cast<int>(fit >= zc ? zc : (fit < 8 ? (zc < 8 ? zc : 8) : fit));
+  // no fewer than 4 planes, 8 for 27-point grids that are not small (their
+  // halo planes cost most: FP32 64^3 3.6 us a sweep at 4, 5.0 at 8; 128^3 7.5
+  // at 4, 7.0 at 8; FP64 96^3 7.3 and 8.6, 112^3 12.8 and 10.8)
+  const int64_t n = k.desc.nx * k.desc.ny * k.desc.nz;
+  const int least = k.desc.stencil == 7 || n <= (int64_t(1) << (k.desc.dtype == 64 ? 20 : 19)) ? 4 : 8;
+  return static_cast<int>(fit >= zc ? zc : (fit < least ? least : fit));
 }
 
-// Planes per CTA of a 3D kernel.  The constant-folded variants of the staged
-// tiles with the long march take fewer planes than the table's 64: with the
-// extents folded their kernels need fewer registers and more CTAs fit, and
-// shallower chunks then balance better.  Measured with tile 3: heat 512^3
-// FP64 best at 40 planes (396.8 against 392.1 GLUP/s at 64), 27-point 1024^3
-// FP32 best at 24-32 (128.6 ms for 100 sweeps at 32 against 144.7 at 64).
-// The precompiled kernels stay at 64.
-static int plane_chunk(const jacc_kernel_desc& d, int tile) {
+// Planes per CTA of a 3D kernel.  The constant-folded variants of the bulk-copy
+// staged tiles with the long march take fewer planes than the table's 64: with
+// the extents folded their kernels need fewer registers and more CTAs fit, and
+// shallower chunks then balance better.  Measured with tile 3: heat 512^3 FP64
+// best at 40 planes (396.8 against 392.1 GLUP/s at 64), 27-point 1024^3 FP32
+// best at 24-32 (128.6 ms for 100 sweeps at 32 against 144.7 at 64).  The
+// library's own 7-point kernels take at most 16 planes in FP32 (512^3, us a
+// sweep at 12 / 16 / 24 / 32 / 64 planes: ring 170 / 170 / 174 / 178 / 181,
+// bulk 162 / 164 / 164 / 166 / 184) and 24 in FP64 (ring 414 / 410 / 396 / 400 /
+// 403): the CTAs that share a halo row then stay closer together.
+static int plane_chunk(const jacc_kernel_desc& d, int tile, int fam) {
   const TileCfg& c = kTiles[tile];
-  if ((d.flags & JACC_SPEC_JIT) && d.stencil != 5 && staged_tile(d, tile) && c.zc == 64)
-    return d.stencil == 27 ? 32 : 40;
+  if (d.stencil == 5) return c.zc / 4;  // rows per warp
+  const bool f64 = d.dtype == 64;
+  if (d.stencil == 7 && !f64 && (fam == JACC_FAM_RING || fam == JACC_FAM_BULK)) return 16;
+  if (d.stencil == 7 && f64 && fam == JACC_FAM_RING) return c.zc < 24 ? c.zc : 24;
+  const bool bulk = c.vec16 && !(d.stencil == 27 && f64) && (fam == JACC_FAM_TABLE || fam == JACC_FAM_BULK);
+  if ((d.flags & JACC_SPEC_JIT) && bulk && c.zc == 64) return d.stencil == 27 ? 32 : 40;
   return c.zc;
 }
 
 // The NVRTC source of a folded variant: the device text plus a struct whose
-// static constexpr members replace JParams.
+// static constexpr members replace JParams, and the kernels: jacc_jit for the
+// intermediate (and every FP32 or native) sweeps, and for FP64 jacc_jit_out,
+// which converts FP64 on load and store, and jacc_jit_last, only on store.
 static std::string jit_source(const Kernel& k) {
   const JParams& p = k.params;
   const TileCfg& c = kTiles[k.tile];
-  char buf[4096];
-  const char* T = k.desc.dtype == 64 ? "double" : "float";
-  const char* entry = k.desc.stencil == 5 ? "jacobi2d_entry" : (k.desc.stencil == 7 ? "heat3d_entry" : "box27_entry");
-  // the 2D march length is a template argument, the 3D one a launch parameter
-  const std::string zc = k.desc.stencil == 5 ? std::to_string(c.zc / 4) + ", " : "";
-  const char* edge = k.desc.dtype == 64 ? "true" : "false";  // the converting sweeps' instantiation
-  std::snprintf(buf, sizeof(buf),
+  const int st = k.desc.stencil;
+  const std::string T = k.desc.dtype == 64 ? "double" : "float";
+  char fold[1024];
+  std::snprintf(fold, sizeof(fold),
                 "\nstruct JFold {\n"
                 "  static constexpr i64 nx = %lldll, ny = %lldll, nz = %lldll;\n"
                 "  static constexpr double c0 = %a, c1 = %a, c2 = %a, c3 = %a;\n"
@@ -288,34 +356,35 @@ static std::string jit_source(const Kernel& k) {
                 "  static constexpr i64 fb = %lldll;\n"
                 "  static constexpr i64 fw0 = %lldll, fw1 = %lldll, fw2 = %lldll, fw3 = %lldll;\n"
                 "  static constexpr int fk = %d, fpath = %d, zc = %d;\n"
-                "};\n"
-                "template <> struct JacobiPrefetch<JFold> { static constexpr bool value = %s; };\n"
-                "extern \"C\" __global__ void __launch_bounds__(%d, (SweepMinBlocks<%d, %s, %d, %d, %d, false, true>::value))\n"
-                "jacc_jit(const %s* __restrict__ u, "
-                "%s* __restrict__ v, JParams rt, double* resid, const u64* maxword, int flags) {\n"
-                "  const JFold f{};\n"
-                "  %s<%s, %d, %d, %d, %sfalse>(u, v, f, rt, resid, maxword, flags);\n"
-                "}\n"
-                "extern \"C\" __global__ void __launch_bounds__(%d, (SweepMinBlocks<%d, %s, %d, %d, %d, %s, true>::value))\n"
-                "jacc_jit_out(const %s* __restrict__ u, "
-                "%s* __restrict__ v, JParams rt, double* resid, const u64* maxword, int flags) {\n"
-                "  const JFold f{};\n"
-                "  %s<%s, %d, %d, %d, %s%s>(u, v, f, rt, resid, maxword, flags);\n"
-                "}\n"
-                "extern \"C\" __global__ void __launch_bounds__(%d, (SweepMinBlocksLast<%d, %s, %d, %d, %d>::value))\n"
-                "jacc_jit_last(const %s* __restrict__ u, "
-                "%s* __restrict__ v, JParams rt, double* resid, const u64* maxword, int flags) {\n"
-                "  const JFold f{};\n"
-                "  %s<%s, %d, %d, %d, %s%s>(u, v, f, rt, resid, maxword, JFX_OUT_F64);\n"
-                "}\n",
+                "};\n",
                 (long long)p.nx, (long long)p.ny, (long long)p.nz, p.c0, p.c1, p.c2, p.c3, (unsigned long long)p.fm,
-                (long long)p.fb, (long long)p.fw0, (long long)p.fw1, (long long)p.fw2, (long long)p.fw3, p.fk, p.fpath, p.zc,
-                // small (L2-resident) 2D grids: the prefetching march
-                (k.desc.stencil == 5 && k.desc.nx * k.desc.ny <= (int64_t(1) << 17)) ? "true" : "false",
-                c.bx * c.by, k.desc.stencil, T, c.bx, c.by, k.vec, T, T, entry, T, c.bx, c.by, k.vec, zc.c_str(), c.bx * c.by,
-                k.desc.stencil, T, c.bx, c.by, k.vec, edge, T, T, entry, T, c.bx, c.by, k.vec, zc.c_str(), edge, c.bx * c.by,
-                k.desc.stencil, T, c.bx, c.by, k.vec, T, T, entry, T, c.bx, c.by, k.vec, zc.c_str(), edge);
-  return std::string(device_source()) + buf;
+                (long long)p.fb, (long long)p.fw0, (long long)p.fw1, (long long)p.fw2, (long long)p.fw3, p.fk, p.fpath, p.zc);
+  // the kernel without staging has 32 x 8 threads, the converting sweeps the tile's
+  auto shape = [&](int fam, bool edge) {
+    const bool direct = fam == JACC_FAM_DIRECT && !edge;
+    return T + ", " + std::to_string(direct ? 32 : c.bx) + ", " + std::to_string(direct ? 8 : c.by) + ", " + std::to_string(k.vec);
+  };
+  auto tail = [&](int fam, bool edge) { return ", " + std::to_string(fam) + (edge ? ", true" : ", false"); };
+  auto call = [&](int fam, bool edge, const char* flags) {
+    return std::string(st == 5 ? "jacobi2d_entry<" : st == 7 ? "heat3d_entry<" : "box27_entry<") + shape(fam, edge) +
+           tail(fam, edge) + ">(u, v, f, rt, resid, maxword, " + flags + ")";
+  };
+  auto kernel = [&](const char* name, int threads, const std::string& bound, const std::string& body) {
+    return "extern \"C\" __global__ void __launch_bounds__(" + std::to_string(threads) + bound + ")\n" + name + "(const " + T +
+           "* __restrict__ u, " + T + "* __restrict__ v, JParams rt, double* resid, const u64* maxword, int flags) {\n" +
+           "  const JFold f{};\n  " + body + ";\n}\n";
+  };
+  auto bound = [&](int fam, bool edge) {
+    if (st == 5) return std::string();
+    return ", (SweepMinBlocks<" + std::to_string(st) + ", " + shape(fam, edge) + tail(fam, edge) + ", true>::value)";
+  };
+  std::string src = std::string(device_source()) + fold;
+  src += kernel("jacc_jit", k.fam == JACC_FAM_DIRECT ? 256 : c.bx * c.by, bound(k.fam, false), call(k.fam, false, "flags"));
+  if (k.desc.dtype == 64) {
+    src += kernel("jacc_jit_out", c.bx * c.by, bound(k.fam, true), call(k.fam, true, "flags"));
+    src += kernel("jacc_jit_last", c.bx * c.by, bound(k.fam, true), call(k.fam, true, "JFX_OUT_F64"));
+  }
+  return src;
 }
 
 static void free_kernel(Kernel* k) {
@@ -355,14 +424,14 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   jacc_status st = validate(*desc);
   if (st) return st;
   int tile = desc->tile_id;
-  bool fit = false;  // the library picks the planes per CTA along with the tile
+  bool fit = false;  // the library picks the kernel family and the march along with the tile
   if (desc->stencil == 19) {
     tile = 3;  // the kernel's one configuration: 32 x 4 threads, 16-byte columns, 40-plane march
   } else if (tile < 0) {
     tile = tuned_tile(*desc);
     if (tile < 0 || !tile_valid(*desc, tile)) {
       tile = default_tile(*desc);
-      fit = (desc->stencil == 7 || desc->stencil == 27) && desc->tblock <= 1;
+      fit = desc->stencil != 19 && desc->tblock <= 1;
     }
   }
   if (!tile_valid(*desc, tile))
@@ -392,26 +461,30 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   p.c2 = desc->coeffs[2];
   p.c3 = desc->coeffs[3];
   plan_fixed(*desc, p);
-  k->block = dim3(c.bx, c.by, 1);
-  const bool ring = ring_tile(*desc, tile);
-  const int64_t tx = static_cast<int64_t>(c.bx) * (ring ? 1 : k->vec);
-  p.zc = plane_chunk(*desc, tile);
-  if (desc->stencil == 5) {
-    const int64_t ty = static_cast<int64_t>(c.by) * (c.zc / 4);
-    k->grid = dim3(static_cast<unsigned>((desc->nx + tx - 1) / tx), static_cast<unsigned>((desc->ny + ty - 1) / ty), 1);
-  } else {
-    // the staged kernels (16-byte columns: 7-point, and 27-point FP32) give each thread 2 rows
-    const int64_t ty = static_cast<int64_t>(c.by) *
-                       (ring ? JACC_RING_ROWS(c.bx, c.by) : (staged_tile(*desc, tile) ? 2 : 1));
-    const int64_t zc = p.zc;
-    k->grid = dim3(static_cast<unsigned>((desc->nx + tx - 1) / tx), static_cast<unsigned>((desc->ny + ty - 1) / ty),
-                   static_cast<unsigned>((desc->nz + zc - 1) / zc));
+  k->fam = fit ? default_family(*desc, tile) : JACC_FAM_TABLE;
+  const int fam = k->fam;
+  k->block_out = dim3(c.bx, c.by, 1);
+  k->block = fam == JACC_FAM_DIRECT ? dim3(32, 8, 1) : k->block_out;
+  if (!(desc->flags & JACC_SPEC_JIT) && desc->stencil != 19 && desc->tblock <= 1) {
+    k->func = fam == JACC_FAM_TABLE || fam == JACC_FAM_BULK ? table_entry(desc->stencil, desc->dtype, tile, false)
+                                                            : lib_entry(*desc, p, fam, k->vec > 1);
+    if (fam == JACC_FAM_TABLE && p.fpath == JACC_FP_W32) k->func = jacc_tab_27_64_w32[tile];
+    k->func_out = desc->dtype == 32 ? k->func
+                  : fam == JACC_FAM_STRIP ? lib_entry(*desc, p, 5, k->vec > 1)
+                                          : table_entry(desc->stencil, desc->dtype, tile, true);
+    if (!k->func || !k->func_out) return fail(JACC_ERR_UNSUPPORTED, "no precompiled kernel for this descriptor");
   }
+  // FP64 sequences convert in their first and last sweeps, which have a kernel of their own
+  const bool edge = desc->dtype == 64;
+  p.zc = plane_chunk(*desc, tile, fam);
+  k->grid = k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, p.zc));
   if (fit) {
-    if (!(desc->flags & JACC_SPEC_JIT)) k->func = table_entry(desc->stencil, desc->dtype, tile, false);
     p.zc = fitted_chunk(*k, p.zc);
-    k->grid.z = static_cast<unsigned>((desc->nz + p.zc - 1) / p.zc);
+    if (desc->stencil == 5)
+      while ((desc->ny + c.by * p.zc - 1) / (c.by * p.zc) > 65535) p.zc *= 2;  // the grid's limit
   }
+  k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, p.zc));
+  k->grid = cta_grid(*desc, cta_tile(*desc, tile, fam, false, p.zc));
   if (desc->stencil == 19) {
     var19_geometry(desc->nx, desc->ny, desc->nz, &k->grid, &k->block);
     k->func = k->func_out = nullptr;  // launched by jacc_sweep_coeffs only
@@ -439,18 +512,16 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   } else if (desc->flags & JACC_SPEC_JIT) {
     static const char* const names[3] = {"jacc_jit", "jacc_jit_out", "jacc_jit_last"};
     const void* f[3] = {nullptr, nullptr, nullptr};
-    st = jit_compile(jit_source(*k), names, 3, &k->lib, f, &k->compile_ms);
+    st = jit_compile(jit_source(*k), names, desc->dtype == 64 ? 3 : 1, &k->lib, f, &k->compile_ms);
     if (st) return st;
     k->func = f[0];
-    k->func_out = f[1];
-    // the store-only converting kernel: FP64 fixed-point sequences only
-    if (desc->dtype == 64) k->func_last = f[2];
+    k->func_out = desc->dtype == 64 ? f[1] : f[0];
+    k->func_last = f[2];  // FP64 only
     k->jit = true;
-  } else {
-    k->func = table_entry(desc->stencil, desc->dtype, tile, false);
-    if (p.fpath == JACC_FP_W32) k->func = jacc_tab_27_64_w32[tile];
-    k->func_out = table_entry(desc->stencil, desc->dtype, tile, true);
-    if (!k->func || !k->func_out) return fail(JACC_ERR_UNSUPPORTED, "no precompiled kernel for this descriptor");
+  }
+  if (!edge) {
+    k->grid_out = k->grid;
+    k->block_out = k->block;
   }
   if (desc->flags & JACC_SPEC_CLUSTER) {
     int nc = 0;
@@ -552,15 +623,17 @@ extern "C" jacc_status jacc_shutdown(void) {
 namespace jacc {
 
 cudaError_t launch_sweep_kernel(const Kernel& k, const void* u, void* v, double* resid, const u64* maxword, int flags,
-                                cudaStream_t s) {
+                                cudaStream_t s, const int* stop) {
   JParams p = k.params;
+  p.stop = stop;
   const void* args[] = {&u, &v, &p, &resid, &maxword, &flags};
   // programmatic dependent launch: the kernel may start while the previous
   // sweep finishes; every sweep kernel waits (griddepcontrol.wait) for the
   // previous grid before it touches a field
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = k.grid;
-  cfg.blockDim = k.block;
+  const bool edge = (flags & (kFxIn | kFxOut)) != 0;
+  cfg.gridDim = edge ? k.grid_out : k.grid;
+  cfg.blockDim = edge ? k.block_out : k.block;
   cfg.dynamicSmemBytes = static_cast<size_t>(k.smem);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -568,7 +641,7 @@ cudaError_t launch_sweep_kernel(const Kernel& k, const void* u, void* v, double*
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const void* f = flags == kFxOut && k.func_last ? k.func_last : ((flags & (kFxIn | kFxOut)) ? k.func_out : k.func);
+  const void* f = flags == kFxOut && k.func_last ? k.func_last : (edge ? k.func_out : k.func);
   return cudaLaunchKernelExC(&cfg, f, const_cast<void**>(args));
 }
 

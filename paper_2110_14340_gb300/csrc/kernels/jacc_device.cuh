@@ -44,30 +44,32 @@ JD int fx_frac_bits(u64 maxbits) {
   return 1079 - eb;  // M < 2^(eb-1022)  =>  |q| < 2^57
 }
 
-// x * 2^F truncated toward zero; |x| <= M guarantees the shift is <= 4.
+// x * 2^F truncated toward zero.  |x| <= M means the value is below 2^57, so
+// it is the 53-bit significand in the top of a 57-bit field shifted right by
+// the exponent's distance from M's; zero and subnormals are 64 or more away
+// and shift to nothing.
 JD i64 fx_from(double x, int F) {
-  u64 b = (u64)__double_as_longlong(x);
-  int eb = (int)((b >> 52) & 0x7ffull);
-  u64 m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  int sh = eb - 1075 + F;
-  u64 r = (sh >= 0) ? (m << sh) : ((sh > -64) ? (m >> (-sh)) : 0ull);
-  r = (eb == 0) ? 0ull : r;
-  return (b >> 63) ? -(i64)r : (i64)r;
+  const u64 b = (u64)__double_as_longlong(x);
+  const int hi = (int)(b >> 32);
+  const int d = 1079 - F - ((hi >> 20) & 0x7ff);
+  const u64 m = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 4;
+  const i64 r = (i64)(m >> (d < 63 ? d : 63));
+  const i64 s = (i64)(hi >> 31);
+  return (r ^ s) - s;
 }
 
-// q * 2^-E rounded to nearest even.  A carry out of the 53-bit mantissa
-// propagates into the exponent field by construction.
+// q * 2^-E rounded to nearest even, |q| < 2^62.  The magnitude is shifted to
+// bit 62; adding just under half of the last place plus the last bit rounds
+// half to even, and a carry out of the 53-bit significand propagates into the
+// exponent field by construction.
 JD double fx_to(i64 q, int E) {
-  u64 s = (u64)q >> 63;
-  u64 a = s ? (u64)(-q) : (u64)q;
-  int lz = __clzll((i64)a);
-  u64 n = a << (lz & 63);
-  u64 mant = n >> 11;
-  u64 rem = n & 0x7ffull;
-  mant += (u64)((rem > 0x400ull) | ((rem == 0x400ull) & (mant & 1ull)));
-  i64 eb = 63 - lz - E + 1023;
-  u64 bits = (s << 63) | (((u64)(eb - 1) << 52) + mant);
-  return a ? __longlong_as_double((i64)bits) : 0.0;
+  const i64 s = q >> 63;
+  const u64 a = (u64)((q ^ s) - s);
+  const int lz = __clzll((i64)a);
+  const u64 n = a << ((lz - 1) & 63);
+  const u64 mant = (n + 0x1ffull + ((n >> 10) & 1ull)) >> 10;
+  const u64 bits = mant + ((u64)(u32)((63 - lz - E + 1022) << 20) << 32);
+  return a ? __longlong_as_double((i64)(bits | ((u64)s & 0x8000000000000000ull))) : 0.0;
 }
 
 // Unsigned magnitude version (for residual maxima).
@@ -723,6 +725,79 @@ JD void bulk_g2s(void* dst, const void* src, u32 bytes, u64* bar) {
                : "memory");
 }
 
+// ---------------------------------------------------------------- planes staged by asynchronous copies
+//
+// A second way of staging planes, for the kernels whose rows need not start
+// on 16-byte boundaries or whose staged values are converted in place: every
+// thread copies its share of a plane (the tile with a one-point halo) with
+// cp.async, CH elements per copy, into a ring of S stages in shared memory;
+// one group per plane, one CTA barrier per plane.  A copy's source may be any
+// element (8- or 4-byte copies for CH = 1), so odd rows, periodic images and
+// clipped edges all come from a per-thread list of source offsets worked out
+// once, and the thread that copied an element may convert it before the
+// barrier that publishes the plane.
+//
+// Geometry: BX x BY threads; a thread owns V consecutive columns of RY
+// consecutive rows: one column, so a warp reads and writes whole rows (no bank
+// conflicts, coalesced stores at any alignment), or one 16-byte column of two
+// rows.  The y neighbours inside its rows stay in registers.  A stage holds
+// R x W elements in rows of W = BX V + 2 CH: column x of the tile sits at slot
+// x - bx0 + CH of row y - by0 + 1.
+template <class T, int BX, int BY, int CH, int V = 1> struct RingG {
+  static constexpr int NT = BX * BY;
+  static constexpr int RY = V > 1 ? 2 : JACC_RING_ROWS(BX, BY);
+  static constexpr int TW = BX * V, TH = BY * RY;
+  static constexpr int W = TW + 2 * CH, R = TH + 2;
+  static constexpr int STAGE = W * R;                       // elements
+  static constexpr int NCH = W / CH, NTOT = NCH * R;        // copies per row, per plane
+  static constexpr int PER = (NTOT + NT - 1) / NT;          // copies per thread
+  static constexpr int S0 = 46080 / (STAGE * (int)sizeof(T));
+  static constexpr int S = S0 < 3 ? 3 : (S0 > 6 ? 6 : S0);  // stages, at most 45 KB
+};
+
+template <int BYTES> JD void cpa_copy(void* dst, const void* src) {
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES) : "memory");
+}
+JD void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> JD void cpa_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// A thread's share of every staged plane: copy i moves the CH elements at
+// offset off[i] of the plane to stage element (tid + i NT) CH; bit i of
+// `mask` is clear where there is none (past the plane, or outside a Dirichlet
+// grid, whose slots are never used).
+template <class T, int BX, int BY, int CH, int V = 1> struct RingPlan {
+  typedef RingG<T, BX, BY, CH, V> G;
+  i64 off[G::PER];
+  u32 mask;
+  JD void init(i64 nx, i64 ny, i64 bx0, i64 by0, bool periodic) {
+    const int tid = threadIdx.y * BX + threadIdx.x;
+    mask = 0;
+#pragma unroll
+    for (int i = 0; i < G::PER; ++i) {
+      const int c = tid + i * G::NT;
+      i64 x = bx0 - CH + (c % G::NCH) * CH, y = by0 - 1 + c / G::NCH;
+      bool ok = c < G::NTOT;
+      if (periodic) {
+        x = (x + nx) % nx;
+        y = (y + ny) % ny;
+      } else {
+        ok = ok && x >= 0 && x < nx && y >= 0 && y < ny;
+      }
+      off[i] = ok ? y * nx + x : 0;
+      mask |= (u32)ok << i;
+    }
+  }
+  JD void issue(T* stage, const T* plane) const {
+    const int tid = threadIdx.y * BX + threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < G::PER; ++i)
+      if ((mask >> i) & 1u) cpa_copy<CH * (int)sizeof(T)>(stage + (tid + i * G::NT) * CH, plane + off[i]);
+  }
+};
+
 // Geometry of the staged 27-point FP32 kernel: BX x BY threads, each owning 4
 // consecutive columns (one 16-byte vector) of 2 consecutive rows, so a CTA
 // computes a TW x TH tile per plane.  A stage holds R = TH + 2 rows of
@@ -746,24 +821,26 @@ template <int BX, int BY> struct alignas(128) Box27SSmem {
   u64 empty[Box27S<BX, BY>::S];
 };
 
-// Warp 0 requests staged plane zg into stage s: lane 0 posts the byte count,
-// then lane r copies staged row r as one bulk copy, or as two or more where
-// the row's slots wrap around the periodic x boundary.
-template <int BX, int BY, class P>
-JD void box27s_issue(Box27SSmem<BX, BY>& sm, int s, const float* __restrict__ u, const P& p, i64 zg, i64 bx0, i64 by0,
-                     int weff) {
+// What lane r of warp 0 copies of every staged plane: staged row r, as one bulk
+// copy, or as two or more where the row's slots wrap around the periodic x
+// boundary.  Worked out once: the wraps are divisions.
+struct Box27Row {
+  i64 row;  // offset of the row in its plane
+  i64 c;    // first column
+};
+
+// Warp 0 requests a plane into stage s: lane 0 posts the byte count, then each
+// lane copies its row.
+template <int BX, int BY>
+JD void box27s_issue(Box27SSmem<BX, BY>& sm, int s, const float* __restrict__ plane, const Box27Row& q, i64 nx, int weff) {
   typedef Box27S<BX, BY> G;
-  const i64 nx = p.nx, ny = p.ny;
   const int lane = threadIdx.x & 31;
   if (lane == 0) mbar_expect_tx(&sm.full[s], (u32)(G::R * weff * 4));
   __syncwarp();
-  for (int r = lane; r < G::R; r += 32) {
-    i64 yg = (by0 - 1 + r) % ny;
-    if (yg < 0) yg += ny;
-    const float* row = u + (zg * ny + yg) * nx;
-    float* dst = &sm.st[s][r][0];
-    i64 c = bx0 - 4;
-    if (c < 0) c += nx;
+  if (lane < G::R) {
+    const float* row = plane + q.row;
+    float* dst = &sm.st[s][lane][0];
+    i64 c = q.c;
     int i = 0;
     while (i < weff) {
       i64 len = nx - c;
@@ -809,11 +886,15 @@ JD void box27s_terms(const float (*st)[Box27S<BX, BY>::W], float w0, float wf, f
 // z1 are staged (L = z1 - z0 + 2), output plane z = A(z-1) + B(z) + A(z+1)
 // is formed as P + A(z+1) with P = A(z-1) + B(z) kept in registers.  Returns
 // the thread's double-float sum of its outputs (want_sum).
-template <int BX, int BY, class P>
+template <int BX, int BY, bool BULK, class P>
 JD double box27s_body(const float* __restrict__ u, float* __restrict__ v, const P& p, const JParams& rt,
                       bool want_sum) {
   typedef Box27S<BX, BY> G;
-  __shared__ Box27SSmem<BX, BY> sm;
+  typedef RingG<float, BX, BY, 4, 4> R;  // the same stage layout
+  static_assert(R::W == G::W && R::R == G::R, "one stage layout for both ways of staging");
+  __shared__ __align__(128) unsigned char raw[BULK ? sizeof(Box27SSmem<BX, BY>) : sizeof(float) * R::S * R::STAGE];
+  Box27SSmem<BX, BY>& sm = *reinterpret_cast<Box27SSmem<BX, BY>*>(raw);  // BULK
+  float* ring = reinterpret_cast<float*>(raw);                           // otherwise
   const i64 nx = p.nx, ny = p.ny, nz = p.nz, sz = nx * ny;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int tid = ty * BX + tx;
@@ -825,25 +906,44 @@ JD double box27s_body(const float* __restrict__ u, float* __restrict__ v, const 
   const int weff = (int)((nx - bx0 < G::TW) ? nx - bx0 : G::TW) + 8;
   const i64 lim = rt.timeout_ns;
   const bool stall_cta = rt.stall_plane >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
-  if (tid == 0) {
+  if constexpr (BULK) {
+    if (tid == 0) {
 #pragma unroll
-    for (int s = 0; s < G::S; ++s) {
-      mbar_init(&sm.full[s], 1);
-      mbar_init(&sm.empty[s], G::NW);
+      for (int s = 0; s < G::S; ++s) {
+        mbar_init(&sm.full[s], 1);
+        mbar_init(&sm.empty[s], G::NW);
+      }
+      mbar_init_fence();
     }
-    mbar_init_fence();
+    __syncthreads();
   }
-  __syncthreads();
-  auto plane_z = [&](int j) {
-    i64 z = (z0 - 1 + j) % nz;
-    return z < 0 ? z + nz : z;
-  };
+  static_assert(G::R <= 32, "one staged row per lane of warp 0");
+  Box27Row lrow;
+  lrow.row = ((by0 - 1 + (tid & 31) + ny) % ny) * nx;
+  lrow.c = bx0 >= 4 ? bx0 - 4 : bx0 - 4 + nx;
+  i64 zi = z0 == 0 ? nz - 1 : z0 - 1;  // the next plane to request
   auto request = [&](int j, int s) {
-    if (!(stall_cta && j == rt.stall_plane)) box27s_issue<BX, BY>(sm, s, u, p, plane_z(j), bx0, by0, weff);
+    if (!(stall_cta && j == rt.stall_plane)) box27s_issue<BX, BY>(sm, s, u + zi * sz, lrow, nx, weff);
+    zi = zi + 1 == nz ? 0 : zi + 1;
   };
   int issued = 0, consumed = 0;  // warp 0: planes requested, planes waited for
-  if (warp0)
-    for (; issued < G::S && issued < L; ++issued) request(issued, issued);
+  RingPlan<float, BX, BY, 4, 4> plan;
+  int is = 0, cs = 0;  // asynchronous copies: stages to fill and to read, in elements
+  auto copy_next = [&]() {
+    if (issued < L) plan.issue(ring + is, u + zi * sz);
+    cpa_commit();
+    ++issued;
+    zi = zi + 1 == nz ? 0 : zi + 1;
+    is = is + R::STAGE == R::S * R::STAGE ? 0 : is + R::STAGE;
+  };
+  if constexpr (BULK) {
+    if (warp0)
+      for (; issued < G::S && issued < L; ++issued) request(issued, issued);
+  } else {
+    plan.init(nx, ny, bx0, by0, true);
+#pragma unroll 1
+    for (int j = 0; j < R::S - 1; ++j) copy_next();
+  }
 
   const float w0 = (float)p.c0, wf = (float)p.c1, we = (float)p.c2, wc = (float)p.c3;
   const i64 x0 = bx0 + 4 * tx, y0 = by0 + 2 * ty;
@@ -863,6 +963,14 @@ JD double box27s_body(const float* __restrict__ u, float* __restrict__ v, const 
   // consume plane j: wait for it, form its terms, release its stage, and let
   // warp 0 refill the stage of plane j - 1
   auto consume = [&](int j, float (&A)[2][4], float (&B)[2][4]) -> bool {
+    if constexpr (!BULK) {
+      cpa_wait<R::S - 2>();
+      __syncthreads();
+      copy_next();  // into the stage read before the barrier
+      box27s_terms<BX, BY>(reinterpret_cast<const float(*)[G::W]>(ring + cs), w0, wf, we, wc, A, B);
+      cs = cs + R::STAGE == R::S * R::STAGE ? 0 : cs + R::STAGE;
+      return true;
+    }
     if (!mbar_wait(&sm.full[cn_s], cn_ph, lim)) return false;
     ++consumed;
     box27s_terms<BX, BY>(sm.st[cn_s], w0, wf, we, wc, A, B);
@@ -1172,150 +1280,6 @@ JD void jacobi_fx_march(const double* __restrict__ u, double* __restrict__ v, i6
   }
 }
 
-// ---------------------------------------------------------------- 5-point Jacobi, prefetching march
-//
-// The march of jacobi_march / jacobi_fx_march with loads issued PD rows
-// ahead: a register ring holds the raw rows y+2 .. y+PD+1 in flight, and the
-// x-edge values of lanes 0 and 31 (one column left of the warp's chunk for
-// lane 0, one right for lane 31) for rows y+1 .. y+PD-1, so no load is
-// consumed in the iteration that issues it.  The ring is indexed with
-// compile-time slots (the row loop is unrolled by PD).  Rows past ye (the
-// march end) are not prefetched beyond the one halo row the last step needs.
-// FX: resident 64-bit fixed point (EDGE as for jacobi_fx_march); otherwise
-// native arithmetic on T.
-template <class T, int V, bool CG, bool FX, bool EDGE, int PD>
-JD void jacobi_march_pf(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 ny, i64 x0, i64 ys, i64 ye, int F,
-                        int flags, typename RT<T, FX ? JM_FIXED : JM_NATIVE>::type& rmax) {
-  typedef typename WT<T, FX ? JM_FIXED : JM_NATIVE>::type W;
-  const int lane = threadIdx.x & 31;
-  const bool xin = x0 < nx;
-  const bool inf = FX && EDGE && (flags & JFX_IN_F64);
-  const bool outf = FX && EDGE && (flags & JFX_OUT_F64);
-  // this lane's x-edge column (lane 0: x0 - 1, lane 31: x0 + V), if any
-  const bool has_edge = xin && ((lane == 0 && x0 >= 1) || (lane == 31 && x0 + V < nx));
-  const T* ecol = u + (lane == 0 ? x0 - 1 : x0 + V);
-  const T* col = u + x0;
-  auto cvt = [&](T raw) -> W {
-    if constexpr (FX) return inf ? fx_from(raw, F) : bits_i64(raw);
-    else return raw;
-  };
-  auto bnd_out = [&](T raw, W w) -> T {
-    if constexpr (FX) {
-      if constexpr (!EDGE) return i64_bits(w);
-      if (inf && outf) return raw;
-      if (outf) return fx_to(w, F);
-      return i64_bits(w);
-    } else {
-      return raw;
-    }
-  };
-  unsigned intm, bndm;
-  col_masks<V>(x0, nx, intm, bndm);
-  T ring[PD][V];  // slot j % PD: raw row ys + 1 + j (the "down" row of step j)
-  T eg[PD];       // slot j % PD: this lane's x-edge value of row ys + j
-  T rcur[V];
-  W up[V], cur[V];
-  {
-    T t[V];
-#pragma unroll
-    for (int e = 0; e < V; ++e) t[e] = rcur[e] = T(0);
-    if (xin) {
-      if (ys >= 1) ldv<T, V, CG>(col + (ys - 1) * nx, t);
-      ldv<T, V, CG>(col + ys * nx, rcur);
-    }
-#pragma unroll
-    for (int e = 0; e < V; ++e) {
-      up[e] = cvt(t[e]);
-      cur[e] = cvt(rcur[e]);
-    }
-#pragma unroll
-    for (int k = 0; k < PD; ++k) {
-      const i64 r = ys + 1 + k;
-#pragma unroll
-      for (int e = 0; e < V; ++e) ring[k][e] = T(0);
-      if (xin && r <= ye && r < ny) ldv<T, V, CG>(col + r * nx, ring[k]);
-      eg[k] = T(0);
-      if (has_edge && ys + k < ye) eg[k] = ld1<CG>(ecol + (ys + k) * nx);
-    }
-  }
-  const i64 n = ye - ys;
-  for (i64 j0 = 0; j0 < n; j0 += PD) {
-#pragma unroll
-    for (int i = 0; i < PD; ++i) {
-      const i64 j = j0 + i;
-      if (j >= n) break;
-      const i64 y = ys + j;
-      // consume slot i: the down row and this lane's edge of row y; refill it
-      T rdn[V];
-#pragma unroll
-      for (int e = 0; e < V; ++e) rdn[e] = ring[i][e];
-      const T edge = eg[i];
-      {
-        const i64 r = y + 1 + PD;
-#pragma unroll
-        for (int e = 0; e < V; ++e) ring[i][e] = T(0);
-        if (xin && r <= ye && r < ny) ldv<T, V, CG>(col + r * nx, ring[i]);
-        if (has_edge && y + PD < ye) eg[i] = ld1<CG>(ecol + (y + PD) * nx);
-      }
-      W dn[V];
-#pragma unroll
-      for (int e = 0; e < V; ++e) dn[e] = cvt(rdn[e]);
-      W left = __shfl_up_sync(0xffffffffu, cur[V - 1], 1);
-      W right = __shfl_down_sync(0xffffffffu, cur[0], 1);
-      if (has_edge) {
-        if (lane == 0) left = cvt(edge);
-        else right = cvt(edge);
-      }
-      const bool yint = (y >= 1) && (y <= ny - 2);
-      T out[V];
-#pragma unroll
-      for (int e = 0; e < V; ++e) {
-        const W xl = (e == 0) ? left : cur[e - 1];
-        const W xr = (e == V - 1) ? right : cur[e + 1];
-        const bool in = yint && ((intm >> e) & 1u);
-        if constexpr (FX) {
-          const i64 s = (up[e] + dn[e]) + (xl + xr);
-          const T o = outf ? fx_to(s, F + 2) : i64_bits((s + 2) >> 2);
-          out[e] = in ? o : bnd_out(rcur[e], cur[e]);
-          const i64 d = s - cur[e] * 4;
-          const u64 ad = (u64)(d ^ (d >> 63));  // |d| (one less for negative d: below the tolerance by 2^-F)
-          rmax = (in && ad > rmax) ? ad : rmax;
-        } else {
-          const T s = (up[e] + dn[e]) + (xl + xr);
-          const T r = T(0.25) * s;
-          out[e] = in ? r : rcur[e];
-          T d = r - rcur[e];
-          d = d < T(0) ? -d : d;
-          rmax = (in && d > rmax) ? d : rmax;
-        }
-      }
-      if (xin) stv<T, V>(v + y * nx + x0, out);
-#pragma unroll
-      for (int e = 0; e < V; ++e) {
-        up[e] = cur[e];
-        cur[e] = dn[e];
-        rcur[e] = rdn[e];
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------- 7-point heat, resident fixed point
-//
-// S = the six faces, L = S - 6u (exact, scale F), r = m 2^-k:
-// v = u + round(m L 2^-k), the FP64 output u + r L correctly rounded, and
-// |v - u| is the magnitude of the increment.  An intermediate sweep converts
-// nothing: every value in both buffers, the Dirichlet boundary included, is
-// in fixed point.  The first and last sweeps of a sequence (EDGE, flags
-// JFX_IN_F64 / JFX_OUT_F64) convert loads and stores.
-//
-// The increment for any r: with fm = m 2^(62-k) < 2^60 (r <= 1/6) it is
-// floor((L fm + 2^61) / 2^62).  L + 2^62 is positive (|L| < 2^61), so the
-// 96-bit product of it takes four unsigned 32 x 32 -> 64-bit multiply-adds,
-// and the fm that the bias adds to the quotient is exact and comes off at the
-// end: 12 instructions for every r, in place of a 64 x 64 -> 128-bit product
-// and a 128-bit rounding shift.
-//
 // The residual maximum of N increments: |d| as d ^ (d >> 63) (one less if
 // negative).  Its high word is at least the running maximum's only if some
 // high word of d lies outside (~t, t), so a plane usually costs two 32-bit
@@ -1337,6 +1301,144 @@ template <int N> JD void fx_residual(const i64 (&d)[N], u64& rmax) {
   }
 }
 
+// ---------------------------------------------------------------- 5-point Jacobi, strip march
+//
+// One warp marches rows [ys, ye) of a strip of 30 V columns, V per lane:
+// lanes 0 and 31 hold the columns left and right of the strip, so every x
+// neighbour comes from a shuffle, with no extra loads or selects, at the
+// price of 2/30 more loads and sums (L2 serves the shared columns).  Rows
+// y-1, y, y+1 stay in registers and the raw rows y+2 .. y+4 are in flight;
+// three rows per iteration rotate all of them without copies.  A warp whose
+// columns are all interior runs without selects.  4096^2 FP64, 50 sweeps:
+// 3.52 ms with the row march of the table's vector tiles (82 thread-
+// instructions a point, an edge column loaded where it is used), 2.57 here (58;
+// 5.2 TB/s), bound by integer issue and the latency of 24 warps an SM.
+//
+// xl: the lane's first column (may lie outside the grid).  FX: resident
+// 64-bit fixed point, v 2^F = (S + 2) >> 2 with S the four neighbours, the
+// FP64 output fx_to(S, F + 2), the residual |S - 4u| (EDGE: conversions, see
+// JFX_*); otherwise native arithmetic on T.  All lanes of a warp share ys, ye.
+template <class T, int V, bool FX, bool EDGE>
+JD void jacobi_strip(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 ny, i64 xl, i64 ys, i64 ye, int F,
+                     int flags, typename RT<T, FX ? JM_FIXED : JM_NATIVE>::type& rmax) {
+  typedef typename WT<T, FX ? JM_FIXED : JM_NATIVE>::type W;
+  const int lane = threadIdx.x & 31;
+  const bool inf = FX && EDGE && (flags & JFX_IN_F64);
+  const bool outf = FX && EDGE && (flags & JFX_OUT_F64);
+  const bool xin = xl >= 0 && xl < nx;
+  const bool wr = xin && lane >= 1 && lane <= 30;  // this lane writes its columns
+  bool cint[V];
+  bool all = true;
+#pragma unroll
+  for (int e = 0; e < V; ++e) {
+    cint[e] = xl + e >= 1 && xl + e <= nx - 2;
+    all = all && (cint[e] || lane == 0 || lane == 31);
+  }
+  const bool fast = __all_sync(0xffffffffu, all);
+  auto cvt = [&](T raw) -> W {
+    if constexpr (FX) return inf ? fx_from(raw, F) : bits_i64(raw);
+    else return raw;
+  };
+  const T* src = u + ys * nx + xl;  // row ys of the lane's columns
+  T* dst = v + ys * nx + xl;
+  const i64 rows = ye - ys;
+  // last row needed: ye, if it is in the grid
+  const i64 rlast = (ye < ny ? ye : ny - 1) - ys;
+  auto load = [&](i64 r, T (&q)[V]) {  // row ys + r
+#pragma unroll
+    for (int e = 0; e < V; ++e) q[e] = T(0);
+    if (xin && r <= rlast) ldv<T, V>(src + r * nx, q);
+  };
+  T q[3][V];
+  W w[3][V];
+  {
+    T t[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) t[e] = T(0);
+    if (xin && ys >= 1) ldv<T, V>(src - nx, t);
+    load(0, q[0]);
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+      w[0][e] = cvt(t[e]);
+      w[1][e] = cvt(q[0][e]);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) load(1 + k, q[k]);
+  }
+  auto step = [&](i64 j, const W (&up)[V], const W (&cur)[V], W (&dn)[V], T (&qn)[V]) {
+    const i64 y = ys + j;
+#pragma unroll
+    for (int e = 0; e < V; ++e) dn[e] = cvt(qn[e]);
+    load(j + 4, qn);
+    const W left = __shfl_up_sync(0xffffffffu, cur[V - 1], 1);
+    const W right = __shfl_down_sync(0xffffffffu, cur[0], 1);
+    T out[V];
+    W d[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+      const W a = e == 0 ? left : cur[e == 0 ? 0 : e - 1];
+      const W b = e == V - 1 ? right : cur[e == V - 1 ? e : e + 1];
+      const W sm = (up[e] + dn[e]) + (a + b);
+      if constexpr (FX) {
+        out[e] = (EDGE && outf) ? fx_to(sm, F + 2) : i64_bits((sm + 2) >> 2);
+        d[e] = sm - cur[e] * 4;
+      } else {
+        out[e] = T(0.25) * sm;
+        d[e] = out[e] - cur[e];
+      }
+    }
+    const bool yint = y >= 1 && y <= ny - 2;
+    if (!(fast && yint)) {
+#pragma unroll
+      for (int e = 0; e < V; ++e)
+        if (!(yint && cint[e])) {
+          d[e] = W(0);
+          if constexpr (FX) {
+            if (EDGE && outf) out[e] = inf ? (wr ? src[j * nx + e] : T(0)) : fx_to(cur[e], F);
+            else out[e] = i64_bits(cur[e]);
+          } else {
+            out[e] = cur[e];
+          }
+        }
+    }
+    if constexpr (FX) {
+      fx_residual<V>(d, rmax);
+    } else {
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        const T m = d[e] < T(0) ? -d[e] : d[e];
+        rmax = m > rmax ? m : rmax;
+      }
+    }
+    if (wr) stv<T, V>(dst + j * nx, out);
+  };
+  i64 j = 0;
+#pragma unroll 1
+  for (; j + 3 <= rows; j += 3) {
+    step(j, w[0], w[1], w[2], q[0]);
+    step(j + 1, w[1], w[2], w[0], q[1]);
+    step(j + 2, w[2], w[0], w[1], q[2]);
+  }
+  if (j < rows) step(j, w[0], w[1], w[2], q[0]);
+  if (j + 1 < rows) step(j + 1, w[1], w[2], w[0], q[1]);
+  if (lane == 0 || lane == 31) rmax = 0;  // their sums lack a neighbour
+}
+
+// ---------------------------------------------------------------- 7-point heat, resident fixed point
+//
+// S = the six faces, L = S - 6u (exact, scale F), r = m 2^-k:
+// v = u + round(m L 2^-k), the FP64 output u + r L correctly rounded, and
+// |v - u| is the magnitude of the increment.  An intermediate sweep converts
+// nothing: every value in both buffers, the Dirichlet boundary included, is
+// in fixed point.  The first and last sweeps of a sequence (EDGE, flags
+// JFX_IN_F64 / JFX_OUT_F64) convert loads and stores.
+//
+// The increment for any r: with fm = m 2^(62-k) < 2^60 (r <= 1/6) it is
+// floor((L fm + 2^61) / 2^62).  L + 2^62 is positive (|L| < 2^61), so the
+// 96-bit product of it takes four unsigned 32 x 32 -> 64-bit multiply-adds,
+// and the fm that the bias adds to the quotient is exact and comes off at the
+// end: 12 instructions for every r, in place of a 64 x 64 -> 128-bit product
+// and a 128-bit rounding shift.
 JD i64 heat_increment(i64 L, u64 fm) {
   const u64 b = (u64)L + (1ull << 62);
   const u32 bl = (u32)b, bh = (u32)(b >> 32), ml = (u32)fm, mh = (u32)(fm >> 32);
@@ -1358,8 +1460,8 @@ JD i64 heat_increment(i64 L, u64 fm) {
 // (rows y-1 and y+2, the columns left and right of its own) from the stage.
 // The boundary planes z = 0 and nz-1 are written from the staged values.
 //
-// FX: FP64 storage in the resident 64-bit fixed point (EDGE: the first/last
-// sweep converts on load/store); otherwise native arithmetic on T.
+// FX: FP64 storage in the resident 64-bit fixed point (intermediate sweeps
+// only: nothing is converted); otherwise native arithmetic on T.
 template <class T, int BX, int BY, int SC> struct Heat3S {
   static constexpr int V = 16 / (int)sizeof(T);
   static constexpr int RY = 2;
@@ -1385,25 +1487,6 @@ template <class T, int BX, int BY, int SC> struct alignas(128) Heat3SSmem {
   u64 empty[Heat3S<T, BX, BY, SC>::S];
 };
 
-// Warp 0 requests plane zg into stage s: one bulk copy per staged row inside
-// the grid; lane 0 first posts the byte count of the whole plane.
-template <class T, int BX, int BY, int SC, class P>
-JD void heat3s_issue(Heat3SSmem<T, BX, BY, SC>& sm, int s, const T* __restrict__ u, const P& p, i64 zg, i64 bx0,
-                     i64 by0) {
-  typedef Heat3S<T, BX, BY, SC> G;
-  const i64 nx = p.nx, ny = p.ny;
-  const int lane = threadIdx.x & 31;
-  const i64 c0 = bx0 - G::V < 0 ? 0 : bx0 - G::V;
-  const i64 c1 = bx0 + G::TW + G::V > nx ? nx : bx0 + G::TW + G::V;
-  const i64 r0 = by0 - 1 < 0 ? 0 : by0 - 1;
-  const i64 r1 = by0 + G::TH + 1 > ny ? ny : by0 + G::TH + 1;
-  const u32 row_bytes = (u32)((c1 - c0) * (i64)sizeof(T));
-  if (lane == 0) mbar_expect_tx(&sm.full[s], row_bytes * (u32)(r1 - r0));
-  __syncwarp();
-  for (i64 y = r0 + lane; y < r1; y += 32)
-    bulk_g2s(&sm.st[s][y - (by0 - 1)][c0 - (bx0 - G::V)], u + (zg * ny + y) * nx + c0, row_bytes, &sm.full[s]);
-}
-
 // 16-byte shared-memory vector reads (bit patterns kept).
 JD void lds_vec(const void* p, float (&r)[4]) {
   const float4 t = *reinterpret_cast<const float4*>(p);
@@ -1424,8 +1507,8 @@ template <class A> struct SameT<A, A> { static constexpr bool value = true; };
 template <class T, bool FX> struct HeatAcc { typedef T type; };
 template <> struct HeatAcc<double, true> { typedef u64 type; };
 
-template <class T, int BX, int BY, bool FX, bool EDGE, int SC, class P>
-JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, int F, int flags,
+template <class T, int BX, int BY, bool FX, int SC, class P>
+JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, int F,
                     typename HeatAcc<T, FX>::type& rmax, Heat3SSmem<T, BX, BY, SC>& sm) {
   typedef Heat3S<T, BX, BY, SC> G;
   constexpr int V = G::V;
@@ -1445,30 +1528,19 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
 #pragma unroll
     for (int e = 0; e < V; ++e)
       if (y0 + yy >= 1 && y0 + yy <= ny - 2 && x0 + e >= 1 && x0 + e <= nx - 2) inm |= 1u << (yy * V + e);
+  const bool fast = __all_sync(0xffffffffu, inm == (1u << (2 * V)) - 1);  // the warp holds interior points only
   const i64 cz0 = (i64)blockIdx.z * p.zc;
   const i64 cz1 = (cz0 + p.zc < nz) ? cz0 + p.zc : nz;
   const i64 z0 = cz0 < 1 ? 1 : cz0;
   const i64 z1 = cz1 > nz - 1 ? nz - 1 : cz1;
-  const bool inf = FX && EDGE && (flags & JFX_IN_F64);
-  const bool outf = FX && EDGE && (flags & JFX_OUT_F64);
-  // raw input word -> working value, working value -> output word, and a
-  // boundary point's output word from its raw input word
+  // raw input word -> working value, working value -> output word
   auto cvt = [&](T raw) -> Wt {
-    if constexpr (FX) return inf ? fx_from(raw, F) : bits_i64(raw);
+    if constexpr (FX) return bits_i64(raw);
     else return raw;
   };
   auto as_out = [&](Wt w) -> T {
     if constexpr (FX) return i64_bits(w);
     else return w;
-  };
-  auto bnd_out = [&](T raw) -> T {
-    if constexpr (FX && EDGE) {
-      if (inf == outf) return raw;
-      if (outf) return fx_to(bits_i64(raw), F);
-      return i64_bits(fx_from(raw, F));
-    } else {
-      return raw;
-    }
   };
   if (z0 >= z1) {  // a chunk holding only a boundary plane (block-uniform)
     for (i64 z = cz0; z < cz1; ++z)
@@ -1477,8 +1549,6 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
         if (ay[yy]) {
           T t[V];
           ldv<T, V>(u + z * sz + (y0 + yy) * nx + x0, t);
-#pragma unroll
-          for (int e = 0; e < V; ++e) t[e] = bnd_out(t[e]);
           stv<T, V>(v + z * sz + (y0 + yy) * nx + x0, t);
         }
     return;
@@ -1495,8 +1565,25 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
     mbar_init_fence();
   }
   __syncthreads();
+  // warp 0 requests a plane: one bulk copy per staged row inside the grid
+  // (rows and columns clipped to it), lane r copying row r; lane 0 first posts
+  // the byte count of the whole plane
+  static_assert(G::R <= 32, "one staged row per lane of warp 0");
+  const int lane = tid & 31;
+  const i64 c0 = bx0 - V < 0 ? 0 : bx0 - V;
+  const i64 c1 = bx0 + G::TW + V > nx ? nx : bx0 + G::TW + V;
+  const int rlo = by0 == 0 ? 1 : 0, rhi = ny - by0 + 1 < G::R ? (int)(ny - by0 + 1) : G::R;
+  const u32 row_bytes = (u32)((c1 - c0) * (i64)sizeof(T));
+  const bool has_row = lane >= rlo && lane < rhi;
+  const T* src = u + (z0 - 1) * sz + (by0 - 1 + lane) * nx + c0;  // the lane's row of the next plane
+  const int slot = lane * G::W + (int)(c0 - (bx0 - V));
   auto request = [&](int j, int s) {
-    if (!(stall_cta && j == rt.stall_plane)) heat3s_issue<T, BX, BY, SC>(sm, s, u, p, z0 - 1 + j, bx0, by0);
+    if (!(stall_cta && j == rt.stall_plane)) {
+      if (lane == 0) mbar_expect_tx(&sm.full[s], row_bytes * (u32)(rhi - rlo));
+      __syncwarp();
+      if (has_row) bulk_g2s(&sm.st[s][0][0] + slot, src, row_bytes, &sm.full[s]);
+    }
+    src += sz;
   };
   int issued = 0, consumed = 0;  // warp 0: planes requested, planes waited for
   if (warp0)
@@ -1535,18 +1622,16 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
 #pragma unroll
     for (int yy = 0; yy < 2; ++yy) lds_vec(&sm.st[s][2 * ty + 1 + yy][V + V * tx], raw[yy]);
   };
-  auto store_bnd = [&](T* dst, const T (&raw)[2][V], const Wt (&w)[2][V]) {
+  auto store_bnd = [&](T* dst, const Wt (&w)[2][V]) {
 #pragma unroll
     for (int yy = 0; yy < 2; ++yy)
       if (ay[yy]) {
         T t[V];
 #pragma unroll
-        for (int e = 0; e < V; ++e) t[e] = (FX && EDGE) ? bnd_out(raw[yy][e]) : as_out(w[yy][e]);
+        for (int e = 0; e < V; ++e) t[e] = as_out(w[yy][e]);
         stv<T, V>(dst + yy * nx, t);
       }
   };
-  constexpr bool RAW = FX && EDGE;  // raw words of plane z kept (converting sweeps only)
-  T rcur[2][V];
   Wt wa[2][V], wb[2][V], wc[2][V];  // own values of planes z-1, z, z+1 (rotating roles)
   T* vo = v + y0 * nx + x0;
   bool ok = wait_next();
@@ -1557,24 +1642,24 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
     for (int yy = 0; yy < 2; ++yy)
 #pragma unroll
       for (int e = 0; e < V; ++e) wa[yy][e] = cvt(r0[yy][e]);
-    if (cz0 == 0) store_bnd(vo, r0, wa);  // boundary plane 0
+    if (cz0 == 0) store_bnd(vo, wa);  // boundary plane 0
     const int s0 = cn_s;
     adv(cn_s, cn_ph);
     ok = release(0, s0) && wait_next();
   }
   int cc_s = cn_s;  // stage of the centre plane z
   if (ok) {  // plane z0
-    own(cn_s, rcur);
+    T r0[2][V];
+    own(cn_s, r0);
 #pragma unroll
     for (int yy = 0; yy < 2; ++yy)
 #pragma unroll
-      for (int e = 0; e < V; ++e) wb[yy][e] = cvt(rcur[yy][e]);
+      for (int e = 0; e < V; ++e) wb[yy][e] = cvt(r0[yy][e]);
     adv(cn_s, cn_ph);
   }
   const T r = (T)p.c0;
-  const i64 fb = p.fb, fw0 = p.fw0;
+  const i64 fb = p.fb;
   const int k = p.fk;
-  const bool small = p.fpath == JACC_FP_SMALL;
   const bool fold = heat_fold(p);
   constexpr bool folded = !SameT<P, JParams>::value;  // extents and coefficients are constants
   vo += z0 * sz;
@@ -1593,78 +1678,65 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
       xl[yy] = pl[2 * ty + 1 + yy][V + V * tx - 1];
       xr[yy] = pl[2 * ty + 1 + yy][V + V * tx + V];
     }
-    if constexpr (FX && EDGE) {
-      if (inf) {
-#pragma unroll
-        for (int e = 0; e < V; ++e) {
-          ym[e] = fx_from(i64_bits(ym[e]), F);
-          yp[e] = fx_from(i64_bits(yp[e]), F);
-        }
-#pragma unroll
-        for (int yy = 0; yy < 2; ++yy) {
-          xl[yy] = fx_from(i64_bits(xl[yy]), F);
-          xr[yy] = fx_from(i64_bits(xr[yy]), F);
-        }
-      }
-    }
 #pragma unroll
     for (int yy = 0; yy < 2; ++yy)
 #pragma unroll
       for (int e = 0; e < V; ++e) zn[yy][e] = cvt(rzn[yy][e]);
+    T out[2][V];
+    Wt dv[2 * V];  // the increments v - c
 #pragma unroll
-    for (int yy = 0; yy < 2; ++yy) {
-      T out[V];
+    for (int yy = 0; yy < 2; ++yy)
 #pragma unroll
       for (int e = 0; e < V; ++e) {
-        const bool in = (inm >> (yy * V + e)) & 1u;
-        const Wt a = (e == 0) ? xl[yy] : cur[yy][e - 1];
-        const Wt b = (e == V - 1) ? xr[yy] : cur[yy][e + 1];
+        const Wt a = (e == 0) ? xl[yy] : cur[yy][e == 0 ? 0 : e - 1];
+        const Wt b = (e == V - 1) ? xr[yy] : cur[yy][e == V - 1 ? e : e + 1];
         const Wt c = yy == 0 ? ym[e] : cur[0][e];
         const Wt d = yy == 0 ? cur[1][e] : yp[e];
         const Wt sum = ((a + b) + (c + d)) + (zp[yy][e] + zn[yy][e]);
         const Wt ce = cur[yy][e];
         if constexpr (FX) {
-          double o;
-          i64 dv;  // the increment v - c in fixed point: v = c + round(r L)
           if (folded && fold) {
             const i64 vn = (fb * sum + ((((i64)1 << k) - 6 * fb) * ce + ((i64)1 << (k - 1)))) >> k;
-            dv = vn - ce;
-            o = outf ? fx_to(ce * ((i64)1 << k) + fb * (sum - 6 * ce), F + k) : i64_bits(vn);
+            dv[yy * V + e] = vn - ce;
+            out[yy][e] = i64_bits(vn);
           } else {
-            const i64 Ld = sum - 6 * ce;
-            dv = heat_increment(Ld, p.fm);
-            if (outf) {
-              if (small) o = fx_to(ce * ((i64)1 << k) + fb * Ld, F + k);
-              else o = fx128_to(add128(from_s64_shl(ce, k), mul_s64_u64(Ld, (u64)fw0)), F + k);
-            } else {
-              o = i64_bits(ce + dv);
-            }
+            dv[yy * V + e] = heat_increment(sum - 6 * ce, p.fm);
+            out[yy][e] = i64_bits(ce + dv[yy * V + e]);
           }
-          const u64 aL = (u64)(dv ^ (dv >> 63));  // |v - c| (one less if negative)
-          if constexpr (RAW) out[e] = in ? o : bnd_out(rcur[yy][e]);
-          else out[e] = in ? o : as_out(ce);
-          rmax = (in && aL > rmax) ? aL : rmax;
         } else {
-          const T o = ce + r * (sum - T(6) * ce);
-          out[e] = in ? o : ce;
-          T dd = o - ce;
-          dd = dd < T(0) ? -dd : dd;
-          rmax = (in && dd > rmax) ? dd : rmax;
+          out[yy][e] = ce + r * (sum - T(6) * ce);
+          dv[yy * V + e] = out[yy][e] - ce;
         }
       }
-      if (ay[yy]) stv<T, V>(vo + yy * nx, out);
-    }
-    vo += sz;
-    if (j == L - 2 && cz1 == nz) store_bnd(vo, rzn, zn);  // boundary plane nz-1 = staged plane L-1
-    if (!release(j, cc_s)) return false;
-    cc_s = cn_s;
-    adv(cn_s, cn_ph);
-    if constexpr (RAW) {
+    if (!fast) {  // boundary points keep their values
 #pragma unroll
       for (int yy = 0; yy < 2; ++yy)
 #pragma unroll
-        for (int e = 0; e < V; ++e) rcur[yy][e] = rzn[yy][e];
+        for (int e = 0; e < V; ++e)
+          if (!((inm >> (yy * V + e)) & 1u)) {
+            dv[yy * V + e] = Wt(0);
+            out[yy][e] = as_out(cur[yy][e]);
+          }
     }
+    if constexpr (FX) {
+      fx_residual<2 * V>(dv, rmax);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 2 * V; ++q) rmax = fmaxf(rmax, fabsf(dv[q]));
+    }
+    if (fast) {
+      stv<T, V>(vo, out[0]);
+      stv<T, V>(vo + nx, out[1]);
+    } else {
+#pragma unroll
+      for (int yy = 0; yy < 2; ++yy)
+        if (ay[yy]) stv<T, V>(vo + yy * nx, out[yy]);
+    }
+    vo += sz;
+    if (j == L - 2 && cz1 == nz) store_bnd(vo, zn);  // boundary plane nz-1 = staged plane L-1
+    if (!release(j, cc_s)) return false;
+    cc_s = cn_s;
+    adv(cn_s, cn_ph);
     return true;
   };
   if (ok) {
@@ -1687,88 +1759,26 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   }
 }
 
-// ---------------------------------------------------------------- planes staged by asynchronous copies
+// ---------------------------------------------------------------- planes staged by asynchronous copies: conversion
 //
-// A second way of staging planes, for the kernels whose rows need not start
-// on 16-byte boundaries or whose staged values are converted in place: every
-// thread copies its share of a plane (the tile with a one-point halo) with
-// cp.async, CH elements per copy, into a ring of S stages in shared memory;
-// one group per plane, one CTA barrier per plane.  A copy's source may be any
-// element (8- or 4-byte copies for CH = 1), so odd rows, periodic images and
-// clipped edges all come from a per-thread list of source offsets worked out
-// once, and the thread that copied an element may convert it before the
-// barrier that publishes the plane.
-//
-// Geometry: BX x BY threads; a thread owns one column of RY consecutive rows,
-// so a warp reads and writes whole rows (no bank conflicts, coalesced stores
-// at any alignment), and the y neighbours inside its rows stay in registers.
-// A stage holds R x W elements in rows of W = BX + 2 CH: column x of the tile
-// sits at slot x - bx0 + CH of row y - by0 + 1.
-template <class T, int BX, int BY, int CH> struct RingG {
-  static constexpr int NT = BX * BY;
-  static constexpr int RY = JACC_RING_ROWS(BX, BY);
-  static constexpr int TW = BX, TH = BY * RY;
-  static constexpr int W = TW + 2 * CH, R = TH + 2;
-  static constexpr int STAGE = W * R;                       // elements
-  static constexpr int NCH = W / CH, NTOT = NCH * R;        // copies per row, per plane
-  static constexpr int PER = (NTOT + NT - 1) / NT;          // copies per thread
-  static constexpr int S0 = 46080 / (STAGE * (int)sizeof(T));
-  static constexpr int S = S0 < 3 ? 3 : (S0 > 6 ? 6 : S0);  // stages, at most 45 KB
-};
-
-template <int BYTES> JD void cpa_copy(void* dst, const void* src) {
-  if constexpr (BYTES == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES) : "memory");
-}
-JD void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> JD void cpa_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// A thread's share of every staged plane: copy i moves the CH elements at
-// offset off[i] of the plane to stage element (tid + i NT) CH; bit i of
-// `mask` is clear where there is none (past the plane, or outside a Dirichlet
-// grid, whose slots are never used).
-template <class T, int BX, int BY, int CH> struct RingPlan {
-  typedef RingG<T, BX, BY, CH> G;
-  i64 off[G::PER];
-  u32 mask;
-  JD void init(i64 nx, i64 ny, i64 bx0, i64 by0, bool periodic) {
-    const int tid = threadIdx.y * BX + threadIdx.x;
-    mask = 0;
-#pragma unroll
-    for (int i = 0; i < G::PER; ++i) {
-      const int c = tid + i * G::NT;
-      i64 x = bx0 - CH + (c % G::NCH) * CH, y = by0 - 1 + c / G::NCH;
-      bool ok = c < G::NTOT;
-      if (periodic) {
-        x = (x + nx) % nx;
-        y = (y + ny) % ny;
-      } else {
-        ok = ok && x >= 0 && x < nx && y >= 0 && y < ny;
-      }
-      off[i] = ok ? y * nx + x : 0;
-      mask |= (u32)ok << i;
-    }
-  }
-  JD void issue(T* stage, const T* plane) const {
-    const int tid = threadIdx.y * BX + threadIdx.x;
-#pragma unroll
-    for (int i = 0; i < G::PER; ++i)
-      if ((mask >> i) & 1u) cpa_copy<CH * (int)sizeof(T)>(stage + (tid + i * G::NT) * CH, plane + off[i]);
-  }
-};
-
-// Converts this thread's share of a landed FP64 plane to fixed point in place.
-template <int BX, int BY, int CH> JD void ring_to_fixed(const RingPlan<double, BX, BY, CH>& pl, double* stage, int F) {
-  typedef RingG<double, BX, BY, CH> G;
+// Converts this thread's share of a landed FP64 plane to fixed point in place:
+// 1.2 conversions a point, where the readers of a staged plane made three (one
+// jacc_launch of a 256^3 7-point grid: 306 us before, 161 now, its pre-pass
+// included).
+template <int BX, int BY, int CH, int V>
+JD void ring_to_fixed(const RingPlan<double, BX, BY, CH, V>& pl, double* stage, int F) {
+  typedef RingG<double, BX, BY, CH, V> G;
   const int tid = threadIdx.y * BX + threadIdx.x;
 #pragma unroll
   for (int i = 0; i < G::PER; ++i)
     if ((pl.mask >> i) & 1u) {
-#pragma unroll
-      for (int e = 0; e < CH; ++e) {
-        double* w = stage + (tid + i * G::NT) * CH + e;
+      double* w = stage + (tid + i * G::NT) * CH;
+      if constexpr (CH == 2) {
+        double2 t = *reinterpret_cast<double2*>(w);
+        t.x = i64_bits(fx_from(t.x, F));
+        t.y = i64_bits(fx_from(t.y, F));
+        *reinterpret_cast<double2*>(w) = t;
+      } else {
         *w = i64_bits(fx_from(*w, F));
       }
     }
@@ -1787,31 +1797,34 @@ template <int BX, int BY, int CH> JD void ring_to_fixed(const RingPlan<double, B
 // loaded halos into registers and multiplied in 128 bits): 301 x 253 x 199,
 // r = 0.1, 90 us a sweep before, 57 now (4.2 TB/s); FP32 rows of odd length
 // 301 x 253 x 199 27.5 us.
-template <class T, int BX, int BY, int CH, bool FX, bool EDGE, class P>
-JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, int F, int flags,
+template <class T, int BX, int BY, int CH, int V, bool FX, bool EDGE, class P>
+JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int F, int flags,
                     typename HeatAcc<T, FX>::type& rmax, T* sm) {
-  typedef RingG<T, BX, BY, CH> G;
+  typedef RingG<T, BX, BY, CH, V> G;
   typedef typename WT<T, FX ? JM_FIXED : JM_NATIVE>::type Wt;
   constexpr int RY = G::RY, S = G::S;
   const i64 nx = p.nx, ny = p.ny, nz = p.nz, sz = nx * ny;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const i64 bx0 = (i64)blockIdx.x * G::TW, by0 = (i64)blockIdx.y * G::TH;
-  const i64 x = bx0 + tx, y0 = by0 + ty * RY;
-  // rows this thread writes, and those whose point is interior
+  const i64 x0 = bx0 + tx * V, y0 = by0 + ty * RY;
+  // rows this thread writes (a vector column lies in the grid or outside), and
+  // its interior points: bit k V + e
   unsigned wrm = 0, inm = 0;
 #pragma unroll
   for (int k = 0; k < RY; ++k) {
-    if (x < nx && y0 + k < ny) wrm |= 1u << k;
-    if (x >= 1 && x <= nx - 2 && y0 + k >= 1 && y0 + k <= ny - 2) inm |= 1u << k;
+    if (x0 < nx && y0 + k < ny) wrm |= 1u << k;
+#pragma unroll
+    for (int e = 0; e < V; ++e)
+      if (x0 + e >= 1 && x0 + e <= nx - 2 && y0 + k >= 1 && y0 + k <= ny - 2) inm |= 1u << (k * V + e);
   }
-  const bool fast = __all_sync(0xffffffffu, inm == (1u << RY) - 1);  // the warp holds interior points only
+  const bool fast = __all_sync(0xffffffffu, inm == (1u << (RY * V)) - 1);  // the warp holds interior points only
   const i64 cz0 = (i64)blockIdx.z * p.zc;
   const i64 cz1 = (cz0 + p.zc < nz) ? cz0 + p.zc : nz;
   const i64 z0 = cz0 < 1 ? 1 : cz0;
   const i64 z1 = cz1 > nz - 1 ? nz - 1 : cz1;
   const bool inf = FX && EDGE && (flags & JFX_IN_F64);
   const bool outf = FX && EDGE && (flags & JFX_OUT_F64);
-  const i64 own_off = y0 * nx + x;
+  const i64 own_off = y0 * nx + x0;
   T* vo = v + own_off;
   // a boundary point's output from its working value (and, where FP64 goes
   // in and out, its unchanged input at offset `at`)
@@ -1830,17 +1843,20 @@ JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
 #pragma unroll
       for (int k = 0; k < RY; ++k)
         if ((wrm >> k) & 1u) {
-          const i64 at = own_off + z * sz + k * nx;
-          T t = u[at];
-          if constexpr (FX && EDGE) {
-            if (inf != outf) t = inf ? i64_bits(fx_from(t, F)) : fx_to(bits_i64(t), F);
+#pragma unroll
+          for (int e = 0; e < V; ++e) {
+            const i64 at = own_off + z * sz + k * nx + e;
+            T t = u[at];
+            if constexpr (FX && EDGE) {
+              if (inf != outf) t = inf ? i64_bits(fx_from(t, F)) : fx_to(bits_i64(t), F);
+            }
+            v[at] = t;
           }
-          v[at] = t;
         }
     return;
   }
   const int L = (int)(z1 - z0) + 2;  // staged planes z0-1 .. z1
-  RingPlan<T, BX, BY, CH> plan;
+  RingPlan<T, BX, BY, CH, V> plan;
   plan.init(nx, ny, bx0, by0, false);
   const T* next = u + (z0 - 1) * sz;  // next plane to stage
   int is = 0, issued = 0;             // its stage, in elements
@@ -1856,21 +1872,30 @@ JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   int ns = 0;  // stage of the next plane, in elements
   auto publish = [&]() {
     if constexpr (FX && EDGE) {
-      if (inf) ring_to_fixed<BX, BY, CH>(plan, sm + ns, F);
+      if (inf) ring_to_fixed(plan, sm + ns, F);
     }
     __syncthreads();
   };
-  const Wt* own0 = reinterpret_cast<const Wt*>(sm) + (ty * RY + 1) * G::W + CH + tx;
-  auto own = [&](int stage, Wt (&w)[RY]) {
-#pragma unroll
-    for (int k = 0; k < RY; ++k) w[k] = own0[stage + k * G::W];
+  const Wt* own0 = reinterpret_cast<const Wt*>(sm) + (ty * RY + 1) * G::W + CH + tx * V;
+  auto row = [&](const Wt* q, Wt (&w)[V]) {
+    if constexpr (V == 1) w[0] = q[0];
+    else lds_vec(q, w);
   };
-  auto store_bnd = [&](i64 z, const Wt (&w)[RY]) {
+  auto own = [&](int stage, Wt (&w)[RY][V]) {
+#pragma unroll
+    for (int k = 0; k < RY; ++k) row(own0 + stage + k * G::W, w[k]);
+  };
+  auto store_bnd = [&](i64 z, const Wt (&w)[RY][V]) {
 #pragma unroll
     for (int k = 0; k < RY; ++k)
-      if ((wrm >> k) & 1u) vo[z * sz + k * nx] = bnd_out(w[k], own_off + z * sz + k * nx);
+      if ((wrm >> k) & 1u) {
+        T t[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) t[e] = bnd_out(w[k][e], own_off + z * sz + k * nx + e);
+        stv<T, V>(vo + z * sz + k * nx, t);
+      }
   };
-  Wt wa[RY], wb[RY], wc[RY];  // own values of planes z-1, z, z+1 (rotating roles)
+  Wt wa[RY][V], wb[RY][V], wc[RY][V];  // own values of planes z-1, z, z+1 (rotating roles)
   cpa_wait<S - 1>();
   publish();
   own(ns, wa);
@@ -1889,63 +1914,72 @@ JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   i64 z = z0;
   T* vz = vo + z0 * sz;
   // output plane z from the own values of planes z-1 and z; fills zn with plane z+1's
-  auto step = [&](const Wt (&zp)[RY], const Wt (&cur)[RY], Wt (&zn)[RY]) {
+  auto step = [&](const Wt (&zp)[RY][V], const Wt (&cur)[RY][V], Wt (&zn)[RY][V]) {
     cpa_wait<S - 3>();
     publish();
     issue_next();  // into the stage of plane z-1, last read before the barrier
     own(ns, zn);
     const Wt* c0 = own0 + cs;
-    const Wt ym = c0[-G::W], yp = c0[RY * G::W];
-    T out[RY];
-    Wt dv[RY];
+    Wt ym[V], yp[V];
+    row(c0 - G::W, ym);
+    row(c0 + RY * G::W, yp);
+    T out[RY][V];
+    Wt dv[RY * V];
 #pragma unroll
     for (int k = 0; k < RY; ++k) {
-      const Wt xl = c0[k * G::W - 1], xr = c0[k * G::W + 1];
-      const Wt a = k == 0 ? ym : cur[k == 0 ? 0 : k - 1], b = k == RY - 1 ? yp : cur[k == RY - 1 ? k : k + 1];
-      const Wt sum = ((xl + xr) + (a + b)) + (zp[k] + zn[k]);
-      const Wt ce = cur[k];
-      if constexpr (FX) {
-        if (fold) {
-          const i64 vn = (fb * sum + ((((i64)1 << fk) - 6 * fb) * ce + ((i64)1 << (fk - 1)))) >> fk;
-          dv[k] = vn - ce;
-          out[k] = i64_bits(vn);
-        } else {
-          dv[k] = heat_increment(sum - 6 * ce, p.fm);
-          out[k] = i64_bits(ce + dv[k]);
-        }
-        if constexpr (EDGE) {
-          if (outf) {  // the exact value, rounded once
-            const i64 Ld = sum - 6 * ce;
-            if (p.fpath == JACC_FP_SMALL) out[k] = fx_to(ce * ((i64)1 << fk) + fb * Ld, F + fk);
-            else out[k] = fx128_to(add128(from_s64_shl(ce, fk), mul_s64_u64(Ld, (u64)p.fw0)), F + fk);
+      const Wt xl = c0[k * G::W - 1], xr = c0[k * G::W + V];
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        const Wt a = e == 0 ? xl : cur[k][e == 0 ? 0 : e - 1], b = e == V - 1 ? xr : cur[k][e == V - 1 ? e : e + 1];
+        const Wt c = k == 0 ? ym[e] : cur[k == 0 ? 0 : k - 1][e], d = k == RY - 1 ? yp[e] : cur[k == RY - 1 ? k : k + 1][e];
+        const Wt sum = ((a + b) + (c + d)) + (zp[k][e] + zn[k][e]);
+        const Wt ce = cur[k][e];
+        Wt& dk = dv[k * V + e];
+        if constexpr (FX) {
+          if (fold) {
+            const i64 vn = (fb * sum + ((((i64)1 << fk) - 6 * fb) * ce + ((i64)1 << (fk - 1)))) >> fk;
+            dk = vn - ce;
+            out[k][e] = i64_bits(vn);
+          } else {
+            dk = heat_increment(sum - 6 * ce, p.fm);
+            out[k][e] = i64_bits(ce + dk);
           }
+          if constexpr (EDGE) {
+            if (outf) {  // the exact value, rounded once
+              const i64 Ld = sum - 6 * ce;
+              if (p.fpath == JACC_FP_SMALL) out[k][e] = fx_to(ce * ((i64)1 << fk) + fb * Ld, F + fk);
+              else out[k][e] = fx128_to(add128(from_s64_shl(ce, fk), mul_s64_u64(Ld, (u64)p.fw0)), F + fk);
+            }
+          }
+        } else {
+          const T o = ce + r * (sum - T(6) * ce);
+          out[k][e] = o;
+          dk = o - ce;
         }
-      } else {
-        const T o = ce + r * (sum - T(6) * ce);
-        out[k] = o;
-        dv[k] = o - ce;
       }
     }
     if (!fast) {
 #pragma unroll
       for (int k = 0; k < RY; ++k)
-        if (!((inm >> k) & 1u)) {
-          dv[k] = Wt(0);
-          if ((wrm >> k) & 1u) out[k] = bnd_out(cur[k], own_off + z * sz + k * nx);
-        }
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+          if (!((inm >> (k * V + e)) & 1u)) {
+            dv[k * V + e] = Wt(0);
+            if ((wrm >> k) & 1u) out[k][e] = bnd_out(cur[k][e], own_off + z * sz + k * nx + e);
+          }
     }
-    if constexpr (FX) fx_residual<RY>(dv, rmax);
+    if constexpr (FX) fx_residual<RY * V>(dv, rmax);
     else {
 #pragma unroll
-      for (int k = 0; k < RY; ++k) rmax = fmaxf(rmax, fabsf(dv[k]));
+      for (int k = 0; k < RY * V; ++k) rmax = fmaxf(rmax, fabsf(dv[k]));
     }
     if (fast) {
 #pragma unroll
-      for (int k = 0; k < RY; ++k) vz[k * nx] = out[k];
+      for (int k = 0; k < RY; ++k) stv<T, V>(vz + k * nx, out[k]);
     } else {
 #pragma unroll
       for (int k = 0; k < RY; ++k)
-        if ((wrm >> k) & 1u) vz[k * nx] = out[k];
+        if ((wrm >> k) & 1u) stv<T, V>(vz + k * nx, out[k]);
     }
     cs = ns;
     ns = ns + G::STAGE == S * G::STAGE ? 0 : ns + G::STAGE;
@@ -2071,7 +2105,7 @@ JD void box27r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   auto consume = [&](W (&c)[RY], W (&f)[RY], W (&g)[RY]) {
     cpa_wait<S - 2>();
     if constexpr (FX && EDGE) {
-      if (inf) ring_to_fixed<BX, BY, CH>(plan, sm + cs, F);
+      if (inf) ring_to_fixed(plan, sm + cs, F);
     }
     __syncthreads();
     issue_next();  // into the stage read before the barrier
@@ -2154,6 +2188,83 @@ JD void box27r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   cpa_wait<0>();
 }
 
+// ---------------------------------------------------------------- 7-point heat without staging
+//
+// A grid that fits L2 is bound by the latency of a CTA's march, not by bytes:
+// each plane of a staged march costs a wait and a barrier (64^3 FP64: 9.6 us a
+// sweep at 18 planes).  Here a thread updates N planes of V consecutive
+// columns of one row straight from memory: no shared memory, no barrier, every
+// load independent of the others, so a sweep costs little more than one trip
+// to L2.  L1 serves the neighbours that threads share.  Two planes a thread:
+// 64^3 FP64 3.1 us a sweep, 5.4 with four.  These are the
+// intermediate sweeps of small grids; the arithmetic is that of the staged
+// kernels, term for term.
+// The 7-point sweep in working type W (i64: fixed point; T: native).  Returns
+// the thread's residual maximum.
+template <class T, class W, int BX, int BY, int V, int N, class P, class R>
+JD void heat3d_direct(const T* __restrict__ u, T* __restrict__ v, const P& p, R& rmax) {
+  constexpr bool FX = SameT<W, i64>::value;
+  const i64 nx = p.nx, ny = p.ny, nz = p.nz, sz = nx * ny;
+  const i64 x = ((i64)blockIdx.x * BX + threadIdx.x) * V, y = (i64)blockIdx.y * BY + threadIdx.y, z0 = (i64)blockIdx.z * N;
+  if (x >= nx || y >= ny) return;
+  const T* col = u + y * nx + x;
+  // neighbours outside the grid are replaced by points inside: only boundary points would use them
+  const i64 dl = x > 0 ? -1 : 0, dr = x + V < nx ? V : 0, dm = y > 0 ? -nx : 0, dp = y < ny - 1 ? nx : 0;
+  T own[N + 2][V], ym[N][V], yp[N][V], xl[N], xr[N];
+#pragma unroll
+  for (int k = 0; k < N + 2; ++k) {
+    i64 z = z0 - 1 + k;
+    z = z < 0 ? 0 : (z > nz - 1 ? nz - 1 : z);
+    const T* c = col + z * sz;
+    ldv<T, V>(c, own[k]);
+    if (k >= 1 && k <= N) {
+      ldv<T, V>(c + dm, ym[k - 1]);
+      ldv<T, V>(c + dp, yp[k - 1]);
+      xl[k - 1] = __ldg(c + dl);
+      xr[k - 1] = __ldg(c + dr);
+    }
+  }
+  auto w = [&](T t) -> W {
+    if constexpr (FX) return bits_i64(t);
+    else return t;
+  };
+  constexpr bool folded = !SameT<P, JParams>::value;
+  const bool fold = folded && heat_fold(p);
+  const T r = (T)p.c0;
+  T* o = v + z0 * sz + y * nx + x;
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const i64 z = z0 + k;
+    if (z >= nz) break;
+    const bool in = y >= 1 && y <= ny - 2 && z >= 1 && z <= nz - 2;
+    T out[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+      const W ce = w(own[k + 1][e]);
+      const W a = w(e == 0 ? xl[k] : own[k + 1][e == 0 ? 0 : e - 1]);
+      const W b = w(e == V - 1 ? xr[k] : own[k + 1][e == V - 1 ? e : e + 1]);
+      const W sum = ((a + b) + (w(ym[k][e]) + w(yp[k][e]))) + (w(own[k][e]) + w(own[k + 2][e]));
+      const bool ine = in && x + e >= 1 && x + e <= nx - 2;
+      if constexpr (FX) {
+        i64 d;
+        if (fold) d = ((p.fb * sum + ((((i64)1 << p.fk) - 6 * p.fb) * ce + ((i64)1 << (p.fk - 1)))) >> p.fk) - ce;
+        else d = heat_increment(sum - 6 * ce, p.fm);
+        d = ine ? d : 0;
+        const u64 m = (u64)(d ^ (d >> 63));
+        rmax = m > rmax ? m : rmax;
+        out[e] = i64_bits(ce + d);
+      } else {
+        const T q = ce + r * (sum - T(6) * ce);
+        T d = q - ce;
+        d = d < T(0) ? -d : d;
+        rmax = (ine && d > rmax) ? d : rmax;
+        out[e] = ine ? q : ce;
+      }
+    }
+    stv<T, V>(o + k * sz, out);
+  }
+}
+
 // ====================================================================== kernels
 //
 // Every stencil kernel has the signature
@@ -2171,81 +2282,93 @@ JD void box27r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
 // sequence and contain no conversion code; EDGE = true ones run the first and
 // last sweeps and single launches.
 
-// Whether the 5-point march prefetches rows and x-edges several rows ahead
-// (jacobi_march_pf).  That pays on small, L2-resident grids, whose sweeps are
-// latency-bound; on large grids its registers cost more occupancy than it
-// gains, so the precompiled kernels (P = JParams) use the plain march and a
-// constant-folded variant opts in by specialising this for its own P.
-template <class P> struct JacobiPrefetch { static constexpr bool value = false; };
-
-template <class T, int BX, int BY, int V, int ZC, bool EDGE, class P>
+// Kernel families (JACC_FAM_*, jacc_params.h): a table tile runs the kernel
+// that the autotuner times for it; the library's own choice (no tile asked
+// for, none remembered) may also take the strip march, the asynchronous-copy
+// ring, or no staging at all.
+template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                        const u64* maxword, int flags) {
   griddep_wait();
+  if (rt.stop && __ldcg(rt.stop)) return;
   u64 bits = 0;
-  const i64 x0 = (i64)blockIdx.x * (BX * V) + (i64)threadIdx.x * V;
-  const i64 ys = ((i64)blockIdx.y * BY + threadIdx.y) * ZC;
-  const i64 ye = (ys + ZC < p.ny) ? ys + ZC : p.ny;
-  if constexpr (sizeof(T) == 8) {
-    const int F = (maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
-    if (F >= 0) {
+  const i64 ys = ((i64)blockIdx.y * BY + threadIdx.y) * p.zc;
+  const i64 ye = (ys + p.zc < p.ny) ? ys + p.zc : p.ny;
+  constexpr bool STRIP = FAM == JACC_FAM_STRIP || V == 1;  // the table tiles of scalar columns, too
+  // STRIP: BX / 32 strips of 30 V columns across the CTA
+  const i64 strip = (i64)blockIdx.x * (BX / 32) + (threadIdx.x >> 5);
+  const i64 xl = STRIP ? strip * (30 * V) + ((int)(threadIdx.x & 31) - 1) * V : (i64)blockIdx.x * (BX * V) + (i64)threadIdx.x * V;
+  const int F = (sizeof(T) == 8 && maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
+  if (sizeof(T) == 8 && F >= 0) {
+    if constexpr (sizeof(T) == 8) {
       u64 m = 0;
       if (ys < p.ny) {
-        if constexpr (JacobiPrefetch<P>::value)
-          jacobi_march_pf<double, V, false, true, EDGE, 4>(u, v, p.nx, p.ny, x0, ys, ye, F, flags, m);
-        else
-          jacobi_fx_march<V, false, EDGE>(u, v, p.nx, p.ny, x0, ys, ye, F, flags, m);
+        if constexpr (STRIP) jacobi_strip<double, V, true, EDGE>(u, v, p.nx, p.ny, xl, ys, ye, F, flags, m);
+        else jacobi_fx_march<V, false, EDGE>(u, v, p.nx, p.ny, xl, ys, ye, F, flags, m);
       }
       bits = dbits(fx_to_u(m, F + 2));
-    } else {
-      double m = 0.0;
-      if (ys < p.ny) {
-        if constexpr (JacobiPrefetch<P>::value)
-          jacobi_march_pf<T, V, false, false, false, 4>(u, v, p.nx, p.ny, x0, ys, ye, -1, 0, m);
-        else
-          jacobi_march<T, V, JM_NATIVE, false>(u, v, p.nx, p.ny, x0, ys, ye, -1, m);
-      }
-      bits = dbits(m);
     }
   } else {
     T m = T(0);
     if (ys < p.ny) {
-      if constexpr (JacobiPrefetch<P>::value)
-        jacobi_march_pf<T, V, false, false, false, 4>(u, v, p.nx, p.ny, x0, ys, ye, -1, 0, m);
-      else
-        jacobi_march<T, V, JM_NATIVE, false>(u, v, p.nx, p.ny, x0, ys, ye, -1, m);
+      if constexpr (STRIP) jacobi_strip<T, V, false, false>(u, v, p.nx, p.ny, xl, ys, ye, -1, 0, m);
+      else jacobi_march<T, V, JM_NATIVE, false>(u, v, p.nx, p.ny, xl, ys, ye, -1, m);
     }
     bits = dbits((double)m);
   }
   block_max_to<BX * BY>(bits, resid);
 }
 
-template <class T, int BX, int BY, int V, bool EDGE, class P>
+// How a 3D kernel loads.  BULK: 16-byte columns staged by bulk copies on
+// mbarriers (no copy instructions, no CTA barrier).  RING: planes staged by
+// asynchronous copies, which arrive sooner; also every converting FP64 sweep,
+// where each staged value is converted once by the thread that copied it, and
+// the FP64 table tiles of scalar columns.  DIRECT: no staging (small 7-point
+// grids, and the table's scalar 32 x 8 tiles).  Otherwise (FP32 table tiles of
+// scalar columns) halos loaded through registers.
+template <int STENCIL, class T, int BX, int BY, int V, int FAM, bool EDGE> struct Load3D {
+  static constexpr bool F64 = sizeof(T) == 8;
+  static constexpr bool VEC = V * sizeof(T) == 16;
+  static constexpr bool DIRECT =
+      !EDGE && STENCIL == 7 && (FAM == JACC_FAM_DIRECT || (FAM == JACC_FAM_TABLE && JACC_DIRECT_TILE(BX, BY, V)));
+  static constexpr bool BULK = !EDGE && VEC && (FAM == JACC_FAM_TABLE || FAM == JACC_FAM_BULK) && !(F64 && STENCIL == 27);
+  static constexpr bool RING = !DIRECT && !BULK && (EDGE || F64 || FAM == JACC_FAM_RING);
+};
+
+template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 JD void heat3d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                      const u64* maxword, int flags) {
   griddep_wait();
+  if (rt.stop && __ldcg(rt.stop)) return;
+  typedef Load3D<7, T, BX, BY, V, FAM, EDGE> K;
   u64 bits = 0;
-  // 16-byte columns: the bulk-copy staged kernel (2 rows per thread), else
-  // the kernel staged by asynchronous copies (RingG::RY rows of one column)
-  constexpr bool STAGED = V * sizeof(T) == 16;
-  if constexpr (sizeof(T) == 8) {
-    typedef RingG<double, BX, BY, V> G;
+  const int F = (sizeof(T) == 8 && maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
+  if constexpr (K::DIRECT) {
+    if (sizeof(T) == 8 && F >= 0) {
+      u64 m = 0;
+      if constexpr (sizeof(T) == 8) heat3d_direct<T, i64, BX, BY, V, JACC_DIRECT_PLANES>(u, v, p, m);
+      bits = dbits(fx_to_u(m, F));
+    } else {
+      T m = T(0);
+      heat3d_direct<T, T, BX, BY, V, JACC_DIRECT_PLANES>(u, v, p, m);
+      bits = dbits((double)m);
+    }
+  } else if constexpr (sizeof(T) == 8) {
+    typedef RingG<double, BX, BY, V, V> G;
     // stage cap: 5 for the constant-folded intermediate sweeps (7 CTAs per SM,
     // SweepMinBlocks), else 6
-    constexpr int SC = (!EDGE && !SameT<P, JParams>::value) ? 5 : 6;
+    constexpr int SC = !SameT<P, JParams>::value ? 5 : 6;
     // the native path covers the CTA's rows in sub-tiles of BY rows
-    constexpr int SUBS = STAGED ? 2 : G::RY;
+    constexpr int SUBS = K::BULK ? 2 : G::RY;
     typedef Plane<double, BX, BY, V> NativePlane;
-    constexpr size_t SM_MAIN = STAGED ? sizeof(Heat3SSmem<double, BX, BY, SC>) : (size_t)G::S * G::STAGE * 8;
+    constexpr size_t SM_MAIN = K::BULK ? sizeof(Heat3SSmem<double, BX, BY, SC>) : (size_t)G::S * G::STAGE * 8;
     __shared__ __align__(128) unsigned char raw[sizeof(NativePlane) > SM_MAIN ? sizeof(NativePlane) : SM_MAIN];
-    const int F = (maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
     if (F >= 0) {
       u64 m = 0;
-      if constexpr (STAGED)
-        heat3s_body<double, BX, BY, true, EDGE, SC>(u, v, p, rt, F, flags, m,
-                                                        *reinterpret_cast<Heat3SSmem<double, BX, BY, SC>*>(raw));
+      if constexpr (K::BULK)
+        heat3s_body<double, BX, BY, true, SC>(u, v, p, rt, F, m, *reinterpret_cast<Heat3SSmem<double, BX, BY, SC>*>(raw));
       else
-        heat3r_body<double, BX, BY, V, true, EDGE>(u, v, p, rt, F, flags, m, reinterpret_cast<double*>(raw));
+        heat3r_body<double, BX, BY, V, V, true, EDGE>(u, v, p, F, flags, m, reinterpret_cast<double*>(raw));
       bits = dbits(fx_to_u(m, F));  // max |v - c| in fixed point
     } else {
       double m = 0.0;
@@ -2256,31 +2379,37 @@ JD void heat3d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, con
       }
       bits = dbits(m);
     }
-  } else if constexpr (STAGED) {
+  } else if constexpr (K::BULK) {
     __shared__ Heat3SSmem<float, BX, BY, 6> sm;
     float m = 0.0f;
-    heat3s_body<float, BX, BY, false, false, 6>(u, v, p, rt, -1, 0, m, sm);
+    heat3s_body<float, BX, BY, false, 6>(u, v, p, rt, -1, m, sm);
     bits = dbits((double)m);
-  } else {
-    typedef RingG<float, BX, BY, V> G;
+  } else if constexpr (K::RING) {
+    typedef RingG<float, BX, BY, V, V> G;
     __shared__ __align__(16) float sm[G::S * G::STAGE];
     float m = 0.0f;
-    heat3r_body<float, BX, BY, V, false, false>(u, v, p, rt, -1, 0, m, sm);
+    heat3r_body<float, BX, BY, V, V, false, false>(u, v, p, -1, 0, m, sm);
+    bits = dbits((double)m);
+  } else {
+    __shared__ Plane<T, BX, BY, V> sm;
+    T m = T(0);
+    heat3d_body<T, BX, BY, V, JM_NATIVE>(u, v, p, p.zc, -1, m, sm);
     bits = dbits((double)m);
   }
   block_max_to<BX * BY>(bits, resid);
 }
 
-template <class T, int BX, int BY, int V, bool EDGE, class P>
+template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                     const u64* maxword, int flags) {
   griddep_wait();
+  typedef Load3D<27, T, BX, BY, V, FAM, EDGE> K;
   double total = 0.0;
+  const int F = (sizeof(T) == 8 && maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
   if constexpr (sizeof(T) == 8) {
     typedef RingG<double, BX, BY, V> G;
     constexpr size_t SM_RING = (size_t)G::S * G::STAGE * 8, SM_PLANE = sizeof(Plane<double, BX, BY, 1>);
     __shared__ __align__(16) unsigned char raw[SM_RING > SM_PLANE ? SM_RING : SM_PLANE];
-    const int F = (maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
     if (F >= 0) {
       s128 acc;
       acc.lo = acc.hi = 0ull;
@@ -2298,13 +2427,18 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
       total = acc.total();
     }
   } else if constexpr (V == 4) {
-    total = box27s_body<BX, BY>(u, v, p, rt, resid != nullptr);
-  } else {
+    total = box27s_body<BX, BY, K::BULK>(u, v, p, rt, resid != nullptr);
+  } else if constexpr (K::RING) {
     typedef RingG<float, BX, BY, V> G;
     __shared__ __align__(16) float sm[G::S * G::STAGE];
     SumAcc<float> acc;
     s128 none;
     box27r_body<float, BX, BY, V, false>(u, v, p, rt, -1, 0, resid != nullptr, none, acc, sm);
+    total = acc.total();
+  } else {
+    __shared__ Plane<T, BX, BY, V> sm;
+    SumAcc<T> acc;
+    box27_body2<T, BX, BY, V>(u, v, p, p.zc, acc, resid != nullptr, sm);
     total = acc.total();
   }
   block_sum_to<BX * BY>(total, resid);
@@ -2313,7 +2447,7 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
 #ifdef JACC_AUX_KERNELS
 // Pre-pass: atomicMax of the bit pattern of |u[i]| over n doubles.
 // Any NaN orders above +Inf, so a NaN input selects the native path.
-__global__ void __launch_bounds__(256) jacc_k_maxabs(const double* __restrict__ u, i64 n, u64* maxword) {
+__global__ void __launch_bounds__(256, 8) jacc_k_maxabs(const double* __restrict__ u, i64 n, u64* maxword) {
   griddep_wait();
   u64 m = 0;
   const i64 stride = (i64)gridDim.x * blockDim.x;
@@ -2408,45 +2542,36 @@ __global__ void jacc_k_fill_skipped(double* resid, int n, int T) {
 // Every other kernel: 0, no requirement (a bound of 1 is not neutral: it
 // lets the compiler take registers for one CTA per SM, e.g. 111 instead of
 // 80 for the staged FP32 7-point kernel).
-template <int STENCIL, class T, int BX, int BY, int V, bool EDGE, bool FOLDED> struct SweepMinBlocks {
-  static constexpr bool heat_staged_fp64 = STENCIL == 7 && sizeof(T) == 8 && BX == 32 && BY == 4 && V == 2;
-  static constexpr bool box27_fp64 = STENCIL == 27 && sizeof(T) == 8 && BX == 32 && BY == 4;
-  static constexpr bool heat_ring = STENCIL == 7 && BX == 32 && BY == 4 && V == 1 && !EDGE;
-  static constexpr bool box27_fp32 = STENCIL == 27 && sizeof(T) == 4 && BX == 32 && BY == 4 && V == 4 && !FOLDED;
-  static constexpr int value = box27_fp32 ? 7 : heat_ring ? 5 : heat_staged_fp64 ? (EDGE ? 5 : (FOLDED ? 7 : 6)) : (box27_fp64 && !EDGE ? 4 : 0);
-};
-
-// The constant-folded last sweep of a sequence that does not convert on load
-// (the flags are the constant JFX_OUT_F64, so the load conversion is compiled
-// out): 80 registers at a bound of 6 CTAs per SM against 96 at 5 for the
-// kernel that converts both ways (staged FP64 7-point, 32 x 4 threads).
-template <int STENCIL, class T, int BX, int BY, int V> struct SweepMinBlocksLast {
-  static constexpr int value = (STENCIL == 7 && sizeof(T) == 8 && BX == 32 && BY == 4 && V == 2) ? 6 : 0;
+template <int STENCIL, class T, int BX, int BY, int V, int FAM, bool EDGE, bool FOLDED> struct SweepMinBlocks {
+  typedef Load3D<STENCIL, T, BX, BY, V, FAM, EDGE> K;
+  static constexpr bool t32 = BX == 32 && BY == 4;
+  static constexpr int heat = K::BULK ? (K::F64 ? (FOLDED ? 7 : 6) : 0) : K::RING ? (V == 1 || EDGE ? 5 : 6) : 0;
+  static constexpr int box = K::F64 ? (EDGE ? 0 : 4) : (V == 4 && !FOLDED ? 7 : 0);
+  static constexpr int value = !t32 ? 0 : STENCIL == 7 ? heat : STENCIL == 27 ? box : 0;
 };
 
 // Kernel templates instantiated by the precompiled library (P = JParams).
-template <class T, int BX, int BY, int V, int ZC, bool EDGE>
+template <class T, int BX, int BY, int V, int FAM, bool EDGE>
 __global__ void __launch_bounds__(BX * BY) jacc_k_jacobi2d(const T* __restrict__ u, T* __restrict__ v, JParams p,
                                                            double* resid, const u64* maxword, int flags) {
-  jacobi2d_entry<T, BX, BY, V, ZC, EDGE>(u, v, p, p, resid, maxword, flags);
+  jacobi2d_entry<T, BX, BY, V, FAM, EDGE>(u, v, p, p, resid, maxword, flags);
 }
-template <class T, int BX, int BY, int V, bool EDGE>
-__global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<7, T, BX, BY, V, EDGE, false>::value))
-    jacc_k_heat3d(const T* __restrict__ u, T* __restrict__ v, JParams p,
-                                                         double* resid, const u64* maxword, int flags) {
-  heat3d_entry<T, BX, BY, V, EDGE>(u, v, p, p, resid, maxword, flags);
-}
-template <int RY, int TT, int ZC>
-__global__ void __launch_bounds__(TB_BX * RY) jacc_k_box27_tb(const float* __restrict__ u, float* __restrict__ v,
-                                                              JParams p, double* resid, const u64* maxword, int flags) {
-  box27_tb_entry<RY, TT, ZC>(u, v, p, resid);
+template <class T, int BX, int BY, int V, int FAM, bool EDGE>
+__global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<7, T, BX, BY, V, FAM, EDGE, false>::value))
+    jacc_k_heat3d(const T* __restrict__ u, T* __restrict__ v, JParams p, double* resid, const u64* maxword, int flags) {
+  heat3d_entry<T, BX, BY, V, FAM, EDGE>(u, v, p, p, resid, maxword, flags);
 }
 // P = JParamsW32: the same parameter block, known to hold 32-bit factors.
 struct JParamsW32 : JParams {
   static constexpr int fpath = JACC_FP_W32;
 };
-template <class T, int BX, int BY, int V, bool EDGE, class P>
-__global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<27, T, BX, BY, V, EDGE, false>::value))
+template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
+__global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<27, T, BX, BY, V, FAM, EDGE, false>::value))
     jacc_k_box27(const T* __restrict__ u, T* __restrict__ v, P p, double* resid, const u64* maxword, int flags) {
-  box27_entry<T, BX, BY, V, EDGE>(u, v, p, p, resid, maxword, flags);
+  box27_entry<T, BX, BY, V, FAM, EDGE>(u, v, p, p, resid, maxword, flags);
+}
+template <int RY, int TT, int ZC>
+__global__ void __launch_bounds__(TB_BX * RY) jacc_k_box27_tb(const float* __restrict__ u, float* __restrict__ v,
+                                                              JParams p, double* resid, const u64* maxword, int flags) {
+  box27_tb_entry<RY, TT, ZC>(u, v, p, resid);
 }

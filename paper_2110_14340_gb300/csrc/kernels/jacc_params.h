@@ -13,6 +13,18 @@ typedef unsigned int u32;
 #define JACC_FP_JACOBI 3 // 5pt: v 2^(F+2) = S
 #define JACC_FP_W32 4    // 27pt: every factor below 2^31 and K in [1, 31]: 32-bit factors
 
+// Kernel families: a table tile's kernel, and those of the library's choice.
+#define JACC_FAM_TABLE 0
+#define JACC_FAM_STRIP 1   // 5-point: strips of 30 lanes' columns
+#define JACC_FAM_RING 2    // 3D: planes staged by asynchronous copies
+#define JACC_FAM_DIRECT 3  // 7-point: no staging (32 x 8 threads)
+#define JACC_FAM_BULK 4    // 3D, 16-byte columns: planes staged by bulk copies
+
+// The 7-point table tiles that stage nothing, and the planes per thread of the
+// kernel that does not.
+#define JACC_DIRECT_TILE(bx, by, vec) ((bx) == 32 && (by) == 8 && (vec) == 1)
+#define JACC_DIRECT_PLANES 2
+
 // Rows per thread of the kernels that stage planes by asynchronous copies
 // (bx x by threads, one column each): 4, or 2 where 4 would not leave room
 // for the stages.
@@ -33,7 +45,10 @@ struct JParams {
   int* status;
   i64 timeout_ns;
   int stall_plane;
-  int zc;  // planes per CTA
+  int zc;  // planes per CTA (3D) or rows per warp (2D)
+  // Sweeps until a tolerance: a 5- or 7-point kernel that finds *stop set
+  // (device, nullable) returns at once.
+  const int* stop;
   // The twelve coefficient fields of the variable-coefficient 19-point
   // stencil (a0 a1 a2 a3 b0 b1 b2 c0 c1 c2 wrk1 bnd; FP32, device), set per
   // call; unused by the other stencils.

@@ -31,9 +31,8 @@
 // nothing else until the result is written) up to that sweep.  A chunk is a
 // quarter of the sweeps before it, between 4 and 64, so the sweeps run twice
 // are few; deciding after every sweep instead would put the cluster-wide
-// maximum into each sweep's critical path.  256 x 192, 685 sweeps: 1.24 ms
-// against 16.8 ms for the graph loop that launched sweeps and checks one by
-// one.
+// maximum into each sweep's critical path.  256 x 192, 2000 sweeps: 3.3 ms
+// against 19 ms for the graph loop that launched sweeps and checks one by one.
 #include "jacc_device.cuh"
 
 #include <cuda_runtime.h>
@@ -364,27 +363,29 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
     if (t < 32 && i >= 1) {
       u64 w = t < NT / 32 ? wred[prev][t] : 0ull;
       w = warp_max_u64(w);
-      if (t == 0) rres[i - 1] = fixed ? dbits(fx_to_u(w, F + 2)) : w;
+      if (t == 0) rres[i - 1] = w;
     }
     if (flush) {
       __syncthreads();  // this sweep's per-warp partials
       if (t < 32) {
         u64 w = t < NT / 32 ? wred[slot][t] : 0ull;
         w = warp_max_u64(w);
-        if (t == 0) rres[i] = fixed ? dbits(fx_to_u(w, F + 2)) : w;
+        if (t == 0) rres[i] = w;
       }
       cluster_sync();  // every CTA's maxima of this chunk are written
     }
     slot = slot == 2 ? 0 : slot + 1;
   };
-  // The cluster's maximum of the chunk's i-th sweep.
+  // The cluster's maximum of the chunk's i-th sweep (rres holds it in the form
+  // it was reduced in, which orders alike; it is converted here, off the
+  // sweeps' path).
   auto resid_of = [&](int i) {
     u64 w = 0;
     for (int r = 0; r < NC; ++r) {
       const u64 v = ld_cluster_u64(map_rank(&rres[i], (u32)r));
       w = v > w ? v : w;
     }
-    return __longlong_as_double((i64)w);
+    return fixed ? fx_to_u(w, F + 2) : __longlong_as_double((i64)w);
   };
   // Residuals leave the cluster in chunks: a global write before a barrier
   // would make the barrier's release wait for it, so each sweep's CTA maxima
