@@ -90,8 +90,8 @@ cudaError_t launch_var19(const float* u, float* v, const JParams& p, double* res
 jacc_status check_buffers(const Kernel& k, const void* a, const void* b);
 // Destroys k's cached jacc_sweep_until graphs.
 void free_until_graphs(Kernel& k);
-cudaError_t launch_until_check(double* slot, int* counter, double* resid, double tol, int max_sweeps,
-                               cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_odd, cudaStream_t s);
+cudaError_t launch_until_check(double* slot, int* counter, int* stop, double* resid, double tol, int max_sweeps,
+                               cudaGraphConditionalHandle h_loop, cudaStream_t s);
 cudaError_t launch_until_final(const int* counter, int* status, int recompute, cudaGraphConditionalHandle h_final,
                                cudaStream_t s);
 

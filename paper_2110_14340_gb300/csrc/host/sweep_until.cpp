@@ -5,9 +5,12 @@
 // once and replayed:
 //   A      the first sweep (u0 -> u1; FP64 fixed point converts on load,
 //          after the max-abs pre-pass) and a one-thread check kernel;
-//   WHILE  (condition set by the checks) a pair of sweeps u1 -> u0 -> u1,
-//          each followed by a check; the second sits in an IF node on the
-//          same decision, so the loop can stop after either;
+//   WHILE  (condition set by the checks) an even number of sweeps u1 -> u0
+//          -> u1 ..., each followed by a check; the check that stops the loop
+//          sets a word that makes the rest of the body return at once (a
+//          conditional node costs several times the launches it guards: two
+//          sweeps per turn of the loop and an IF around the second took 24 us
+//          a sweep on small grids);
 //   F      a one-thread kernel that writes the sweep count and the result
 //          buffer and picks the final sweep;
 //   SWITCH the final sweep run again from the state before it with FP64
@@ -93,23 +96,23 @@ static jacc_status build_until(const Kernel& k, void* u0, void* u1, int32_t max_
   u64* maxword = ug.scratch;
   double* slot = reinterpret_cast<double*>(ug.scratch + 1);
   int* counter = reinterpret_cast<int*>(ug.scratch + 2);
+  int* stop = counter + 1;
   double* spare = reinterpret_cast<double*>(ug.scratch + 3);
   const u64* mw = fixed ? maxword : nullptr;
   jacc_status st = cuda_check(cudaGraphCreate(&ug.graph, 0), "cudaGraphCreate");
   if (st) return st;
-  cudaGraphConditionalHandle h_loop, h_odd, h_final;
+  cudaGraphConditionalHandle h_loop, h_final;
   st = cuda_check(cudaGraphConditionalHandleCreate(&h_loop, ug.graph, 0, 0), "conditional handle");
-  if (!st) st = cuda_check(cudaGraphConditionalHandleCreate(&h_odd, ug.graph, 0, 0), "conditional handle");
   if (!st) st = cuda_check(cudaGraphConditionalHandleCreate(&h_final, ug.graph, 3, cudaGraphCondAssignDefault),
                            "conditional handle");
   if (st) return st;
   const void* cu0 = u0;
   const void* cu1 = u1;
-  auto sweep = [&](const void* src, void* dst, double* r, int flags) {
-    return cuda_check(launch_sweep_kernel(k, src, dst, r, mw, flags, s), "stencil launch");
+  auto sweep = [&](const void* src, void* dst, double* r, int flags, const int* guard = nullptr) {
+    return cuda_check(launch_sweep_kernel(k, src, dst, r, mw, flags, s, guard), "stencil launch");
   };
   auto check = [&]() {
-    return cuda_check(launch_until_check(slot, counter, resid, tol, max_sweeps, h_loop, h_odd, s), "check launch");
+    return cuda_check(launch_until_check(slot, counter, stop, resid, tol, max_sweeps, h_loop, s), "check launch");
   };
   // A: zero the slots and the counter, pre-pass, first sweep, check
   cudaGraph_t gA = nullptr;
@@ -128,27 +131,21 @@ static jacc_status build_until(const Kernel& k, void* u0, void* u1, int32_t max_
   if (!st) st = add_child(ug.graph, nullptr, gA, &nA);
   cudaGraphDestroy(gA);  // the child node holds a copy
   if (st) return st;
-  // WHILE: u1 -> u0, check, IF { u0 -> u1, check }
+  // WHILE: pairs of u1 -> u0, check, u0 -> u1, check.  Small fields take 16
+  // sweeps per turn, fields whose sweeps dwarf a turn of the loop take 4.
   cudaGraph_t* wb = nullptr;
   st = add_conditional(ug.graph, nA, h_loop, cudaGraphCondTypeWhile, 1, &nW, &wb);
   if (st) return st;
-  cudaGraph_t gE = nullptr;
-  st = cuda_check(cudaGraphCreate(&gE, 0), "cudaGraphCreate");
-  if (st) return st;
-  st = capture_into(gE, s, [&]() -> jacc_status {
-    jacc_status e = sweep(cu1, u0, slot, 0);
-    return e ? e : check();
-  });
-  cudaGraphNode_t nE = nullptr, nI = nullptr;
-  if (!st) st = add_child(wb[0], nullptr, gE, &nE);
-  cudaGraphDestroy(gE);
-  if (st) return st;
-  cudaGraph_t* ib = nullptr;
-  st = add_conditional(wb[0], nE, h_odd, cudaGraphCondTypeIf, 1, &nI, &ib);
-  if (st) return st;
-  st = capture_into(ib[0], s, [&]() -> jacc_status {
-    jacc_status e = sweep(cu0, u1, slot, 0);
-    return e ? e : check();
+  const int pairs = k.desc.nx * k.desc.ny * k.desc.nz < (int64_t(1) << 22) ? 8 : 2;
+  st = capture_into(wb[0], s, [&]() -> jacc_status {
+    jacc_status e = ok();
+    for (int i = 0; i < pairs && !e; ++i) {
+      e = sweep(cu1, u0, slot, 0, stop);
+      if (!e) e = check();
+      if (!e) e = sweep(cu0, u1, slot, 0, stop);
+      if (!e) e = check();
+    }
+    return e;
   });
   if (st) return st;
   // F: status and the choice of the final sweep

@@ -8,18 +8,22 @@
 namespace {
 
 // After each sweep: move the sweep's residual from its accumulation slot to
-// resid[i], clear the slot for the next sweep, count the sweep, and set the
-// loop's conditions: continue while resid > tol and fewer than max sweeps ran.
-__global__ void jacc_k_until_check(double* slot, int* counter, double* resid, double tol, int max_sweeps,
-                                   cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_odd) {
-  const double r = *slot;
+// resid[i], clear the slot for the next sweep and count the sweep.  Once a
+// residual reaches the tolerance, or max sweeps ran, the stop word is set: the
+// sweeps and checks left in the loop's body then return at once, and the loop
+// ends.
+__global__ void jacc_k_until_check(double* slot, int* counter, int* stop, double* resid, double tol, int max_sweeps,
+                                   cudaGraphConditionalHandle h_loop) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (__ldcg(stop)) return;
+  const double r = __ldcg(slot);
   *slot = 0.0;
   const int i = *counter;
   resid[i] = r;
   *counter = i + 1;
-  const unsigned more = (r > tol && i + 1 < max_sweeps) ? 1u : 0u;
-  cudaGraphSetConditional(h_loop, more);
-  cudaGraphSetConditional(h_odd, more);
+  const bool more = r > tol && i + 1 < max_sweeps;
+  if (!more) *stop = 1;
+  cudaGraphSetConditional(h_loop, more ? 1u : 0u);
 }
 
 // After the loop: report the sweep count and the result buffer, and pick the
@@ -39,10 +43,18 @@ __global__ void jacc_k_until_final(const int* counter, int* status, int recomput
 
 namespace jacc {
 
-cudaError_t launch_until_check(double* slot, int* counter, double* resid, double tol, int max_sweeps,
-                               cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_odd, cudaStream_t s) {
-  jacc_k_until_check<<<1, 1, 0, s>>>(slot, counter, resid, tol, max_sweeps, h_loop, h_odd);
-  return cudaGetLastError();
+cudaError_t launch_until_check(double* slot, int* counter, int* stop, double* resid, double tol, int max_sweeps,
+                               cudaGraphConditionalHandle h_loop, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(1);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, jacc_k_until_check, slot, counter, stop, resid, tol, max_sweeps, h_loop);
 }
 
 cudaError_t launch_until_final(const int* counter, int* status, int recompute, cudaGraphConditionalHandle h_final,
