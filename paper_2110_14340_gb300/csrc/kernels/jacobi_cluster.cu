@@ -210,43 +210,81 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
   }
   const u32 pushes = ikind & 0xccccccccu;  // this thread's push bits
   int slot = 0;                            // wred slot of sweep k: k % 3
-  // Sweep k, the i-th of its chunk; `flush` ends the chunk: every CTA's maxima
-  // of the chunk are then in rres.  `last` writes the result.
+  // The end of a sweep, the i-th of its chunk, whose largest residual word of
+  // this thread is `word`; `flush` ends the chunk: every CTA's maxima of the
+  // chunk are then in rres.
+  auto finish = [&](u64 word, int i, bool flush) {
+    // One cluster barrier per sweep, split in two: its arrive releases this
+    // sweep's field writes (local and pushed), and the warp's residual
+    // maximum (the maximum magnitude in fixed point, or the bits of the
+    // non-negative maximum, which order alike) is reduced while the other
+    // CTAs arrive.  The per-warp partials of sweep k go to wred[k % 3]; they
+    // are read after the next sweep's barrier, whose arrive releases them,
+    // and the slot is next written two sweeps later, after warp 0 has
+    // arrived past its read.
+    cluster_arrive();
+    const u64 bits = warp_max_u64(word);
+    if ((t & 31) == 0) wred[slot][t >> 5] = bits;
+    cluster_wait();
+    const int prev = slot == 0 ? 2 : slot - 1;
+    // warp 0: this CTA's residual of sweep k - 1 (a flush took the last of a chunk)
+    if (t < 32 && i >= 1) {
+      u64 w = t < NT / 32 ? wred[prev][t] : 0ull;
+      w = warp_max_u64(w);
+      if (t == 0) rres[i - 1] = w;
+    }
+    if (flush) {
+      __syncthreads();  // this sweep's per-warp partials
+      if (t < 32) {
+        u64 w = t < NT / 32 ? wred[slot][t] : 0ull;
+        w = warp_max_u64(w);
+        if (t == 0) rres[i] = w;
+      }
+      cluster_sync();  // every CTA's maxima of this chunk are written
+    }
+    slot = slot == 2 ? 0 : slot + 1;
+  };
+  // Sweep k of hoisted items, and any other sweep (`last` writes the result).
+  // Two loops: the first one's body is all that a long sequence runs.
+  auto hot_sweep = [&](int k, int i, bool flush) {
+    const u64* src = (k & 1) ? bufB : bufA;
+    u64* dst = (k & 1) ? bufA : bufB;
+    // intermediate fixed-point sweeps: hoisted items, 16-byte shared-memory
+    // accesses, no per-sweep index arithmetic; then the edge rows (their
+    // values re-read from this thread's own stores) into the neighbours'
+    // halo rows
+    const u64 rmax_fx = fx_items(src, dst, pitch, ioff, ikind, fast, nit);
+    if (pushes) {
+#pragma unroll
+      for (int i = 0; i < kMaxItems; ++i) {
+        if (i >= nit) break;
+        const u32 kd = ikind >> (4 * i);
+        if (!(kd & 12u)) continue;
+        const longlong2 v = *reinterpret_cast<const longlong2*>(dst + ioff[i]);
+        if (kd & 4u) {  // first own row -> the previous CTA's lower halo row
+          const u32 ra = map_rank(dst + ioff[i] + rows * pitch, rank - 1);
+          st_cluster_u64(ra, (u64)v.x);
+          st_cluster_u64(ra + 8, (u64)v.y);
+        }
+        if (kd & 8u) {  // last own row -> the next CTA's upper halo row
+          const u32 ra = map_rank(dst + ioff[i] - nr * pitch, rank + 1);
+          st_cluster_u64(ra, (u64)v.x);
+          st_cluster_u64(ra + 8, (u64)v.y);
+        }
+      }
+    }
+    finish(rmax_fx, i, flush);
+  };
   auto sweep = [&](int k, int i, bool flush, bool last) {
     const u64* src = (k & 1) ? bufB : bufA;
     u64* dst = (k & 1) ? bufA : bufB;
     u64 rmax_fx = 0;
     double rmax_nat = 0.0;
-    int lr = 1 + t / half, cp = t % half;
-    if (fixed && !last && hoisted) {
-      // intermediate fixed-point sweeps: hoisted items, 16-byte shared-memory
-      // accesses, no per-sweep index arithmetic; then the edge rows (their
-      // values re-read from this thread's own stores) into the neighbours'
-      // halo rows
-      rmax_fx = fx_items(src, dst, pitch, ioff, ikind, fast, nit);
-      if (pushes) {
-#pragma unroll
-        for (int i = 0; i < kMaxItems; ++i) {
-          if (i >= nit) break;
-          const u32 kd = ikind >> (4 * i);
-          if (!(kd & 12u)) continue;
-          const longlong2 v = *reinterpret_cast<const longlong2*>(dst + ioff[i]);
-          if (kd & 4u) {  // first own row -> the previous CTA's lower halo row
-            const u32 ra = map_rank(dst + ioff[i] + rows * pitch, rank - 1);
-            st_cluster_u64(ra, (u64)v.x);
-            st_cluster_u64(ra + 8, (u64)v.y);
-          }
-          if (kd & 8u) {  // last own row -> the next CTA's upper halo row
-            const u32 ra = map_rank(dst + ioff[i] - nr * pitch, rank + 1);
-            st_cluster_u64(ra, (u64)v.x);
-            st_cluster_u64(ra + 8, (u64)v.y);
-          }
-        }
-      }
-    } else if (fixed && !last) {
+    if (fixed && !last) {
       // intermediate fixed-point sweeps: a column pair per item, 16-byte
       // shared-memory accesses (pitch is even, so every pair is aligned; an
       // odd nx pads each row by one word, which is written but never used)
+      int lr = 1 + t / half, cp = t % half;
       for (int it = t; it < nitems; it += NT) {
         const i64 x0 = 2 * (i64)cp;
         const i64 g = r0 - 1 + lr;
@@ -286,6 +324,7 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
         }
       }
     } else {
+      int lr = 1 + t / half, cp = t % half;
       for (int it = t; it < nitems; it += NT) {
         const i64 x0 = 2 * (i64)cp;
         const i64 g = r0 - 1 + lr;
@@ -346,35 +385,7 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
         }
       }
     }
-    // One cluster barrier per sweep, split in two: its arrive releases this
-    // sweep's field writes (local and pushed), and the warp's residual
-    // maximum (the maximum magnitude in fixed point, or the bits of the
-    // non-negative maximum, which order alike) is reduced while the other
-    // CTAs arrive.  The per-warp partials of sweep k go to wred[k % 3]; they
-    // are read after the next sweep's barrier, whose arrive releases them,
-    // and the slot is next written two sweeps later, after warp 0 has
-    // arrived past its read.
-    cluster_arrive();
-    const u64 bits = warp_max_u64(fixed ? rmax_fx : dbits(rmax_nat));
-    if ((t & 31) == 0) wred[slot][t >> 5] = bits;
-    cluster_wait();
-    const int prev = slot == 0 ? 2 : slot - 1;
-    // warp 0: this CTA's residual of sweep k - 1 (a flush took the last of a chunk)
-    if (t < 32 && i >= 1) {
-      u64 w = t < NT / 32 ? wred[prev][t] : 0ull;
-      w = warp_max_u64(w);
-      if (t == 0) rres[i - 1] = w;
-    }
-    if (flush) {
-      __syncthreads();  // this sweep's per-warp partials
-      if (t < 32) {
-        u64 w = t < NT / 32 ? wred[slot][t] : 0ull;
-        w = warp_max_u64(w);
-        if (t == 0) rres[i] = w;
-      }
-      cluster_sync();  // every CTA's maxima of this chunk are written
-    }
-    slot = slot == 2 ? 0 : slot + 1;
+    finish(fixed ? rmax_fx : dbits(rmax_nat), i, flush);
   };
   // The cluster's maximum of the chunk's i-th sweep (rres holds it in the form
   // it was reduced in, which orders alike; it is converted here, off the
@@ -390,12 +401,25 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
   // Residuals leave the cluster in chunks: a global write before a barrier
   // would make the barrier's release wait for it, so each sweep's CTA maxima
   // stay in shared memory until the chunk ends (plain stores, no atomics).
+  const bool hot = fixed && hoisted;
   if constexpr (!UNTIL) {
-    for (int base = 0; base < n; base += kResChunk) {
-      const int len = min(kResChunk, n - base);
-      for (int i = 0; i < len; ++i) sweep(base + i, i, i == len - 1, base + i == n - 1);
+    auto store = [&](int k, int i) {
       if (rank == 0 && a.resid)
-        for (int r = t; r < len; r += NT) a.resid[base + r] = resid_of(r);
+        for (int r = t; r <= i; r += NT) a.resid[k - i + r] = resid_of(r);
+    };
+    int k = 0;
+    if (hot)
+      for (; k < n - 1; ++k) {
+        const int i = k % kResChunk;
+        const bool flush = i == kResChunk - 1;
+        hot_sweep(k, i, flush);
+        if (flush) store(k, i);
+      }
+    for (; k < n; ++k) {
+      const int i = k % kResChunk;
+      const bool last = k == n - 1, flush = i == kResChunk - 1 || last;
+      sweep(k, i, flush, last);
+      if (flush) store(k, i);
     }
   } else {
     __shared__ int s_stop;
@@ -406,7 +430,10 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
       if (base)  // the chunk's start (the first one's is the input)
         for (i64 lr = 1; lr <= nr; ++lr)
           for (i64 x = t; x < nx; x += NT) a.keep[(r0 - 1 + lr) * nx + x] = __longlong_as_double((i64)cur[lr * pitch + x]);
-      for (int i = 0; i < len; ++i) sweep(base + i, i, i == len - 1, false);
+      if (hot)
+        for (int i = 0; i < len; ++i) hot_sweep(base + i, i, i == len - 1);
+      else
+        for (int i = 0; i < len; ++i) sweep(base + i, i, i == len - 1, false);
       if (t == 0) s_stop = len;
       __syncthreads();
       if (t < len) {
@@ -434,7 +461,10 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
           }
         }
         cluster_sync();
-        for (int k = base; k < n - 1; ++k) sweep(k, 0, false, false);
+        if (hot)
+          for (int k = base; k < n - 1; ++k) hot_sweep(k, 0, false);
+        else
+          for (int k = base; k < n - 1; ++k) sweep(k, 0, false, false);
       }
       a.res = (n & 1) ? a.keep : a.u_out;
       a.oth = (n & 1) ? a.u_out : a.keep;
