@@ -60,6 +60,7 @@ struct Kernel {
   cudaLibrary_t lib = nullptr;  // NVRTC module, if jit
   dim3 grid, block;
   dim3 grid_out, block_out;     // geometry of func_out and func_last
+  int zc_out = 0;               // their JParams::zc
   int fam = 0;                  // JACC_FAM_*
   int smem = 0;                 // dynamic shared memory per CTA of `func`
   int tblock = 1;

@@ -316,6 +316,38 @@ static int fitted_chunk(const Kernel& k, int zc) {
   const int least = k.desc.stencil == 7 || n <= (int64_t(1) << (k.desc.dtype == 64 ? 20 : 19)) ? 4 : 8;
   return static_cast<int>(fit >= zc ? zc : (fit < least ? least : fit));
 }
+// Planes per CTA of the converting 3D kernel (single launches, the first and
+// last sweep of a sequence) under the same condition.  It is bound by its
+// integer work, its CTAs take equally long and few waves of them run, so the
+// waves are filled: the chunk with the least waves * (planes + 3 to start up),
+// between 4 and 32 planes (256^3 heat, one launch: 145 us at 24 planes, 1.85
+// waves; 165 at 14, 3.2 waves; 163 at 32, 1.35; 301 x 253 x 199: 153 at 24,
+// 174 at 14 and at 32).
+static int fitted_chunk_out(const Kernel& k, int zc) {
+  int dev = 0, nsm = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k.func_out, static_cast<int>(k.block_out.x * k.block_out.y), 0) !=
+          cudaSuccess ||
+      per < 1) {
+    cudaGetLastError();
+    return zc;
+  }
+  const int64_t columns = static_cast<int64_t>(k.grid_out.x) * k.grid_out.y, slots = static_cast<int64_t>(nsm) * per;
+  int64_t least = INT64_MAX;
+  int best = zc;
+  for (int z = 32; z >= 4; --z) {
+    const int64_t chunks = (k.desc.nz + z - 1) / z;
+    if (chunks > 65535) break;
+    const int64_t cost = (columns * chunks + slots - 1) / slots * (z + 3);
+    if (cost < least) {
+      least = cost;
+      best = z;
+    }
+  }
+  return best;
+}
+
 
 // Planes per CTA of a 3D kernel.  The constant-folded variants of the bulk-copy
 // staged tiles with the long march take fewer planes than the table's 64: with
@@ -483,7 +515,8 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
     if (desc->stencil == 5)
       while ((desc->ny + c.by * p.zc - 1) / (c.by * p.zc) > 65535) p.zc *= 2;  // the grid's limit
   }
-  k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, p.zc));
+  k->zc_out = fit && edge && k->func_out && desc->stencil != 5 ? fitted_chunk_out(*k, p.zc) : p.zc;
+  k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, k->zc_out));
   k->grid = cta_grid(*desc, cta_tile(*desc, tile, fam, false, p.zc));
   if (desc->stencil == 19) {
     var19_geometry(desc->nx, desc->ny, desc->nz, &k->grid, &k->block);
@@ -632,6 +665,7 @@ cudaError_t launch_sweep_kernel(const Kernel& k, const void* u, void* v, double*
   // previous grid before it touches a field
   cudaLaunchConfig_t cfg = {};
   const bool edge = (flags & (kFxIn | kFxOut)) != 0;
+  if (edge) p.zc = k.zc_out;
   cfg.gridDim = edge ? k.grid_out : k.grid;
   cfg.blockDim = edge ? k.block_out : k.block;
   cfg.dynamicSmemBytes = static_cast<size_t>(k.smem);

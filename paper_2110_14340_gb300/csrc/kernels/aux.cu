@@ -14,7 +14,7 @@ cudaError_t launch_maxabs(const double* u, long long n, u64* maxword, cudaStream
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     nsm = 152;
   long long pairs = n / 2;
-  long long blocks = (pairs + 255) / 256;
+  long long blocks = (pairs + 1023) / 1024;  // 1024 pairs at a time
   if (blocks < 1) blocks = 1;
   if (blocks > 8ll * nsm) blocks = 8ll * nsm;
   jacc_k_maxabs<<<(unsigned)blocks, 256, 0, s>>>(u, n, maxword);

@@ -96,23 +96,21 @@ JD s128 from_s64_shl(i64 a, int k) {  // a * 2^k, 0 <= k < 64
   r.hi = (k == 0) ? (u64)(a >> 63) : (u64)(a >> (64 - k));
   return r;
 }
-// (x.hi:x.lo) * 2^-E rounded to nearest even.
+// (x.hi:x.lo) * 2^-E rounded to nearest even, by selections only: the
+// magnitude's top 63 significant bits, the last one set when any bit below it
+// was, then the rounding of fx_to.
 JD double fx128_to(s128 x, int E) {
-  u64 s = x.hi >> 63;
-  u64 lo = x.lo, hi = x.hi;
-  if (s) { lo = ~lo + 1ull; hi = ~hi + (u64)(lo == 0ull); }
-  int lz = hi ? __clzll((i64)hi) : 64 + __clzll((i64)lo);
-  u64 nh, nl;
-  if (lz >= 64) { nh = lo << (lz - 64); nl = 0ull; }
-  else if (lz == 0) { nh = hi; nl = lo; }
-  else { nh = (hi << lz) | (lo >> (64 - lz)); nl = lo << lz; }
-  u64 mant = nh >> 11;
-  u64 rem = nh & 0x7ffull;
-  u64 sticky = (u64)(nl != 0ull);
-  mant += (u64)((rem > 0x400ull) | ((rem == 0x400ull) & ((mant & 1ull) | sticky)));
-  i64 eb = 127 - lz - E + 1023;
-  u64 bits = (s << 63) | (((u64)(eb - 1) << 52) + mant);
-  return (lo | hi) ? __longlong_as_double((i64)bits) : 0.0;
+  const u64 s = (u64)((i64)x.hi >> 63);
+  const u64 lo = (x.lo ^ s) - s;
+  const u64 hi = (x.hi ^ s) + (u64)(s != 0ull && lo == 0ull);
+  const bool low = hi == 0ull;
+  const u64 h = low ? lo : hi, l = low ? 0ull : lo;
+  const int lz = __clzll((i64)h) & 63;
+  const u64 m = (h << lz) | ((l >> 1) >> (63 - lz));
+  const u64 n = (m >> 1) | (m & 1ull) | (u64)((l << lz) != 0ull);
+  const u64 mant = (n + 0x1ffull + ((n >> 10) & 1ull)) >> 10;
+  const u64 bits = mant + ((u64)(u32)(((low ? 63 : 127) - lz - E + 1022) << 20) << 32);
+  return h ? __longlong_as_double((i64)(bits | (s & 0x8000000000000000ull))) : 0.0;
 }
 
 // ---------------------------------------------------------------- load / store helpers
@@ -1448,6 +1446,28 @@ JD i64 heat_increment(i64 L, u64 fm) {
   return (i64)(((hi << 2) | ((u32)mid >> 30)) - fm);
 }
 
+// The same increment, and in `out` the FP64 value of the exact u + r L, which
+// is ce 2^62 + L fm at scale F + 62 (below 2^119): all 128 bits of the product
+// are kept, so the increment and the output share it.
+JD i64 heat_increment_out(i64 L, u64 fm, i64 ce, int F, double& out) {
+  const u64 b = (u64)L + (1ull << 62);
+  const u32 bl = (u32)b, bh = (u32)(b >> 32), ml = (u32)fm, mh = (u32)(fm >> 32);
+  const u64 p0 = (u64)bl * ml;
+  u64 mid = (u64)bl * mh + (p0 >> 32);
+  mid = (u64)bh * ml + mid;
+  s128 x;
+  x.hi = (u64)bh * mh + (mid >> 32);
+  x.lo = (mid << 32) | (u32)p0;
+  const i64 d = (i64)((((x.hi << 3) | (x.lo >> 61)) + 1) >> 1) - (i64)fm;
+  const i64 c = ce - (i64)fm;
+  s128 h;
+  h.lo = (u64)c << 62;
+  h.hi = (u64)(c >> 2);
+  x = add128(x, h);
+  out = fx128_to(x, F + 62);
+  return d;
+}
+
 // ---------------------------------------------------------------- 7-point heat, bulk-copy staged planes
 //
 // Same staging as the 27-point kernel (bulk copies on full/empty mbarriers,
@@ -1925,38 +1945,44 @@ JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int 
     row(c0 + RY * G::W, yp);
     T out[RY][V];
     Wt dv[RY * V];
+    // f(sum of the six faces, centre, increment, output) for every point
+    auto each = [&](auto f) {
 #pragma unroll
-    for (int k = 0; k < RY; ++k) {
-      const Wt xl = c0[k * G::W - 1], xr = c0[k * G::W + V];
+      for (int k = 0; k < RY; ++k) {
+        const Wt xl = c0[k * G::W - 1], xr = c0[k * G::W + V];
 #pragma unroll
-      for (int e = 0; e < V; ++e) {
-        const Wt a = e == 0 ? xl : cur[k][e == 0 ? 0 : e - 1], b = e == V - 1 ? xr : cur[k][e == V - 1 ? e : e + 1];
-        const Wt c = k == 0 ? ym[e] : cur[k == 0 ? 0 : k - 1][e], d = k == RY - 1 ? yp[e] : cur[k == RY - 1 ? k : k + 1][e];
-        const Wt sum = ((a + b) + (c + d)) + (zp[k][e] + zn[k][e]);
-        const Wt ce = cur[k][e];
-        Wt& dk = dv[k * V + e];
-        if constexpr (FX) {
-          if (fold) {
-            const i64 vn = (fb * sum + ((((i64)1 << fk) - 6 * fb) * ce + ((i64)1 << (fk - 1)))) >> fk;
-            dk = vn - ce;
-            out[k][e] = i64_bits(vn);
-          } else {
-            dk = heat_increment(sum - 6 * ce, p.fm);
-            out[k][e] = i64_bits(ce + dk);
-          }
-          if constexpr (EDGE) {
-            if (outf) {  // the exact value, rounded once
-              const i64 Ld = sum - 6 * ce;
-              if (p.fpath == JACC_FP_SMALL) out[k][e] = fx_to(ce * ((i64)1 << fk) + fb * Ld, F + fk);
-              else out[k][e] = fx128_to(add128(from_s64_shl(ce, fk), mul_s64_u64(Ld, (u64)p.fw0)), F + fk);
-            }
-          }
-        } else {
-          const T o = ce + r * (sum - T(6) * ce);
-          out[k][e] = o;
-          dk = o - ce;
+        for (int e = 0; e < V; ++e) {
+          const Wt a = e == 0 ? xl : cur[k][e == 0 ? 0 : e - 1], b = e == V - 1 ? xr : cur[k][e == V - 1 ? e : e + 1];
+          const Wt c = k == 0 ? ym[e] : cur[k == 0 ? 0 : k - 1][e], d = k == RY - 1 ? yp[e] : cur[k == RY - 1 ? k : k + 1][e];
+          f(((a + b) + (c + d)) + (zp[k][e] + zn[k][e]), cur[k][e], dv[k * V + e], out[k][e]);
         }
       }
+    };
+    if constexpr (!FX) {
+      each([&](T sum, T ce, T& dk, T& o) {
+        o = ce + r * (sum - T(6) * ce);
+        dk = o - ce;
+      });
+    } else if (EDGE && outf) {  // the exact value, rounded once
+      if (p.fpath == JACC_FP_SMALL)
+        each([&](i64 sum, i64 ce, i64& dk, T& o) {
+          const i64 w = fb * (sum - 6 * ce);
+          dk = (w + (((i64)1 << fk) >> 1)) >> fk;
+          o = fx_to(ce * ((i64)1 << fk) + w, F + fk);
+        });
+      else
+        each([&](i64 sum, i64 ce, i64& dk, T& o) { dk = heat_increment_out(sum - 6 * ce, p.fm, ce, F, o); });
+    } else if (fold) {
+      each([&](i64 sum, i64 ce, i64& dk, T& o) {
+        const i64 vn = (fb * sum + ((((i64)1 << fk) - 6 * fb) * ce + ((i64)1 << (fk - 1)))) >> fk;
+        dk = vn - ce;
+        o = i64_bits(vn);
+      });
+    } else {
+      each([&](i64 sum, i64 ce, i64& dk, T& o) {
+        dk = heat_increment(sum - 6 * ce, p.fm);
+        o = i64_bits(ce + dk);
+      });
     }
     if (!fast) {
 #pragma unroll
@@ -2445,41 +2471,43 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
 }
 
 #ifdef JACC_AUX_KERNELS
-// Pre-pass: atomicMax of the bit pattern of |u[i]| over n doubles.
-// Any NaN orders above +Inf, so a NaN input selects the native path.
+// Pre-pass: atomicMax over n doubles of the high word of |u[i]|, its last bit
+// set where the low word is not zero (so only zeros give zero).  Of the
+// maximum the scale takes the exponent alone: NaN and infinities select the
+// native path, as does a field of subnormals.  Three 32-bit operations a value
+// instead of a 64-bit mask, comparison and two selections leave the loads as
+// the bound: four of 16 bytes in flight in each of a full SM's threads.
 __global__ void __launch_bounds__(256, 8) jacc_k_maxabs(const double* __restrict__ u, i64 n, u64* maxword) {
   griddep_wait();
-  u64 m = 0;
-  const i64 stride = (i64)gridDim.x * blockDim.x;
+  u32 m = 0;
   const i64 n2 = n / 2;
-  const double2* u2 = reinterpret_cast<const double2*>(u);
-  auto take = [&](double2 t) {
-    const u64 a = dbits(t.x) & 0x7fffffffffffffffull, c = dbits(t.y) & 0x7fffffffffffffffull;
-    m = a > m ? a : m;
-    m = c > m ? c : m;
-  };
-  i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-  // four independent 16-byte loads in flight per thread (one resident wave)
-  for (; i + 3 * stride < n2; i += 4 * stride) {
-    double2 t[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) t[q] = __ldg(u2 + i + q * stride);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) take(t[q]);
+  const uint4* u2 = reinterpret_cast<const uint4*>(u);
+  auto word = [](u32 hi, u32 lo) { return (hi & 0x7fffffffu) | min(lo, 1u); };
+  auto take = [&](uint4 t) { m = max(max(m, word(t.y, t.x)), word(t.w, t.z)); };
+  // a block takes 1024 consecutive words of 16 bytes at a time
+  const i64 full = n2 / 1024;
+#pragma unroll 1
+  for (i64 b = blockIdx.x; b < full; b += gridDim.x) {
+    const uint4* q = u2 + b * 1024 + threadIdx.x;
+    const uint4 t0 = __ldg(q), t1 = __ldg(q + 256), t2 = __ldg(q + 512), t3 = __ldg(q + 768);
+    take(t0);
+    take(t1);
+    take(t2);
+    take(t3);
   }
-  for (; i < n2; i += stride) take(__ldg(u2 + i));
+  if (blockIdx.x == full % gridDim.x)
+    for (i64 i = full * 1024 + threadIdx.x; i < n2; i += blockDim.x) take(__ldg(u2 + i));
   if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-    u64 a = dbits(u[n - 1]) & 0x7fffffffffffffffull;
-    m = a > m ? a : m;
+    const u64 a = dbits(u[n - 1]);
+    m = max(m, word((u32)(a >> 32), (u32)a));
   }
-  m = warp_max_u64(m);
-  __shared__ u64 red[8];
+  m = __reduce_max_sync(0xffffffffu, m);
+  __shared__ u32 red[8];
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x < 32) {
-    u64 w = threadIdx.x < 8 ? red[threadIdx.x] : 0ull;
-    w = warp_max_u64(w);
-    if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long*>(maxword), (unsigned long long)w);
+    const u32 w = __reduce_max_sync(0xffffffffu, threadIdx.x < 8 ? red[threadIdx.x] : 0u);
+    if (threadIdx.x == 0) atomicMax(reinterpret_cast<unsigned long long*>(maxword), (unsigned long long)w << 32);
   }
 }
 
