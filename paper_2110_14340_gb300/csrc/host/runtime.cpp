@@ -246,8 +246,9 @@ static CtaTile cta_tile(const jacc_kernel_desc& d, int tile, int fam, bool edge,
   const TileCfg& c = kTiles[tile];
   const int V = c.vec16 ? (d.dtype == 64 ? 2 : 4) : 1;
   if (d.stencil == 5)
-    return fam == JACC_FAM_STRIP || V == 1 ? CtaTile{static_cast<int64_t>(c.bx / 32) * 30 * V, c.by, zc}
-                                 : CtaTile{static_cast<int64_t>(c.bx) * V, c.by, zc};
+    return fam == JACC_FAM_STRIP || V == 1 || ((d.flags & JACC_SPEC_JIT) && d.nx * d.ny <= JACC_SMALL_GRID)
+               ? CtaTile{static_cast<int64_t>(c.bx / 32) * 30 * V, c.by, zc}
+               : CtaTile{static_cast<int64_t>(c.bx) * V, c.by, zc};
   const bool f64 = d.dtype == 64;
   if (d.stencil == 7 && !edge && (fam == JACC_FAM_DIRECT || (fam == JACC_FAM_TABLE && JACC_DIRECT_TILE(c.bx, c.by, V))))
     return CtaTile{static_cast<int64_t>(32) * V, 8, JACC_DIRECT_PLANES};

@@ -2312,6 +2312,12 @@ JD void heat3d_direct(const T* __restrict__ u, T* __restrict__ v, const P& p, R&
 // that the autotuner times for it; the library's own choice (no tile asked
 // for, none remembered) may also take the strip march, the asynchronous-copy
 // ring, or no staging at all.
+// A folded grid of at most JACC_SMALL_GRID points takes the strip march also
+// where a tile with 16-byte columns was asked for: its few rows in flight are
+// latency-bound there (256 x 256 FP64, tile 1: 2.2 us a sweep, 3.0 by rows; at
+// 4096 x 4096 52 and 50).
+template <class P> struct SmallFold { static constexpr bool value = P::nx * P::ny <= JACC_SMALL_GRID; };
+template <> struct SmallFold<JParams> { static constexpr bool value = false; };
 template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                        const u64* maxword, int flags) {
@@ -2320,7 +2326,8 @@ JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, c
   u64 bits = 0;
   const i64 ys = ((i64)blockIdx.y * BY + threadIdx.y) * p.zc;
   const i64 ye = (ys + p.zc < p.ny) ? ys + p.zc : p.ny;
-  constexpr bool STRIP = FAM == JACC_FAM_STRIP || V == 1;  // the table tiles of scalar columns, too
+  // scalar columns and small folded grids march strips whatever the tile
+  constexpr bool STRIP = FAM == JACC_FAM_STRIP || V == 1 || SmallFold<P>::value;
   // STRIP: BX / 32 strips of 30 V columns across the CTA
   const i64 strip = (i64)blockIdx.x * (BX / 32) + (threadIdx.x >> 5);
   const i64 xl = STRIP ? strip * (30 * V) + ((int)(threadIdx.x & 31) - 1) * V : (i64)blockIdx.x * (BX * V) + (i64)threadIdx.x * V;

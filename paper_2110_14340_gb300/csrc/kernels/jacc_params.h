@@ -25,6 +25,9 @@ typedef unsigned int u32;
 #define JACC_DIRECT_TILE(bx, by, vec) ((bx) == 32 && (by) == 8 && (vec) == 1)
 #define JACC_DIRECT_PLANES 2
 
+// Points up to which a folded 5-point kernel marches strips whatever its tile.
+#define JACC_SMALL_GRID (1 << 17)
+
 // Rows per thread of the kernels that stage planes by asynchronous copies
 // (bx x by threads, one column each): 4, or 2 where 4 would not leave room
 // for the stages.
