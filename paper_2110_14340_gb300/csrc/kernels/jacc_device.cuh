@@ -1305,18 +1305,19 @@ template <int N> JD void fx_residual(const i64 (&d)[N], u64& rmax) {
 // lanes 0 and 31 hold the columns left and right of the strip, so every x
 // neighbour comes from a shuffle, with no extra loads or selects, at the
 // price of 2/30 more loads and sums (L2 serves the shared columns).  Rows
-// y-1, y, y+1 stay in registers and the raw rows y+2 .. y+4 are in flight;
-// three rows per iteration rotate all of them without copies.  A warp whose
+// y-1, y, y+1 stay in registers and the raw rows y+2 .. y+1+D are in flight;
+// D rows per iteration rotate all of them without copies.  A warp whose
 // columns are all interior runs without selects.  4096^2 FP64, 50 sweeps:
 // 3.52 ms with the row march of the table's vector tiles (82 thread-
-// instructions a point, an edge column loaded where it is used), 2.57 here (58;
-// 5.2 TB/s), bound by integer issue and the latency of 24 warps an SM.
+// instructions a point, an edge column loaded where it is used), 2.43 here
+// (5.6 TB/s; 2.55 with 64-bit row offsets multiplied out for every row, 80
+// registers instead of 66), bound by the latency of the warps an SM holds.
 //
 // xl: the lane's first column (may lie outside the grid).  FX: resident
 // 64-bit fixed point, v 2^F = (S + 2) >> 2 with S the four neighbours, the
 // FP64 output fx_to(S, F + 2), the residual |S - 4u| (EDGE: conversions, see
 // JFX_*); otherwise native arithmetic on T.  All lanes of a warp share ys, ye.
-template <class T, int V, bool FX, bool EDGE>
+template <class T, int V, bool FX, bool EDGE, int D>
 JD void jacobi_strip(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 ny, i64 xl, i64 ys, i64 ye, int F,
                      int flags, typename RT<T, FX ? JM_FIXED : JM_NATIVE>::type& rmax) {
   typedef typename WT<T, FX ? JM_FIXED : JM_NATIVE>::type W;
@@ -1339,15 +1340,19 @@ JD void jacobi_strip(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 ny,
   };
   const T* src = u + ys * nx + xl;  // row ys of the lane's columns
   T* dst = v + ys * nx + xl;
-  const i64 rows = ye - ys;
+  // row counts relative to ys fit 32 bits; the pointers advance row by row
+  const int rows = (int)(ye - ys);
   // last row needed: ye, if it is in the grid
-  const i64 rlast = (ye < ny ? ye : ny - 1) - ys;
-  auto load = [&](i64 r, T (&q)[V]) {  // row ys + r
+  const int rlast = xin ? (int)((ye < ny ? ye : ny - 1) - ys) : -1;
+  const int jlo = ys < 1 ? 1 : 0, jhi = (int)(ny - 2 - ys < rows ? ny - 2 - ys : rows);  // interior rows
+  const T* ln = src;  // next row to load
+  auto load = [&](int r, T (&q)[V]) {  // row ys + r, in order
 #pragma unroll
     for (int e = 0; e < V; ++e) q[e] = T(0);
-    if (xin && r <= rlast) ldv<T, V>(src + r * nx, q);
+    if (r <= rlast) ldv<T, V>(ln, q);
+    ln += nx;
   };
-  T q[3][V];
+  T q[D][V];
   W w[3][V];
   {
     T t[V];
@@ -1361,13 +1366,12 @@ JD void jacobi_strip(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 ny,
       w[1][e] = cvt(q[0][e]);
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) load(1 + k, q[k]);
+    for (int k = 0; k < D; ++k) load(1 + k, q[k]);
   }
-  auto step = [&](i64 j, const W (&up)[V], const W (&cur)[V], W (&dn)[V], T (&qn)[V]) {
-    const i64 y = ys + j;
+  auto step = [&](int j, const W (&up)[V], const W (&cur)[V], W (&dn)[V], T (&qn)[V]) {
 #pragma unroll
     for (int e = 0; e < V; ++e) dn[e] = cvt(qn[e]);
-    load(j + 4, qn);
+    load(j + 1 + D, qn);
     const W left = __shfl_up_sync(0xffffffffu, cur[V - 1], 1);
     const W right = __shfl_down_sync(0xffffffffu, cur[0], 1);
     T out[V];
@@ -1385,14 +1389,14 @@ JD void jacobi_strip(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 ny,
         d[e] = out[e] - cur[e];
       }
     }
-    const bool yint = y >= 1 && y <= ny - 2;
+    const bool yint = j >= jlo && j <= jhi;
     if (!(fast && yint)) {
 #pragma unroll
       for (int e = 0; e < V; ++e)
         if (!(yint && cint[e])) {
           d[e] = W(0);
           if constexpr (FX) {
-            if (EDGE && outf) out[e] = inf ? (wr ? src[j * nx + e] : T(0)) : fx_to(cur[e], F);
+            if (EDGE && outf) out[e] = inf ? (wr ? src[(i64)j * nx + e] : T(0)) : fx_to(cur[e], F);
             else out[e] = i64_bits(cur[e]);
           } else {
             out[e] = cur[e];
@@ -1408,17 +1412,18 @@ JD void jacobi_strip(const T* __restrict__ u, T* __restrict__ v, i64 nx, i64 ny,
         rmax = m > rmax ? m : rmax;
       }
     }
-    if (wr) stv<T, V>(dst + j * nx, out);
+    if (wr) stv<T, V>(dst, out);
+    dst += nx;
   };
-  i64 j = 0;
+  int j = 0;
 #pragma unroll 1
-  for (; j + 3 <= rows; j += 3) {
-    step(j, w[0], w[1], w[2], q[0]);
-    step(j + 1, w[1], w[2], w[0], q[1]);
-    step(j + 2, w[2], w[0], w[1], q[2]);
+  for (; j + D <= rows; j += D) {
+#pragma unroll
+    for (int i = 0; i < D; ++i) step(j + i, w[i % 3], w[(i + 1) % 3], w[(i + 2) % 3], q[i]);
   }
-  if (j < rows) step(j, w[0], w[1], w[2], q[0]);
-  if (j + 1 < rows) step(j + 1, w[1], w[2], w[0], q[1]);
+#pragma unroll
+  for (int i = 0; i < D - 1; ++i)
+    if (j + i < rows) step(j + i, w[i % 3], w[(i + 1) % 3], w[(i + 2) % 3], q[i]);
   if (lane == 0 || lane == 31) rmax = 0;  // their sums lack a neighbour
 }
 
@@ -2318,6 +2323,11 @@ JD void heat3d_direct(const T* __restrict__ u, T* __restrict__ v, const P& p, R&
 // 4096 x 4096 52 and 50).
 template <class P> struct SmallFold { static constexpr bool value = P::nx * P::ny <= JACC_SMALL_GRID; };
 template <> struct SmallFold<JParams> { static constexpr bool value = false; };
+// A folded FP64 grid of more than JACC_LARGE_GRID points, which streams from
+// HBM, has six rows in flight instead of three and marches twice the rows
+// (4096^2 44.7 us a sweep against 47.6; FP32 21.7 against 20.1).
+template <class P> struct LargeFold { static constexpr bool value = P::nx * P::ny > JACC_LARGE_GRID; };
+template <> struct LargeFold<JParams> { static constexpr bool value = false; };
 template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                        const u64* maxword, int flags) {
@@ -2328,6 +2338,7 @@ JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, c
   const i64 ye = (ys + p.zc < p.ny) ? ys + p.zc : p.ny;
   // scalar columns and small folded grids march strips whatever the tile
   constexpr bool STRIP = FAM == JACC_FAM_STRIP || V == 1 || SmallFold<P>::value;
+  constexpr int DEPTH = !EDGE && V == 2 && LargeFold<P>::value ? 6 : 3;
   // STRIP: BX / 32 strips of 30 V columns across the CTA
   const i64 strip = (i64)blockIdx.x * (BX / 32) + (threadIdx.x >> 5);
   const i64 xl = STRIP ? strip * (30 * V) + ((int)(threadIdx.x & 31) - 1) * V : (i64)blockIdx.x * (BX * V) + (i64)threadIdx.x * V;
@@ -2336,7 +2347,7 @@ JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, c
     if constexpr (sizeof(T) == 8) {
       u64 m = 0;
       if (ys < p.ny) {
-        if constexpr (STRIP) jacobi_strip<double, V, true, EDGE>(u, v, p.nx, p.ny, xl, ys, ye, F, flags, m);
+        if constexpr (STRIP) jacobi_strip<double, V, true, EDGE, DEPTH>(u, v, p.nx, p.ny, xl, ys, ye, F, flags, m);
         else jacobi_fx_march<V, false, EDGE>(u, v, p.nx, p.ny, xl, ys, ye, F, flags, m);
       }
       bits = dbits(fx_to_u(m, F + 2));
@@ -2344,7 +2355,7 @@ JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, c
   } else {
     T m = T(0);
     if (ys < p.ny) {
-      if constexpr (STRIP) jacobi_strip<T, V, false, false>(u, v, p.nx, p.ny, xl, ys, ye, -1, 0, m);
+      if constexpr (STRIP) jacobi_strip<T, V, false, false, DEPTH>(u, v, p.nx, p.ny, xl, ys, ye, -1, 0, m);
       else jacobi_march<T, V, JM_NATIVE, false>(u, v, p.nx, p.ny, xl, ys, ye, -1, m);
     }
     bits = dbits((double)m);

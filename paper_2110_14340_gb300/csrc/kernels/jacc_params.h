@@ -27,6 +27,8 @@ typedef unsigned int u32;
 
 // Points up to which a folded 5-point kernel marches strips whatever its tile.
 #define JACC_SMALL_GRID (1 << 17)
+// Points above which an FP64 one has six rows in flight.
+#define JACC_LARGE_GRID (1 << 23)
 
 // Rows per thread of the kernels that stage planes by asynchronous copies
 // (bx x by threads, one column each): 4, or 2 where 4 would not leave room

@@ -3,7 +3,8 @@
 // tile_id = 4 * shape + 2 * long_march + vec:
 //   shape (threads bx x by): 32x4, 32x8, 64x4, 64x8, 128x2, 128x4
 //   long_march: 0 -> zc = 16, 1 -> zc = 64   (planes per CTA in 3D;
-//               2D kernels march zc / 4 rows per thread)
+//               2D kernels march zc / 4 rows per thread; a kernel whose tile the
+//               library chose marches what fits the GPU)
 //   vec:        0 -> one element per thread in x, 1 -> a 16-byte vector
 //               (2 doubles or 4 floats)
 #pragma once
