@@ -465,6 +465,14 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
     tile = 3;  // the kernel's one configuration: 32 x 4 threads, 16-byte columns, 40-plane march
   } else if (tile < 0) {
     tile = tuned_tile(*desc);
+    // Picks are timed on precompiled kernels, where the 32 x 4 scalar tile's
+    // asynchronous copies beat the bulk copies of the same tile with 16-byte
+    // columns; folded, the order is the other way round for fields that stream
+    // from HBM (512^3 FP64, us a sweep, scalar and 16-byte: precompiled 385 and
+    // 413, folded 380 and 355).
+    if (tile >= 0 && (desc->flags & JACC_SPEC_JIT) && desc->stencil == 7 && desc->dtype == 64 && kTiles[tile].bx == 32 &&
+        kTiles[tile].by == 4 && desc->nx * desc->ny * desc->nz >= (int64_t(1) << 25) && tile_valid(*desc, tile | 1))
+      tile |= 1;
     if (tile < 0 || !tile_valid(*desc, tile)) {
       tile = default_tile(*desc);
       fit = desc->stencil != 19 && desc->tblock <= 1;
