@@ -42,8 +42,26 @@ def test_jacobi2d_f64_folded_strips_equal_integer_arithmetic(nx, tile):
     check_jacobi2d_f64(nx, 11, tile, True)
 
 
-def check_jacobi2d_f64(nx, ny, tile, jit):
+# the pre-pass reads 2048 values at a time: the largest on both sides of a block's end
+@pytest.mark.parametrize("nx,ny", [(23, 89), (512, 4), (683, 3), (64, 64), (241, 17)])
+@pytest.mark.parametrize("at", [0, 2047, -1])
+def test_fixed_point_scale_follows_the_largest_value_wherever_it_is(nx, ny, at):
+    check_jacobi2d_f64(nx, ny, -1, False, spike=min(at, nx * ny - 1))
+
+
+def test_a_field_of_subnormals_takes_native_arithmetic():
+    u = np.zeros((9, 62))
+    u[4, 30] = 5e-324
+    u[5, 31] = 4e-310
+    g, _, gr = run(jacc.Kernel(jacc.STENCIL_5PT, jacc.F64, 62, 9, 1), u, 2)
+    t, _, tr = run(jacc.Kernel(jacc.STENCIL_5PT, jacc.F64, 62, 9, 1, arith=jacc.ARITH_NATIVE), u, 2)
+    assert np.array_equal(g, t) and np.array_equal(gr, tr)
+
+
+def check_jacobi2d_f64(nx, ny, tile, jit, spike=None):
     u = 2.0 * inputs.uniform64(41, nx * ny).reshape(ny, nx) - 1.0
+    if spike is not None:
+        u.ravel()[spike] = -1000.0
     F = 57 - math.frexp(float(np.max(np.abs(u))))[1]
     k = jacc.Kernel(jacc.STENCIL_5PT, jacc.F64, nx, ny, 1, tile_id=tile, jit=jit)
     assert k.info()["fixed_point"]
@@ -111,6 +129,31 @@ def test_f64_choice_takes_native_arithmetic_for_non_finite_fields(stencil, shape
     t, _, tr = run(jacc.Kernel(stencil, jacc.F64, nx, ny, nz, coeffs=coeffs, arith=jacc.ARITH_NATIVE), u, 2)
     assert np.array_equal(g, t, equal_nan=True)
     assert np.array_equal(gr, tr, equal_nan=True)
+
+
+# a folded grid that streams from HBM has more rows in flight and per warp
+def test_jacobi2d_f64_large_folded_strips_equal_the_precompiled_kernel():
+    nx, ny = 4098, 2051
+    assert nx * ny > 1 << 23
+    u = 2.0 * inputs.uniform64(46, nx * ny).reshape(ny, nx) - 1.0
+    got = run(jacc.Kernel(jacc.STENCIL_5PT, jacc.F64, nx, ny, 1, jit=True), u, 3)
+    want = run(jacc.Kernel(jacc.STENCIL_5PT, jacc.F64, nx, ny, 1, tile_id=1), u, 3)
+    for g, w in zip(got, want):
+        assert np.array_equal(g.view(np.int64), w.view(np.int64))
+
+
+# the converting kernel has a plane count of its own where the library chooses
+@pytest.mark.parametrize("nx,ny,nz", [(130, 66, 70), (131, 67, 71), (256, 200, 131)])
+@pytest.mark.parametrize("stencil,coeffs", [(7, (0.125,)), (7, (0.1,)), (27, (0.5, 1 / 16, 1 / 128, 1 / 256))])
+def test_f64_single_launch_equals_table_tile(stencil, coeffs, nx, ny, nz):
+    u = 2.0 * inputs.uniform64(47, nx * ny * nz).reshape(nz, ny, nx) - 1.0
+    g, _, gr = run(jacc.Kernel(stencil, jacc.F64, nx, ny, nz, coeffs=coeffs), u, 1)
+    t, _, tr = run(jacc.Kernel(stencil, jacc.F64, nx, ny, nz, coeffs=coeffs, tile_id=0), u, 1)
+    assert np.array_equal(g, t)
+    if stencil == 7:
+        assert np.array_equal(gr, tr)
+    else:
+        assert np.max(np.abs(gr - tr)) <= 1e-12 * float(np.sum(np.abs(u)))
 
 
 def check_until(k, u, stops, most):
