@@ -204,15 +204,20 @@ jacc_status jacc_region_boxes_affine(int32_t nloops, const jacc_loop_affine* loo
  * dtype JACC_F32 stores and computes FP32 (arith is ignored).
  *
  * tile_id selects one of JACC_NUM_TILES tile configurations (see
- * jacc_tile_info), or -1 to let the library choose (the autotuner's cached
- * pick for this shape if one exists, else a default).
+ * jacc_tile_info), or -1 to let the library choose: the autotuner's cached
+ * pick for this shape if one exists (large 7PT FP64 grids with JACC_SPEC_JIT:
+ * with 16-byte columns where the pick has scalar ones), else a kernel of the library's own for
+ * this size, type and row alignment, which may load its input in another way
+ * than the tile that jacc_kernel_info names (strips of rows for 5PT, planes
+ * staged by asynchronous or bulk copies or not at all for 7PT and 27PT) and
+ * marches as many planes or rows per CTA as fill the GPU.
  *
  * flags: JACC_SPEC_JIT compiles a variant with the extents and coefficients
  * folded in as constants (NVRTC, sm_103a; cached in memory and, if the
- * environment variable JACC_CACHE_DIR names a directory, on disk); for the
- * 3D tiles with 16-byte columns and the long march it marches 40 planes per
- * CTA (27PT: 32) instead of the table's 64 (jacc_kernel_info reports the
- * grid).
+ * environment variable JACC_CACHE_DIR names a directory, on disk); where it
+ * stages planes by bulk copies, with the 16-byte columns and the long march of
+ * an explicit tile, it marches 40 planes per CTA (27PT: 32) instead of the
+ * table's 64 (jacc_kernel_info reports the grid).
  * Without it the handle uses a precompiled kernel that takes them as
  * arguments.
  * JACC_SPEC_CLUSTER (5PT FP64 only; no counterpart in the paper): jacc_sweep
@@ -276,9 +281,10 @@ jacc_status jacc_kernel_info(jacc_kernel k, jacc_kernel_info_t* out);
 jacc_status jacc_release(jacc_kernel k);
 
 /* Device status of a handle's launches (no counterpart in the paper).  The
- * 27PT FP32 kernels with 16-byte columns stage their input planes in shared
- * memory with bulk copies and wait for them on mbarriers; each such wait is
- * bounded (default 2 s).  A wait that runs out writes JACC_ERR_TIMEOUT to the
+ * 7PT and 27PT FP32 kernels of explicit tiles with 16-byte columns (and those
+ * that the library chooses for fields that stream from HBM) stage their input
+ * planes in shared memory with bulk copies and wait for them on mbarriers;
+ * each such wait is bounded (default 2 s).  Other kernels have no such waits.  A wait that runs out writes JACC_ERR_TIMEOUT to the
  * handle's device status word and its CTA returns early, so the output of
  * that launch is incomplete.  jacc_kernel_status synchronises the device,
  * stores the word (JACC_OK or JACC_ERR_TIMEOUT) in *status and clears it.
@@ -372,11 +378,14 @@ jacc_status jacc_sweep_coeffs(jacc_kernel k, void* u0, void* u1, int32_t nsweeps
 /* jacc_sweep_until (no counterpart in the paper, which runs a fixed iteration
  * count; §5.2 notes that Himeno reduces its error each iteration): sweeps
  * u0 -> u1 -> u0 ... until a sweep's residual is <= tol or max_sweeps sweeps
- * ran, with the loop and its exit test on the device: one CUDA graph (cached
- * per kernel, fields, max_sweeps, tol and output arrays, dropped by
- * jacc_release) whose WHILE conditional node runs the sweeps, each followed by
- * a one-thread kernel that stores the residual and sets the loop condition;
- * the host never waits.  5PT and 7PT only (their residual is max |v - u|);
+ * ran, with the loop and its exit test on the device; the host never waits.
+ * FP64 5PT grids of at most 2^17 points that fit one cluster (see
+ * JACC_SPEC_CLUSTER) run in one launch of it.  Otherwise it is one CUDA graph
+ * (cached per kernel, fields, max_sweeps, tol and output arrays, dropped by
+ * jacc_release) whose WHILE conditional node runs 16 sweeps a turn (4 of large
+ * fields), each followed by a one-thread kernel that stores the residual and
+ * tells the sweeps after it, and the loop, to stop.
+ * 5PT and 7PT only (their residual is max |v - u|);
  * 27PT is JACC_ERR_UNSUPPORTED.  tol finite and >= 0, max_sweeps >= 1.
  *   resid_dev  (device, max_sweeps doubles, required): resid_dev[i] for each
  *              sweep i that ran; later slots are untouched.
@@ -499,8 +508,8 @@ jacc_status jacc_autotune_forget(void);
  *               device FP32) into *loss_dev and its gradient into grad_dev
  *               (8705 floats); no update.
  * train       : `epochs` full-batch Adam steps (beta1 0.9, beta2 0.999,
- *               eps 1e-8, bias-corrected) with learning rate lr, run as CUDA
- *               graphs on `stream`; *loss_dev (nullable) = loss before the
+ *               eps 1e-8, bias-corrected) with learning rate lr, run on
+ *               `stream` (more than 128 epochs as CUDA graphs); *loss_dev (nullable) = loss before the
  *               last step.
  * predict     : y_dev[i] = network(x_dev[i]).
  * pick        : nq queries of JACC_NUM_TILES feature rows each (feats_dev
