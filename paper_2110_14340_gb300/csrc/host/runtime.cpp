@@ -9,6 +9,7 @@
 // as arguments); with it, NVRTC compiles the same template with them folded.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -213,6 +214,24 @@ int default_tile(const jacc_kernel_desc& d) {
   return vec_ok ? 1 : 0;
 }
 
+// CTAs that a grid holds at most in y and in z.
+constexpr int64_t kGridYZ = 65535;
+
+// Whether the few planes per CTA of the kernel without staging keep its grid
+// within that limit (up to 131070 planes; a loop over the rest in the kernel
+// itself cost every grid 5 to 15 %).
+static bool direct_fits(const jacc_kernel_desc& d) {
+  return (d.nz + JACC_DIRECT_PLANES - 1) / JACC_DIRECT_PLANES <= kGridYZ;
+}
+
+// The kernel family of a table tile: its own kernel, but the ring for the
+// tiles that stage nothing where those would take too many CTAs.
+static int table_family(const jacc_kernel_desc& d, int tile) {
+  const TileCfg& c = kTiles[tile];
+  const bool direct = d.stencil == 7 && JACC_DIRECT_TILE(c.bx, c.by, c.vec16 ? 2 : 1);
+  return direct && !direct_fits(d) ? JACC_FAM_RING : JACC_FAM_TABLE;
+}
+
 // The kernel family of the library's own choice.  7-point grids that live in
 // L2 need no staging (us a sweep without / with the ring: FP32 64^3 1.8 / 3.3,
 // 128^3 4.2 / 4.9, 160^3 9.9 / 10.4, 216^3 18.0 / 16.0; FP64 64^3 3.1 / 5.4,
@@ -230,7 +249,7 @@ static int default_family(const jacc_kernel_desc& d, int tile) {
   const int64_t n = d.nx * d.ny * d.nz;
   if (d.stencil == 7) {
     const int64_t direct = vec ? (f64 ? int64_t(1) << 21 : int64_t(1) << 22) : (f64 ? int64_t(1) << 20 : int64_t(5) << 17);
-    if (n <= direct) return JACC_FAM_DIRECT;
+    if (n <= direct && direct_fits(d)) return JACC_FAM_DIRECT;
   }
   const bool bulk = d.stencil == 7 ? n * (f64 ? 8 : 4) >= (int64_t(1) << 28) : !f64 && n * 4 >= (int64_t(1) << 30);
   const bool pays = (d.flags & JACC_SPEC_JIT) || (d.stencil == 7 && !f64);
@@ -262,6 +281,12 @@ static dim3 cta_grid(const jacc_kernel_desc& d, const CtaTile& t) {
   if (d.stencil == 5) return dim3(up(d.nx, t.cols), up(d.ny, t.rows * t.march), 1);
   return dim3(up(d.nx, t.cols), up(d.ny, t.rows), up(d.nz, t.march));
 }
+// The least planes per CTA that keep a 3D grid within its limit in z: more
+// than the tile's own where the library's kernels march fewer (131071 planes
+// upwards).
+static int least_chunk(const jacc_kernel_desc& d) {
+  return d.stencil == 5 ? 1 : static_cast<int>((d.nz + kGridYZ - 1) / kGridYZ);
+}
 
 bool tile_valid(const jacc_kernel_desc& d, int t) {
   const TileCfg& c = kTiles[t];
@@ -271,7 +296,7 @@ bool tile_valid(const jacc_kernel_desc& d, int t) {
   const int64_t gy = d.stencil == 5 ? (d.ny + c.by * (c.zc / 4) - 1) / (c.by * (c.zc / 4)) : (d.ny + c.by - 1) / c.by;
   const int64_t gz = d.stencil == 5 ? 1 : (d.nz + c.zc - 1) / c.zc;
   const int64_t gx = (d.nx + c.bx * V - 1) / (c.bx * V);
-  return gx < (1ll << 31) && gy <= 65535 && gz <= 65535;
+  return gx < (1ll << 31) && gy <= kGridYZ && gz <= kGridYZ;
 }
 
 static std::string key_of(const jacc_kernel_desc& d, int tile, bool fit) {
@@ -342,7 +367,7 @@ static int fitted_chunk_out(const Kernel& k, int zc) {
   int best = zc;
   for (int z = 32; z >= 4; --z) {
     const int64_t chunks = (k.desc.nz + z - 1) / z;
-    if (chunks > 65535) break;
+    if (chunks > kGridYZ) break;
     const int64_t cost = (columns * chunks + slots - 1) / slots * (z + 3);
     if (cost < least) {
       least = cost;
@@ -520,13 +545,13 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   p.c2 = desc->coeffs[2];
   p.c3 = desc->coeffs[3];
   plan_fixed(*desc, p);
-  k->fam = fit ? default_family(*desc, tile) : JACC_FAM_TABLE;
+  k->fam = fit ? default_family(*desc, tile) : table_family(*desc, tile);
   const int fam = k->fam;
   k->block_out = dim3(c.bx, c.by, 1);
   k->block = fam == JACC_FAM_DIRECT ? dim3(32, 8, 1) : k->block_out;
   if (!(desc->flags & JACC_SPEC_JIT) && desc->stencil != 19 && desc->tblock <= 1) {
     k->func = fam == JACC_FAM_TABLE || fam == JACC_FAM_BULK ? table_entry(desc->stencil, desc->dtype, tile, false)
-                                                            : lib_entry(*desc, p, fam, k->vec > 1);
+                                                            : lib_entry(*desc, p, fit ? fam : 5, k->vec > 1);
     if (fam == JACC_FAM_TABLE && p.fpath == JACC_FP_W32) k->func = jacc_tab_27_64_w32[tile];
     k->func_out = desc->dtype == 32 ? k->func
                   : fam == JACC_FAM_STRIP ? lib_entry(*desc, p, 5, k->vec > 1)
@@ -540,8 +565,9 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   if (fit) {
     p.zc = fitted_chunk(*k, p.zc);
     if (desc->stencil == 5)
-      while ((desc->ny + c.by * p.zc - 1) / (c.by * p.zc) > 65535) p.zc *= 2;  // the grid's limit
+      while ((desc->ny + c.by * p.zc - 1) / (c.by * p.zc) > kGridYZ) p.zc *= 2;  // the grid's limit
   }
+  if (desc->stencil != 19 && desc->tblock <= 1) p.zc = std::max(p.zc, least_chunk(*desc));
   k->zc_out = fit && edge && k->func_out && desc->stencil != 5 ? fitted_chunk_out(*k, p.zc) : p.zc;
   k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, k->zc_out));
   k->grid = cta_grid(*desc, cta_tile(*desc, tile, fam, false, p.zc));

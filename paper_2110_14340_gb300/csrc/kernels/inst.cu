@@ -39,8 +39,9 @@ typedef float JT;
 extern "C" const void* const JTABNAME(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY)};
 extern "C" const void* const JTABOUT(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY_OUT)};
 
-// The library's own kernels, [family][16-byte columns]; the last row (5-point
-// FP64) holds the strip march of the converting sweeps.
+// The library's own kernels, [family][16-byte columns]; the last row holds the
+// strip march of the converting sweeps (5-point FP64) and the ring of the
+// table's scalar 32 x 8 tiles (7-point).
 #define JPAIR(BX, BY, FAM, O) {JKERN(BX, BY, 1, FAM, O), JKERN(BX, BY, JVEC, FAM, O)}
 #define JNONE {nullptr, nullptr}
 extern "C" const void* const JTABLIB(JACC_INST_STENCIL, JACC_INST_DTYPE)[6][2] = {
@@ -48,7 +49,8 @@ extern "C" const void* const JTABLIB(JACC_INST_STENCIL, JACC_INST_DTYPE)[6][2] =
 #if JACC_INST_STENCIL == 5
     JPAIR(32, 4, JACC_FAM_STRIP, false), JNONE, JNONE, JNONE, JPAIR(32, 4, JACC_FAM_STRIP, JEDGE),
 #elif JACC_INST_STENCIL == 7
-    JNONE, JPAIR(32, 4, JACC_FAM_RING, false), JPAIR(32, 8, JACC_FAM_DIRECT, false), JNONE, JNONE,
+    JNONE, JPAIR(32, 4, JACC_FAM_RING, false), JPAIR(32, 8, JACC_FAM_DIRECT, false), JNONE,
+    {JKERN(32, 8, 1, JACC_FAM_RING, false), nullptr},
 #else
     JNONE, JPAIR(32, 4, JACC_FAM_RING, false), JNONE, JNONE, JNONE,
 #endif
