@@ -437,21 +437,6 @@ static std::string jit_source(const Kernel& k) {
   };
   auto bound = [&](int fam, bool edge) {
     if (st == 5) return std::string();
-    // The folded FP32 27-point kernel of 32 x 4 threads staged by bulk copies
-    // takes 72 registers (7 CTAs an SM) or, bounded, 64 (8): whichever fills
-    // its waves better (us a sweep at 7 and 8: 1024^3, 30.8 and 26.9 waves,
-    // 1332 and 1308; 768^3, 13.0 and 11.4 waves, 577 and 595; 512^3, 3.8 and
-    // 3.4, 195.7 and 196.2).
-    if (st == 27 && k.desc.dtype == 32 && k.vec == 4 && c.bx == 32 && c.by == 4 &&
-        (fam == JACC_FAM_TABLE || fam == JACC_FAM_BULK)) {
-      int dev = 0, nsm = 0;
-      if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
-        const int64_t ctas = static_cast<int64_t>(k.grid.x) * k.grid.y * k.grid.z, s7 = 7 * nsm, s8 = 8 * nsm;
-        if ((ctas + s8 - 1) / s8 * 8 <= (ctas + s7 - 1) / s7 * 7) return std::string(", 8");
-      } else {
-        cudaGetLastError();
-      }
-    }
     return ", (SweepMinBlocks<" + std::to_string(st) + ", " + shape(fam, edge) + tail(fam, edge) + ", true>::value)";
   };
   std::string src = std::string(device_source()) + fold;

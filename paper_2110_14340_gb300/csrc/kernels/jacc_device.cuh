@@ -821,11 +821,21 @@ template <int BX, int BY> struct alignas(128) Box27SSmem {
 
 // What lane r of warp 0 copies of every staged plane: staged row r, as one bulk
 // copy, or as two or more where the row's slots wrap around the periodic x
-// boundary.  Worked out once: the wraps are divisions.
+// boundary.
 struct Box27Row {
   i64 row;  // offset of the row in its plane
   i64 c;    // first column
 };
+
+// Whether a CTA works its rows and planes out once and carries them (every
+// thread holds the registers, though only warp 0's lanes use them), or for
+// every request.  Folded kernels know that a staged row wraps once at most
+// (ny >= R): a comparison or two per request, and 64 registers, 8 CTAs an SM,
+// instead of 72 and 7 (32 x 4 threads, us a sweep carried / not: 1024^3 1309 /
+// 1294, 768^3 577 / 573, 512^3 196 / 190, 800 x 900 x 1000 1014 / 976).
+// Precompiled ones would divide: 1024^3 1468 carried, 1565 not.
+template <class P, int R> struct Box27Carry { static constexpr bool value = P::ny < R; };
+template <int R> struct Box27Carry<JParams, R> { static constexpr bool value = true; };
 
 // Warp 0 requests a plane into stage s: lane 0 posts the byte count, then each
 // lane copies its row.
@@ -916,13 +926,20 @@ JD double box27s_body(const float* __restrict__ u, float* __restrict__ v, const 
     __syncthreads();
   }
   static_assert(G::R <= 32, "one staged row per lane of warp 0");
+  constexpr bool CARRY = Box27Carry<P, G::R>::value;
   Box27Row lrow;
-  lrow.row = ((by0 - 1 + (tid & 31) + ny) % ny) * nx;
+  if constexpr (CARRY) lrow.row = ((by0 - 1 + (tid & 31) + ny) % ny) * nx;
   lrow.c = bx0 >= 4 ? bx0 - 4 : bx0 - 4 + nx;
   i64 zi = z0 == 0 ? nz - 1 : z0 - 1;  // the next plane to request
   auto request = [&](int j, int s) {
+    if constexpr (!CARRY) {  // staged rows -1 .. ny + TH and planes -1 .. nz: one wrap at most
+      const i64 y = by0 - 1 + (tid & 31);
+      lrow.row = (y < 0 ? y + ny : (y >= ny ? y - ny : y)) * nx;
+      zi = z0 - 1 + j;
+      zi = zi < 0 ? zi + nz : (zi >= nz ? zi - nz : zi);
+    }
     if (!(stall_cta && j == rt.stall_plane)) box27s_issue<BX, BY>(sm, s, u + zi * sz, lrow, nx, weff);
-    zi = zi + 1 == nz ? 0 : zi + 1;
+    if constexpr (CARRY) zi = zi + 1 == nz ? 0 : zi + 1;
   };
   int issued = 0, consumed = 0;  // warp 0: planes requested, planes waited for
   RingPlan<float, BX, BY, 4, 4> plan;
