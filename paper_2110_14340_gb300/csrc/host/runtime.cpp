@@ -535,8 +535,8 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   k->block_out = dim3(c.bx, c.by, 1);
   k->block = fam == JACC_FAM_DIRECT ? dim3(32, 8, 1) : k->block_out;
   if (!(desc->flags & JACC_SPEC_JIT) && desc->stencil != 19 && desc->tblock <= 1) {
-    k->func = fam == JACC_FAM_TABLE || fam == JACC_FAM_BULK ? table_entry(desc->stencil, desc->dtype, tile, false)
-                                                            : lib_entry(*desc, p, fit ? fam : 5, k->vec > 1);
+    k->func = fam == JACC_FAM_TABLE ? table_entry(desc->stencil, desc->dtype, tile, false)
+                                    : lib_entry(*desc, p, fit ? fam : 5, k->vec > 1);
     if (fam == JACC_FAM_TABLE && p.fpath == JACC_FP_W32) k->func = jacc_tab_27_64_w32[tile];
     k->func_out = desc->dtype == 32 ? k->func
                   : fam == JACC_FAM_STRIP ? lib_entry(*desc, p, 5, k->vec > 1)

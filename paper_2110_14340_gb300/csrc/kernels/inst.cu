@@ -16,24 +16,32 @@ typedef float JT;
 #endif
 
 #if JACC_INST_STENCIL == 5
-#define JKERN(BX, BY, V, FAM, O) (const void*)jacc_k_jacobi2d<JT, BX, BY, V, FAM, O>
+#define JKERNP(BX, BY, V, FAM, O, ...) (const void*)jacc_k_jacobi2d<JT, BX, BY, V, FAM, O, __VA_ARGS__>
 #elif JACC_INST_STENCIL == 7
-#define JKERN(BX, BY, V, FAM, O) (const void*)jacc_k_heat3d<JT, BX, BY, V, FAM, O>
+#define JKERNP(BX, BY, V, FAM, O, ...) (const void*)jacc_k_heat3d<JT, BX, BY, V, FAM, O, __VA_ARGS__>
 #else
-#define JKERN(BX, BY, V, FAM, O) (const void*)jacc_k_box27<JT, BX, BY, V, FAM, O, JParams>
+#define JKERNP(BX, BY, V, FAM, O, ...) (const void*)jacc_k_box27<JT, BX, BY, V, FAM, O, __VA_ARGS__>
 #endif
+#define JKERN(BX, BY, V, FAM, O) JKERNP(BX, BY, V, FAM, O, JParams)
+// the tile's march length, where it is a constant
+#define JTABP(BX, BY, V, ZC) TableP<JACC_INST_STENCIL, JT, BX, BY, V, ZC>::type
 
 #define JCAT3(a, b, c) a##b##_##c
 #define JCAT4(a, b, c, d) a##b##_##c##d
 #define JTABNAME(s, d) JCAT3(jacc_tab_, s, d)
 #define JTABOUT(s, d) JCAT4(jacc_tab_, s, d, _out)
 #define JTABLIB(s, d) JCAT4(jacc_tab_, s, d, _lib)
-#define JENTRY(id, BX, BY, VEC, ZC) JKERN(BX, BY, ((VEC) ? JVEC : 1), JACC_FAM_TABLE, false),
-#define JENTRY_OUT(id, BX, BY, VEC, ZC) JKERN(BX, BY, ((VEC) ? JVEC : 1), JACC_FAM_TABLE, JEDGE),
+#define JENTRY(id, BX, BY, VEC, ZC) \
+  JKERNP(BX, BY, ((VEC) ? JVEC : 1), JACC_FAM_TABLE, false, JTABP(BX, BY, ((VEC) ? JVEC : 1), ZC)),
+#if JACC_INST_STENCIL == 5 || JACC_INST_DTYPE == 32
+#define JENTRY_OUT(id, BX, BY, VEC, ZC) \
+  JKERNP(BX, BY, ((VEC) ? JVEC : 1), JACC_FAM_TABLE, JEDGE, JTABP(BX, BY, ((VEC) ? JVEC : 1), ZC)),
+#else  // rings, whose planes per CTA the library may choose
+#define JENTRY_OUT(id, BX, BY, VEC, ZC) JKERN(BX, BY, ((VEC) ? JVEC : 1), JACC_FAM_TABLE, true),
+#endif
 
 // Table 1: the intermediate sweeps of a fixed-point sequence (and every FP32
-// or native sweep); the march length (planes per CTA, rows per warp) is a
-// launch parameter.  Table 2 ("_out"): the first and last sweeps of a
+// or native sweep).  Table 2 ("_out"): the first and last sweeps of a
 // fixed-point sequence and single launches, which convert FP64 on load and/or
 // store; identical to table 1 for FP32.
 extern "C" const void* const JTABNAME(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY)};
@@ -49,8 +57,8 @@ extern "C" const void* const JTABLIB(JACC_INST_STENCIL, JACC_INST_DTYPE)[6][2] =
 #if JACC_INST_STENCIL == 5
     JPAIR(32, 4, JACC_FAM_STRIP, false), JNONE, JNONE, JNONE, JPAIR(32, 4, JACC_FAM_STRIP, JEDGE),
 #elif JACC_INST_STENCIL == 7
-    JNONE, JPAIR(32, 4, JACC_FAM_RING, false), JPAIR(32, 8, JACC_FAM_DIRECT, false), JNONE,
-    {JKERN(32, 8, 1, JACC_FAM_RING, false), nullptr},
+    JNONE, JPAIR(32, 4, JACC_FAM_RING, false), JPAIR(32, 8, JACC_FAM_DIRECT, false),
+    {nullptr, JKERN(32, 4, JVEC, JACC_FAM_BULK, false)}, {JKERN(32, 8, 1, JACC_FAM_RING, false), nullptr},
 #else
     JNONE, JPAIR(32, 4, JACC_FAM_RING, false), JNONE, JNONE, JNONE,
 #endif

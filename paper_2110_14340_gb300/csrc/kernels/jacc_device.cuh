@@ -32,6 +32,18 @@
 
 #define JD __device__ __forceinline__
 
+// The parameter block of a table tile's kernel: the march length is the tile's
+// own, known to the compiler.
+template <int ZC> struct JParamsZ : JParams {
+  static constexpr int zc = ZC;
+};
+// The parameter block with 32-bit fixed-point factors (JACC_FP_W32).
+struct JParamsW32 : JParams {
+  static constexpr int fpath = JACC_FP_W32;
+};
+// Whether extents and coefficients are constants (P is none of these blocks).
+template <class P> struct Folded { static constexpr bool value = !__is_base_of(JParams, P); };
+
 // ---------------------------------------------------------------- fixed point
 
 // Fraction bits for the sweep from the bit pattern of max|u| (non-negative
@@ -834,8 +846,8 @@ struct Box27Row {
 // instead of 72 and 7 (32 x 4 threads, us a sweep carried / not: 1024^3 1309 /
 // 1294, 768^3 577 / 573, 512^3 196 / 190, 800 x 900 x 1000 1014 / 976).
 // Precompiled ones would divide: 1024^3 1468 carried, 1565 not.
-template <class P, int R> struct Box27Carry { static constexpr bool value = P::ny < R; };
-template <int R> struct Box27Carry<JParams, R> { static constexpr bool value = true; };
+template <class P, int R, bool FOLDED = Folded<P>::value> struct Box27Carry { static constexpr bool value = true; };
+template <class P, int R> struct Box27Carry<P, R, true> { static constexpr bool value = P::ny < R; };
 
 // Warp 0 requests a plane into stage s: lane 0 posts the byte count, then each
 // lane copies its row.
@@ -1712,7 +1724,7 @@ JD void heat3s_body(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   const i64 fb = p.fb;
   const int k = p.fk;
   const bool fold = heat_fold(p);
-  constexpr bool folded = !SameT<P, JParams>::value;  // extents and coefficients are constants
+  constexpr bool folded = Folded<P>::value;  // extents and coefficients are constants
   vo += z0 * sz;
   // one output plane (staged plane j, 1 <= j <= L-2) from the own values of
   // planes j-1 (zp) and j (cur); fills zn with those of plane j+1
@@ -1969,7 +1981,7 @@ JD void heat3r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int 
   int cs = ns;  // stage of the centre plane
   ns += G::STAGE;
   const T r = (T)p.c0;
-  constexpr bool folded = !SameT<P, JParams>::value;
+  constexpr bool folded = Folded<P>::value;
   const bool fold = folded && heat_fold(p);
   const i64 fb = p.fb;
   const int fk = p.fk;
@@ -2301,7 +2313,7 @@ JD void heat3d_direct(const T* __restrict__ u, T* __restrict__ v, const P& p, R&
     if constexpr (FX) return bits_i64(t);
     else return t;
   };
-  constexpr bool folded = !SameT<P, JParams>::value;
+  constexpr bool folded = Folded<P>::value;
   const bool fold = folded && heat_fold(p);
   const T r = (T)p.c0;
   T* o = v + z0 * sz + y * nx + x;
@@ -2363,13 +2375,13 @@ JD void heat3d_direct(const T* __restrict__ u, T* __restrict__ v, const P& p, R&
 // where a tile with 16-byte columns was asked for: its few rows in flight are
 // latency-bound there (256 x 256 FP64, tile 1: 2.2 us a sweep, 3.0 by rows; at
 // 4096 x 4096 52 and 50).
-template <class P> struct SmallFold { static constexpr bool value = P::nx * P::ny <= JACC_SMALL_GRID; };
-template <> struct SmallFold<JParams> { static constexpr bool value = false; };
+template <class P, bool FOLDED = Folded<P>::value> struct SmallFold { static constexpr bool value = false; };
+template <class P> struct SmallFold<P, true> { static constexpr bool value = P::nx * P::ny <= JACC_SMALL_GRID; };
 // A folded FP64 grid of more than JACC_LARGE_GRID points, which streams from
 // HBM, has six rows in flight instead of three and marches twice the rows
 // (4096^2 44.7 us a sweep against 47.6; FP32 21.7 against 20.1).
-template <class P> struct LargeFold { static constexpr bool value = P::nx * P::ny > JACC_LARGE_GRID; };
-template <> struct LargeFold<JParams> { static constexpr bool value = false; };
+template <class P, bool FOLDED = Folded<P>::value> struct LargeFold { static constexpr bool value = false; };
+template <class P> struct LargeFold<P, true> { static constexpr bool value = P::nx * P::ny > JACC_LARGE_GRID; };
 template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, double* resid,
                        const u64* maxword, int flags) {
@@ -2443,7 +2455,7 @@ JD void heat3d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, con
     typedef RingG<double, BX, BY, V, V> G;
     // stage cap: 5 for the constant-folded intermediate sweeps (7 CTAs per SM,
     // SweepMinBlocks), else 6
-    constexpr int SC = !SameT<P, JParams>::value ? 5 : 6;
+    constexpr int SC = Folded<P>::value ? 5 : 6;
     // the native path covers the CTA's rows in sub-tiles of BY rows
     constexpr int SUBS = K::BULK ? 2 : G::RY;
     typedef Plane<double, BX, BY, V> NativePlane;
@@ -2627,6 +2639,12 @@ __global__ void jacc_k_fill_skipped(double* resid, int n, int T) {
 // and 518 at 5 (spills).
 // The precompiled staged FP32 27-point kernel: 7 CTAs (at most 72 registers;
 // left alone it spills at 64).
+// Table tiles of 256 or 512 threads with 16-byte columns, where a CTA fewer an
+// SM costs a wave (us a sweep, unbounded / bounded): FP32 27-point of 512
+// threads, 90 / 64 registers, tile 15 512^3 641 / 411, tile 21 192 x 160 x 144
+// 72 / 48; FP32 7-point of 256, 80 / 64, tile 5 256^3 39 / 29 and 512^3 199 /
+// 185 (64 x 60 x 62, where every CTA fits at once, 18.3 / 19.9); 5-point of 512,
+// FP64 74 / 64, tile 13 4096^2 100 / 69, FP32 48 / 40, tile 21 31.8 / 29.1.
 // Every other kernel: 0, no requirement (a bound of 1 is not neutral: it
 // lets the compiler take registers for one CTA per SM, e.g. 111 instead of
 // 80 for the staged FP32 7-point kernel).
@@ -2635,24 +2653,40 @@ template <int STENCIL, class T, int BX, int BY, int V, int FAM, bool EDGE, bool 
   static constexpr bool t32 = BX == 32 && BY == 4;
   static constexpr int heat = K::BULK ? (K::F64 ? (FOLDED ? 7 : 6) : 0) : K::RING ? (V == 1 || EDGE ? 5 : 6) : 0;
   static constexpr int box = K::F64 ? (EDGE ? 0 : 4) : (V == 4 && !FOLDED ? 7 : 0);
-  static constexpr int value = !t32 ? 0 : STENCIL == 7 ? heat : STENCIL == 27 ? box : 0;
+  static constexpr bool wide = K::VEC && FAM == JACC_FAM_TABLE && !FOLDED && !EDGE;
+  static constexpr int NT = BX * BY;
+  static constexpr int wide5 = NT == 512 ? (K::F64 ? 2 : 3) : 0, wide7 = !K::F64 && NT == 256 ? 4 : 0,
+                       wide27 = !K::F64 && NT == 512 ? 2 : 0;
+  static constexpr int other = !wide ? 0 : STENCIL == 5 ? wide5 : STENCIL == 7 ? wide7 : wide27;
+  static constexpr int value = !t32 ? other : STENCIL == 7 ? heat : STENCIL == 27 ? box : 0;
 };
 
-// Kernel templates instantiated by the precompiled library (P = JParams).
-template <class T, int BX, int BY, int V, int FAM, bool EDGE>
-__global__ void __launch_bounds__(BX * BY) jacc_k_jacobi2d(const T* __restrict__ u, T* __restrict__ v, JParams p,
-                                                           double* resid, const u64* maxword, int flags) {
+// The parameter block of a table tile's kernel.  The march length is a constant
+// where the kernel marches rows or planes from registers or bulk copies: as an
+// argument it costs registers, or the compiler moves the loads of the next
+// plane to where they are used (us a sweep, argument / constant: FP32 27-point
+// tile 0 512^3 893 / 730 and 192 x 160 x 144 35.2 / 25.9, FP64 5-point tile 7
+// 4096^2 76.1 / 70.1).  Strips, rings and the kernel without staging take it as
+// an argument.
+template <class A, class B, bool FIRST> struct PickT { typedef A type; };
+template <class A, class B> struct PickT<A, B, false> { typedef B type; };
+template <int STENCIL, class T, int BX, int BY, int V, int ZC> struct TableP {
+  typedef Load3D<STENCIL, T, BX, BY, V, JACC_FAM_TABLE, false> K;
+  static constexpr bool FIXED = STENCIL == 5 ? V > 1 : !(K::RING || K::DIRECT);
+  typedef typename PickT<JParamsZ<STENCIL == 5 ? ZC / 4 : ZC>, JParams, FIXED>::type type;
+};
+
+// Kernel templates instantiated by the precompiled library.
+template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
+__global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<5, T, BX, BY, V, FAM, EDGE, false>::value))
+    jacc_k_jacobi2d(const T* __restrict__ u, T* __restrict__ v, P p, double* resid, const u64* maxword, int flags) {
   jacobi2d_entry<T, BX, BY, V, FAM, EDGE>(u, v, p, p, resid, maxword, flags);
 }
-template <class T, int BX, int BY, int V, int FAM, bool EDGE>
+template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 __global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<7, T, BX, BY, V, FAM, EDGE, false>::value))
-    jacc_k_heat3d(const T* __restrict__ u, T* __restrict__ v, JParams p, double* resid, const u64* maxword, int flags) {
+    jacc_k_heat3d(const T* __restrict__ u, T* __restrict__ v, P p, double* resid, const u64* maxword, int flags) {
   heat3d_entry<T, BX, BY, V, FAM, EDGE>(u, v, p, p, resid, maxword, flags);
 }
-// P = JParamsW32: the same parameter block, known to hold 32-bit factors.
-struct JParamsW32 : JParams {
-  static constexpr int fpath = JACC_FP_W32;
-};
 template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
 __global__ void __launch_bounds__(BX * BY, (SweepMinBlocks<27, T, BX, BY, V, FAM, EDGE, false>::value))
     jacc_k_box27(const T* __restrict__ u, T* __restrict__ v, P p, double* resid, const u64* maxword, int flags) {
