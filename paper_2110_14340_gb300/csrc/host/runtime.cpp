@@ -225,11 +225,23 @@ static bool direct_fits(const jacc_kernel_desc& d) {
 }
 
 // The kernel family of a table tile: its own kernel, but the ring for the
-// tiles that stage nothing where those would take too many CTAs.
+// tiles that stage nothing where those would take too many CTAs, or where the
+// grid is too large for them (FP64, see default_family: 192 x 160 x 144 26.9 us a
+// sweep without staging, 22.4 with the ring; 512^3 798 and 480).
 static int table_family(const jacc_kernel_desc& d, int tile) {
   const TileCfg& c = kTiles[tile];
   const bool direct = d.stencil == 7 && JACC_DIRECT_TILE(c.bx, c.by, c.vec16 ? 2 : 1);
-  return direct && !direct_fits(d) ? JACC_FAM_RING : JACC_FAM_TABLE;
+  const bool large = d.dtype == 64 && d.nx * d.ny * d.nz > (int64_t(1) << 20);
+  return direct && (large || !direct_fits(d)) ? JACC_FAM_RING : JACC_FAM_TABLE;
+}
+
+// Whether the planes per CTA are fitted to the grid: kernels of the library's
+// choice, and the FP64 scalar 7-point tiles, whose ring covers four rows per
+// thread: with all of the tile's planes small grids do not fill the GPU (us a
+// sweep, all / fitted: 64 x 60 x 62 tile 10 37.9 / 6.4, 192 x 160 x 144 39.7 /
+// 22.2; large grids take all of them either way).
+static bool fits_planes(const jacc_kernel_desc& d, int tile, bool fit) {
+  return fit || (d.stencil == 7 && d.dtype == 64 && !kTiles[tile].vec16);
 }
 
 // The kernel family of the library's own choice.  7-point grids that live in
@@ -307,9 +319,8 @@ static std::string key_of(const jacc_kernel_desc& d, int tile, bool fit) {
   return std::string(reinterpret_cast<const char*>(&c), sizeof(c)) + (fit ? "f" : "t");
 }
 
-// Planes per CTA (3D) or rows per warp (2D) of a kernel whose tile the library
-// chose itself.  3D: at most
-// the tile's own, and few enough that the grid has at least 2.5 times the
+// Planes per CTA (3D) or rows per warp (2D) of a kernel that takes what fits
+// the grid.  3D: at most the tile's own, and few enough that the grid has at least 2.5 times the
 // CTAs that the device holds at once.  With fewer, the last wave leaves SMs
 // idle: 301 x 253 x 199 FP64 at 64 planes (640 CTAs on 152 SMs) 65.2 us a
 // sweep, at 16 planes (2080) 55.7, at 8 (4000) 57.3; 511^3, whose grid is
@@ -547,7 +558,7 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   const bool edge = desc->dtype == 64;
   p.zc = plane_chunk(*desc, tile, fam);
   k->grid = k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, p.zc));
-  if (fit) {
+  if (fits_planes(*desc, tile, fit)) {
     p.zc = fitted_chunk(*k, p.zc);
     if (desc->stencil == 5)
       while ((desc->ny + c.by * p.zc - 1) / (c.by * p.zc) > kGridYZ) p.zc *= 2;  // the grid's limit
