@@ -32,6 +32,9 @@ extern "C" const void* const jacc_tab_7_32_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_64_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_32_out[JACC_NTILES];
 extern "C" const void* const jacc_tab_27_64_w32[JACC_NTILES];
+extern "C" const void* const jacc_tab_5_64_native[JACC_NTILES];
+extern "C" const void* const jacc_tab_7_64_native[JACC_NTILES];
+extern "C" const void* const jacc_tab_27_64_native[JACC_NTILES];
 extern "C" const void* const jacc_tab_5_64_lib[6][2];
 extern "C" const void* const jacc_tab_5_32_lib[6][2];
 extern "C" const void* const jacc_tab_7_64_lib[6][2];
@@ -191,6 +194,10 @@ static jacc_status validate(const jacc_kernel_desc& d) {
   return ok();
 }
 
+static const void* native_entry(int stencil, int tile) {
+  return (stencil == 5 ? jacc_tab_5_64_native : stencil == 7 ? jacc_tab_7_64_native : jacc_tab_27_64_native)[tile];
+}
+
 // The library's own kernel (entry `row` of its table), or null.
 static const void* lib_entry(const jacc_kernel_desc& d, const JParams& p, int row, bool vec) {
   const bool f64 = d.dtype == 64;
@@ -214,6 +221,22 @@ int default_tile(const jacc_kernel_desc& d) {
   return vec_ok ? 1 : 0;
 }
 
+// Whether the descriptor's sweeps always run native FP64 arithmetic.
+static bool native_fp64(const jacc_kernel_desc& d, int fpath) {
+  return d.dtype == 64 && d.stencil != 19 && fpath == JACC_FP_NONE;
+}
+
+// The default tile of native FP64 sweeps, bound by the FP64 pipe.  2D: 16-byte
+// columns and four rows per thread from 2^19 points on, where the grid leaves
+// L2 (4096^2: 259 us a sweep, 288 by strips); below, more and narrower CTAs.
+static int default_tile_native(const jacc_kernel_desc& d) {
+  if (d.stencil == 5) {
+    const int t = d.nx * d.ny < (int64_t(1) << 19) ? 8 : d.nx % 2 ? 16 : 17;
+    if (tile_valid(d, t)) return t;
+  }
+  return default_tile(d);
+}
+
 // CTAs that a grid holds at most in y and in z.
 constexpr int64_t kGridYZ = 65535;
 
@@ -228,8 +251,9 @@ static bool direct_fits(const jacc_kernel_desc& d) {
 // tiles that stage nothing where those would take too many CTAs, or where the
 // grid is too large for them (FP64, see default_family: 192 x 160 x 144 26.9 us a
 // sweep without staging, 22.4 with the ring; 512^3 798 and 480).
-static int table_family(const jacc_kernel_desc& d, int tile) {
+static int table_family(const jacc_kernel_desc& d, int tile, int fpath) {
   const TileCfg& c = kTiles[tile];
+  if (native_fp64(d, fpath)) return JACC_FAM_NATIVE;
   const bool direct = d.stencil == 7 && JACC_DIRECT_TILE(c.bx, c.by, c.vec16 ? 2 : 1);
   const bool large = d.dtype == 64 && d.nx * d.ny * d.nz > (int64_t(1) << 20);
   return direct && (large || !direct_fits(d)) ? JACC_FAM_RING : JACC_FAM_TABLE;
@@ -240,8 +264,8 @@ static int table_family(const jacc_kernel_desc& d, int tile) {
 // thread: with all of the tile's planes small grids do not fill the GPU (us a
 // sweep, all / fitted: 64 x 60 x 62 tile 10 37.9 / 6.4, 192 x 160 x 144 39.7 /
 // 22.2; large grids take all of them either way).
-static bool fits_planes(const jacc_kernel_desc& d, int tile, bool fit) {
-  return fit || (d.stencil == 7 && d.dtype == 64 && !kTiles[tile].vec16);
+static bool fits_planes(const jacc_kernel_desc& d, int tile, int fam, bool fit) {
+  return fit || (d.stencil == 7 && d.dtype == 64 && !kTiles[tile].vec16 && fam != JACC_FAM_NATIVE);
 }
 
 // The kernel family of the library's own choice.  7-point grids that live in
@@ -276,10 +300,13 @@ struct CtaTile {
 static CtaTile cta_tile(const jacc_kernel_desc& d, int tile, int fam, bool edge, int zc) {
   const TileCfg& c = kTiles[tile];
   const int V = c.vec16 ? (d.dtype == 64 ? 2 : 4) : 1;
-  if (d.stencil == 5)
-    return fam == JACC_FAM_STRIP || V == 1 || ((d.flags & JACC_SPEC_JIT) && d.nx * d.ny <= JACC_SMALL_GRID)
-               ? CtaTile{static_cast<int64_t>(c.bx / 32) * 30 * V, c.by, zc}
-               : CtaTile{static_cast<int64_t>(c.bx) * V, c.by, zc};
+  const CtaTile rows{static_cast<int64_t>(c.bx) * V, c.by, zc};
+  if (d.stencil == 5) {
+    const bool small = (d.flags & JACC_SPEC_JIT) && d.nx * d.ny <= JACC_SMALL_GRID;
+    const bool strips = small || (fam != JACC_FAM_NATIVE && (fam == JACC_FAM_STRIP || V == 1));
+    return strips ? CtaTile{static_cast<int64_t>(c.bx / 32) * 30 * V, c.by, zc} : rows;
+  }
+  if (fam == JACC_FAM_NATIVE) return rows;
   const bool f64 = d.dtype == 64;
   if (d.stencil == 7 && !edge && (fam == JACC_FAM_DIRECT || (fam == JACC_FAM_TABLE && JACC_DIRECT_TILE(c.bx, c.by, V))))
     return CtaTile{static_cast<int64_t>(32) * V, 8, JACC_DIRECT_PLANES};
@@ -403,6 +430,7 @@ static int plane_chunk(const jacc_kernel_desc& d, int tile, int fam) {
   const TileCfg& c = kTiles[tile];
   if (d.stencil == 5) return c.zc / 4;  // rows per warp
   const bool f64 = d.dtype == 64;
+  if (fam == JACC_FAM_NATIVE) return c.zc;
   if (d.stencil == 7 && !f64 && (fam == JACC_FAM_RING || fam == JACC_FAM_BULK)) return 16;
   if (d.stencil == 7 && f64 && fam == JACC_FAM_RING) return c.zc < 24 ? c.zc : 24;
   const bool bulk = c.vec16 && !(d.stencil == 27 && f64) && (fam == JACC_FAM_TABLE || fam == JACC_FAM_BULK);
@@ -413,7 +441,8 @@ static int plane_chunk(const jacc_kernel_desc& d, int tile, int fam) {
 // The NVRTC source of a folded variant: the device text plus a struct whose
 // static constexpr members replace JParams, and the kernels: jacc_jit for the
 // intermediate (and every FP32 or native) sweeps, and for FP64 jacc_jit_out,
-// which converts FP64 on load and store, and jacc_jit_last, only on store.
+// in fixed point which converts FP64 on load and store, and jacc_jit_last, only
+// on store.
 static std::string jit_source(const Kernel& k) {
   const JParams& p = k.params;
   const TileCfg& c = kTiles[k.tile];
@@ -452,7 +481,7 @@ static std::string jit_source(const Kernel& k) {
   };
   std::string src = std::string(device_source()) + fold;
   src += kernel("jacc_jit", k.fam == JACC_FAM_DIRECT ? 256 : c.bx * c.by, bound(k.fam, false), call(k.fam, false, "flags"));
-  if (k.desc.dtype == 64) {
+  if (k.desc.dtype == 64 && k.fam != JACC_FAM_NATIVE) {
     src += kernel("jacc_jit_out", c.bx * c.by, bound(k.fam, true), call(k.fam, true, "flags"));
     src += kernel("jacc_jit_last", c.bx * c.by, bound(k.fam, true), call(k.fam, true, "JFX_OUT_F64"));
   }
@@ -495,6 +524,9 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   if (!desc || !out) return fail(JACC_ERR_INVALID_ARG, "NULL descriptor or output");
   jacc_status st = validate(*desc);
   if (st) return st;
+  JParams plan{};
+  plan_fixed(*desc, plan);
+  const bool native = native_fp64(*desc, plan.fpath);
   int tile = desc->tile_id;
   bool fit = false;  // the library picks the kernel family and the march along with the tile
   if (desc->stencil == 19) {
@@ -510,8 +542,8 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
         kTiles[tile].by == 4 && desc->nx * desc->ny * desc->nz >= (int64_t(1) << 25) && tile_valid(*desc, tile | 1))
       tile |= 1;
     if (tile < 0 || !tile_valid(*desc, tile)) {
-      tile = default_tile(*desc);
-      fit = desc->stencil != 19 && desc->tblock <= 1;
+      tile = native ? default_tile_native(*desc) : default_tile(*desc);
+      fit = desc->stencil != 19 && desc->tblock <= 1 && !native;
     }
   }
   if (!tile_valid(*desc, tile))
@@ -533,6 +565,7 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   const TileCfg& c = kTiles[tile];
   k->vec = c.vec16 ? 16 / k->elem : 1;
   JParams& p = k->params;
+  p = plan;
   p.nx = desc->nx;
   p.ny = desc->ny;
   p.nz = desc->nz;
@@ -540,25 +573,25 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   p.c1 = desc->coeffs[1];
   p.c2 = desc->coeffs[2];
   p.c3 = desc->coeffs[3];
-  plan_fixed(*desc, p);
-  k->fam = fit ? default_family(*desc, tile) : table_family(*desc, tile);
+  k->fam = fit ? default_family(*desc, tile) : table_family(*desc, tile, p.fpath);
   const int fam = k->fam;
+  // fixed-point sequences convert in their first and last sweeps, which have a kernel of their own
+  const bool edge = desc->dtype == 64 && !native;
   k->block_out = dim3(c.bx, c.by, 1);
   k->block = fam == JACC_FAM_DIRECT ? dim3(32, 8, 1) : k->block_out;
   if (!(desc->flags & JACC_SPEC_JIT) && desc->stencil != 19 && desc->tblock <= 1) {
-    k->func = fam == JACC_FAM_TABLE ? table_entry(desc->stencil, desc->dtype, tile, false)
-                                    : lib_entry(*desc, p, fit ? fam : 5, k->vec > 1);
+    k->func = native ? native_entry(desc->stencil, tile)
+              : fam == JACC_FAM_TABLE ? table_entry(desc->stencil, desc->dtype, tile, false)
+                                      : lib_entry(*desc, p, fit ? fam : 5, k->vec > 1);
     if (fam == JACC_FAM_TABLE && p.fpath == JACC_FP_W32) k->func = jacc_tab_27_64_w32[tile];
-    k->func_out = desc->dtype == 32 ? k->func
+    k->func_out = !edge ? k->func
                   : fam == JACC_FAM_STRIP ? lib_entry(*desc, p, 5, k->vec > 1)
                                           : table_entry(desc->stencil, desc->dtype, tile, true);
     if (!k->func || !k->func_out) return fail(JACC_ERR_UNSUPPORTED, "no precompiled kernel for this descriptor");
   }
-  // FP64 sequences convert in their first and last sweeps, which have a kernel of their own
-  const bool edge = desc->dtype == 64;
   p.zc = plane_chunk(*desc, tile, fam);
   k->grid = k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, p.zc));
-  if (fits_planes(*desc, tile, fit)) {
+  if (fits_planes(*desc, tile, fam, fit)) {
     p.zc = fitted_chunk(*k, p.zc);
     if (desc->stencil == 5)
       while ((desc->ny + c.by * p.zc - 1) / (c.by * p.zc) > kGridYZ) p.zc *= 2;  // the grid's limit
@@ -594,11 +627,11 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   } else if (desc->flags & JACC_SPEC_JIT) {
     static const char* const names[3] = {"jacc_jit", "jacc_jit_out", "jacc_jit_last"};
     const void* f[3] = {nullptr, nullptr, nullptr};
-    st = jit_compile(jit_source(*k), names, desc->dtype == 64 ? 3 : 1, &k->lib, f, &k->compile_ms);
+    st = jit_compile(jit_source(*k), names, edge ? 3 : 1, &k->lib, f, &k->compile_ms);
     if (st) return st;
     k->func = f[0];
-    k->func_out = desc->dtype == 64 ? f[1] : f[0];
-    k->func_last = f[2];  // FP64 only
+    k->func_out = edge ? f[1] : f[0];
+    k->func_last = f[2];  // fixed point only
     k->jit = true;
   }
   if (!edge) {

@@ -47,6 +47,15 @@ typedef float JT;
 extern "C" const void* const JTABNAME(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY)};
 extern "C" const void* const JTABOUT(JACC_INST_STENCIL, JACC_INST_DTYPE)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY_OUT)};
 
+#if JACC_INST_DTYPE == 64
+// The tiles' kernels in native FP64 arithmetic.
+#define JENTRY_NATIVE(id, BX, BY, VEC, ZC)                        \
+  JKERNP(BX, BY, ((VEC) ? JVEC : 1), JACC_FAM_NATIVE, false, \
+         TableP<JACC_INST_STENCIL, JT, BX, BY, ((VEC) ? JVEC : 1), ZC, true>::type),
+#define JTABNATIVE(s) JCAT3(jacc_tab_, s, 64_native)
+extern "C" const void* const JTABNATIVE(JACC_INST_STENCIL)[JACC_NTILES] = {JACC_TILE_LIST(JENTRY_NATIVE)};
+#endif
+
 // The library's own kernels, [family][16-byte columns]; the last row holds the
 // strip march of the converting sweeps (5-point FP64) and the ring of the
 // table's scalar 32 x 8 tiles (7-point).

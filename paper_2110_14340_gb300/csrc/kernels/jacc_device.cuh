@@ -2370,7 +2370,11 @@ JD void heat3d_direct(const T* __restrict__ u, T* __restrict__ v, const P& p, R&
 // Kernel families (JACC_FAM_*, jacc_params.h): a table tile runs the kernel
 // that the autotuner times for it; the library's own choice (no tile asked
 // for, none remembered) may also take the strip march, the asynchronous-copy
-// ring, or no staging at all.
+// ring, or no staging at all.  FP64 handles that never run in fixed point
+// (JACC_ARITH_NATIVE, non-convex coefficients) take kernels of their own
+// (JACC_FAM_NATIVE): the fixed-point kernels also hold a native branch, for
+// fields that turn out not to fit the format, but its CTAs cover several rows a
+// thread one after the other, under register bounds made for integers.
 // A folded grid of at most JACC_SMALL_GRID points takes the strip march also
 // where a tile with 16-byte columns was asked for: its few rows in flight are
 // latency-bound there (256 x 256 FP64, tile 1: 2.2 us a sweep, 3.0 by rows; at
@@ -2391,14 +2395,17 @@ JD void jacobi2d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, c
   const i64 ys = ((i64)blockIdx.y * BY + threadIdx.y) * p.zc;
   const i64 ye = (ys + p.zc < p.ny) ? ys + p.zc : p.ny;
   // scalar columns and small folded grids march strips whatever the tile
-  constexpr bool STRIP = FAM == JACC_FAM_STRIP || V == 1 || SmallFold<P>::value;
+  // (native FP64 arithmetic only the latter: its own pipe bounds it, and a strip
+  // updates 2/30 of its points twice)
+  constexpr bool NATIVE = FAM == JACC_FAM_NATIVE;
+  constexpr bool STRIP = SmallFold<P>::value || (!NATIVE && (FAM == JACC_FAM_STRIP || V == 1));
   constexpr int DEPTH = !EDGE && V == 2 && LargeFold<P>::value ? 6 : 3;
   // STRIP: BX / 32 strips of 30 V columns across the CTA
   const i64 strip = (i64)blockIdx.x * (BX / 32) + (threadIdx.x >> 5);
   const i64 xl = STRIP ? strip * (30 * V) + ((int)(threadIdx.x & 31) - 1) * V : (i64)blockIdx.x * (BX * V) + (i64)threadIdx.x * V;
-  const int F = (sizeof(T) == 8 && maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
-  if (sizeof(T) == 8 && F >= 0) {
-    if constexpr (sizeof(T) == 8) {
+  const int F = (!NATIVE && sizeof(T) == 8 && maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
+  if (!NATIVE && sizeof(T) == 8 && F >= 0) {
+    if constexpr (!NATIVE && sizeof(T) == 8) {
       u64 m = 0;
       if (ys < p.ny) {
         if constexpr (STRIP) jacobi_strip<double, V, true, EDGE, DEPTH>(u, v, p.nx, p.ny, xl, ys, ye, F, flags, m);
@@ -2430,7 +2437,7 @@ template <int STENCIL, class T, int BX, int BY, int V, int FAM, bool EDGE> struc
   static constexpr bool DIRECT =
       !EDGE && STENCIL == 7 && (FAM == JACC_FAM_DIRECT || (FAM == JACC_FAM_TABLE && JACC_DIRECT_TILE(BX, BY, V)));
   static constexpr bool BULK = !EDGE && VEC && (FAM == JACC_FAM_TABLE || FAM == JACC_FAM_BULK) && !(F64 && STENCIL == 27);
-  static constexpr bool RING = !DIRECT && !BULK && (EDGE || F64 || FAM == JACC_FAM_RING);
+  static constexpr bool RING = !DIRECT && !BULK && FAM != JACC_FAM_NATIVE && (EDGE || F64 || FAM == JACC_FAM_RING);
 };
 
 template <class T, int BX, int BY, int V, int FAM, bool EDGE, class P>
@@ -2441,7 +2448,12 @@ JD void heat3d_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, con
   typedef Load3D<7, T, BX, BY, V, FAM, EDGE> K;
   u64 bits = 0;
   const int F = (sizeof(T) == 8 && maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
-  if constexpr (K::DIRECT) {
+  if constexpr (FAM == JACC_FAM_NATIVE) {
+    __shared__ Plane<T, BX, BY, V> sm;
+    T m = T(0);
+    heat3d_body<T, BX, BY, V, JM_NATIVE>(u, v, p, p.zc, -1, m, sm);
+    bits = dbits((double)m);
+  } else if constexpr (K::DIRECT) {
     if (sizeof(T) == 8 && F >= 0) {
       u64 m = 0;
       if constexpr (sizeof(T) == 8) heat3d_direct<T, i64, BX, BY, V, JACC_DIRECT_PLANES>(u, v, p, m);
@@ -2504,7 +2516,12 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
   typedef Load3D<27, T, BX, BY, V, FAM, EDGE> K;
   double total = 0.0;
   const int F = (sizeof(T) == 8 && maxword && p.fpath != JACC_FP_NONE) ? fx_frac_bits(*maxword) : -1;
-  if constexpr (sizeof(T) == 8) {
+  if constexpr (FAM == JACC_FAM_NATIVE) {
+    __shared__ Plane<T, BX, BY, V> sm;
+    SumAcc<T> acc;
+    box27_body2<T, BX, BY, V>(u, v, p, p.zc, acc, resid != nullptr, sm);
+    total = acc.total();
+  } else if constexpr (sizeof(T) == 8) {
     typedef RingG<double, BX, BY, V> G;
     constexpr size_t SM_RING = (size_t)G::S * G::STAGE * 8, SM_PLANE = sizeof(Plane<double, BX, BY, 1>);
     __shared__ __align__(16) unsigned char raw[SM_RING > SM_PLANE ? SM_RING : SM_PLANE];
@@ -2652,7 +2669,7 @@ template <int STENCIL, class T, int BX, int BY, int V, int FAM, bool EDGE, bool 
   typedef Load3D<STENCIL, T, BX, BY, V, FAM, EDGE> K;
   static constexpr bool t32 = BX == 32 && BY == 4;
   static constexpr int heat = K::BULK ? (K::F64 ? (FOLDED ? 7 : 6) : 0) : K::RING ? (V == 1 || EDGE ? 5 : 6) : 0;
-  static constexpr int box = K::F64 ? (EDGE ? 0 : 4) : (V == 4 && !FOLDED ? 7 : 0);
+  static constexpr int box = FAM == JACC_FAM_NATIVE ? 0 : K::F64 ? (EDGE ? 0 : 4) : (V == 4 && !FOLDED ? 7 : 0);
   static constexpr bool wide = K::VEC && FAM == JACC_FAM_TABLE && !FOLDED && !EDGE;
   static constexpr int NT = BX * BY;
   static constexpr int wide5 = NT == 512 ? (K::F64 ? 2 : 3) : 0, wide7 = !K::F64 && NT == 256 ? 4 : 0,
@@ -2670,9 +2687,9 @@ template <int STENCIL, class T, int BX, int BY, int V, int FAM, bool EDGE, bool 
 // an argument.
 template <class A, class B, bool FIRST> struct PickT { typedef A type; };
 template <class A, class B> struct PickT<A, B, false> { typedef B type; };
-template <int STENCIL, class T, int BX, int BY, int V, int ZC> struct TableP {
+template <int STENCIL, class T, int BX, int BY, int V, int ZC, bool NATIVE = false> struct TableP {
   typedef Load3D<STENCIL, T, BX, BY, V, JACC_FAM_TABLE, false> K;
-  static constexpr bool FIXED = STENCIL == 5 ? V > 1 : !(K::RING || K::DIRECT);
+  static constexpr bool FIXED = NATIVE || (STENCIL == 5 ? V > 1 : !(K::RING || K::DIRECT));
   typedef typename PickT<JParamsZ<STENCIL == 5 ? ZC / 4 : ZC>, JParams, FIXED>::type type;
 };
 

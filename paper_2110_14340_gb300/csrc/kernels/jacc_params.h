@@ -19,6 +19,7 @@ typedef unsigned int u32;
 #define JACC_FAM_RING 2    // 3D: planes staged by asynchronous copies
 #define JACC_FAM_DIRECT 3  // 7-point: no staging (32 x 8 threads)
 #define JACC_FAM_BULK 4    // 3D, 16-byte columns: planes staged by bulk copies
+#define JACC_FAM_NATIVE 5  // FP64 arithmetic throughout (JACC_FP_NONE): a tile's rows or planes in registers
 
 // The 7-point table tiles that stage nothing, and the planes per thread of the
 // kernel that does not.
