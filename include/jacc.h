@@ -382,9 +382,9 @@ jacc_status jacc_sweep_coeffs(jacc_kernel k, void* u0, void* u1, int32_t nsweeps
  * FP64 5PT grids of at most 2^17 points that fit one cluster (see
  * JACC_SPEC_CLUSTER) run in one launch of it.  Otherwise it is one CUDA graph
  * (cached per kernel, fields, max_sweeps, tol and output arrays, dropped by
- * jacc_release) whose WHILE conditional node runs 16 sweeps a turn (4 of large
- * fields), each followed by a one-thread kernel that stores the residual and
- * tells the sweeps after it, and the loop, to stop.
+ * jacc_release) whose WHILE conditional nodes run 4 sweeps a turn, 16 from the
+ * 18th on (large fields 4 throughout), each followed by a one-thread kernel that
+ * stores the residual and tells the sweeps after it, and the loop, to stop.
  * 5PT and 7PT only (their residual is max |v - u|);
  * 27PT is JACC_ERR_UNSUPPORTED.  tol finite and >= 0, max_sweeps >= 1.
  *   resid_dev  (device, max_sweeps doubles, required): resid_dev[i] for each

@@ -92,7 +92,8 @@ jacc_status check_buffers(const Kernel& k, const void* a, const void* b);
 // Destroys k's cached jacc_sweep_until graphs.
 void free_until_graphs(Kernel& k);
 cudaError_t launch_until_check(double* slot, int* counter, int* stop, double* resid, double tol, int max_sweeps,
-                               cudaGraphConditionalHandle h_loop, cudaStream_t s);
+                               cudaGraphConditionalHandle h_loop, int until, cudaGraphConditionalHandle h_next,
+                               cudaStream_t s);
 cudaError_t launch_until_final(const int* counter, int* status, int recompute, cudaGraphConditionalHandle h_final,
                                cudaStream_t s);
 

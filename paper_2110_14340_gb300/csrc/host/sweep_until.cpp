@@ -7,10 +7,9 @@
 //          after the max-abs pre-pass) and a one-thread check kernel;
 //   WHILE  (condition set by the checks) an even number of sweeps u1 -> u0
 //          -> u1 ..., each followed by a check; the check that stops the loop
-//          sets a word that makes the rest of the body return at once (a
-//          conditional node costs several times the launches it guards: two
-//          sweeps per turn of the loop and an IF around the second took 24 us
-//          a sweep on small grids);
+//          sets a word that makes the rest of the body return at once.  Small
+//          fields have two such loops one after the other, of shorter and longer
+//          turns;
 //   F      a one-thread kernel that writes the sweep count and the result
 //          buffer and picks the final sweep;
 //   SWITCH the final sweep run again from the state before it with FP64
@@ -101,8 +100,23 @@ static jacc_status build_until(const Kernel& k, void* u0, void* u1, int32_t max_
   const u64* mw = fixed ? maxword : nullptr;
   jacc_status st = cuda_check(cudaGraphCreate(&ug.graph, 0), "cudaGraphCreate");
   if (st) return st;
-  cudaGraphConditionalHandle h_loop, h_final;
-  st = cuda_check(cudaGraphConditionalHandleCreate(&h_loop, ug.graph, 0, 0), "conditional handle");
+  // The loops in order: sweeps per turn, and the count at which the next loop
+  // takes over.  A sweep left in a turn after the stop costs about 2 us on small
+  // fields (6 on 160^3), a turn or a loop that is not entered 4, so the first
+  // turns are short and later ones long (256 x 192 FP32, us a call, turns of 16
+  // throughout / so: 2 sweeps 61 / 46, 5 64 / 50, 17 78 / 94, 400 1306 / 1328;
+  // 160^3 2 sweeps 159 / 68).  Fields whose sweeps dwarf a turn take 4 throughout.
+  struct Loop {
+    int sweeps, until;
+  };
+  static const Loop small[2] = {{4, 17}, {16, INT32_MAX}}, large[1] = {{4, INT32_MAX}};
+  const bool is_small = k.desc.nx * k.desc.ny * k.desc.nz < (int64_t(1) << 22);
+  const Loop* const loops = is_small ? small : large;
+  const int nloops = is_small ? 2 : 1;
+  cudaGraphConditionalHandle h_loop[3], h_final;
+  for (int l = 0; l < nloops && !st; ++l)  // a loop that no check reaches does not run
+    st = cuda_check(cudaGraphConditionalHandleCreate(&h_loop[l], ug.graph, 0, cudaGraphCondAssignDefault), "conditional handle");
+  h_loop[nloops] = h_loop[nloops - 1];  // never set: the last loop has no end but the stop
   if (!st) st = cuda_check(cudaGraphConditionalHandleCreate(&h_final, ug.graph, 3, cudaGraphCondAssignDefault),
                            "conditional handle");
   if (st) return st;
@@ -111,8 +125,10 @@ static jacc_status build_until(const Kernel& k, void* u0, void* u1, int32_t max_
   auto sweep = [&](const void* src, void* dst, double* r, int flags, const int* guard = nullptr) {
     return cuda_check(launch_sweep_kernel(k, src, dst, r, mw, flags, s, guard), "stencil launch");
   };
-  auto check = [&]() {
-    return cuda_check(launch_until_check(slot, counter, stop, resid, tol, max_sweeps, h_loop, s), "check launch");
+  auto check = [&](int l) {
+    return cuda_check(launch_until_check(slot, counter, stop, resid, tol, max_sweeps, h_loop[l], loops[l].until,
+                                         h_loop[l + 1], s),
+                      "check launch");
   };
   // A: zero the slots and the counter, pre-pass, first sweep, check
   cudaGraph_t gA = nullptr;
@@ -124,30 +140,30 @@ static jacc_status build_until(const Kernel& k, void* u0, void* u1, int32_t max_
       e = cuda_check(launch_maxabs(static_cast<const double*>(u0), k.desc.nx * k.desc.ny * k.desc.nz, maxword, s),
                      "max-abs pre-pass");
     if (!e) e = sweep(cu0, u1, slot, kFxIn);
-    if (!e) e = check();
+    if (!e) e = check(0);
     return e;
   });
   cudaGraphNode_t nA = nullptr, nW = nullptr, nF = nullptr, nS = nullptr;
   if (!st) st = add_child(ug.graph, nullptr, gA, &nA);
   cudaGraphDestroy(gA);  // the child node holds a copy
   if (st) return st;
-  // WHILE: pairs of u1 -> u0, check, u0 -> u1, check.  Small fields take 16
-  // sweeps per turn, fields whose sweeps dwarf a turn of the loop take 4.
-  cudaGraph_t* wb = nullptr;
-  st = add_conditional(ug.graph, nA, h_loop, cudaGraphCondTypeWhile, 1, &nW, &wb);
-  if (st) return st;
-  const int pairs = k.desc.nx * k.desc.ny * k.desc.nz < (int64_t(1) << 22) ? 8 : 2;
-  st = capture_into(wb[0], s, [&]() -> jacc_status {
-    jacc_status e = ok();
-    for (int i = 0; i < pairs && !e; ++i) {
-      e = sweep(cu1, u0, slot, 0, stop);
-      if (!e) e = check();
-      if (!e) e = sweep(cu0, u1, slot, 0, stop);
-      if (!e) e = check();
-    }
-    return e;
-  });
-  if (st) return st;
+  // WHILE loops: pairs of u1 -> u0, check, u0 -> u1, check
+  for (int l = 0; l < nloops; ++l) {
+    cudaGraph_t* wb = nullptr;
+    st = add_conditional(ug.graph, l ? nW : nA, h_loop[l], cudaGraphCondTypeWhile, 1, &nW, &wb);
+    if (st) return st;
+    st = capture_into(wb[0], s, [&]() -> jacc_status {
+      jacc_status e = ok();
+      for (int i = 0; i < loops[l].sweeps / 2 && !e; ++i) {
+        e = sweep(cu1, u0, slot, 0, stop);
+        if (!e) e = check(l);
+        if (!e) e = sweep(cu0, u1, slot, 0, stop);
+        if (!e) e = check(l);
+      }
+      return e;
+    });
+    if (st) return st;
+  }
   // F: status and the choice of the final sweep
   cudaGraph_t gF = nullptr;
   st = cuda_check(cudaGraphCreate(&gF, 0), "cudaGraphCreate");

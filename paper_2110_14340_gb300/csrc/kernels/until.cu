@@ -11,9 +11,9 @@ namespace {
 // resid[i], clear the slot for the next sweep and count the sweep.  Once a
 // residual reaches the tolerance, or max sweeps ran, the stop word is set: the
 // sweeps and checks left in the loop's body then return at once, and the loop
-// ends.
+// ends.  It also ends, and the next one begins, when `until` sweeps ran.
 __global__ void jacc_k_until_check(double* slot, int* counter, int* stop, double* resid, double tol, int max_sweeps,
-                                   cudaGraphConditionalHandle h_loop) {
+                                   cudaGraphConditionalHandle h_loop, int until, cudaGraphConditionalHandle h_next) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (__ldcg(stop)) return;
   const double r = __ldcg(slot);
@@ -23,7 +23,9 @@ __global__ void jacc_k_until_check(double* slot, int* counter, int* stop, double
   *counter = i + 1;
   const bool more = r > tol && i + 1 < max_sweeps;
   if (!more) *stop = 1;
-  cudaGraphSetConditional(h_loop, more ? 1u : 0u);
+  const bool here = i + 1 < until;
+  cudaGraphSetConditional(h_loop, more && here ? 1u : 0u);
+  if (!here) cudaGraphSetConditional(h_next, more ? 1u : 0u);
 }
 
 // After the loop: report the sweep count and the result buffer, and pick the
@@ -44,7 +46,8 @@ __global__ void jacc_k_until_final(const int* counter, int* status, int recomput
 namespace jacc {
 
 cudaError_t launch_until_check(double* slot, int* counter, int* stop, double* resid, double tol, int max_sweeps,
-                               cudaGraphConditionalHandle h_loop, cudaStream_t s) {
+                               cudaGraphConditionalHandle h_loop, int until, cudaGraphConditionalHandle h_next,
+                               cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(1);
   cfg.blockDim = dim3(1);
@@ -54,7 +57,8 @@ cudaError_t launch_until_check(double* slot, int* counter, int* stop, double* re
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, jacc_k_until_check, slot, counter, stop, resid, tol, max_sweeps, h_loop);
+  return cudaLaunchKernelEx(&cfg, jacc_k_until_check, slot, counter, stop, resid, tol, max_sweeps, h_loop, until,
+                            h_next);
 }
 
 cudaError_t launch_until_final(const int* counter, int* status, int recompute, cudaGraphConditionalHandle h_final,
