@@ -153,15 +153,28 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
   const int F = a.native ? -1 : fx_frac_bits(gmax);
   const bool fixed = F >= 0;
 
-  // load own rows and the two halo rows, converted to the working form
-  for (i64 lr = 0; lr < nr + 2; ++lr) {
-    const i64 g = r0 - 1 + lr;
-    if (g < 0 || g >= ny) continue;
-    for (i64 x = t; x < nx; x += NT) {
-      const double d = a.u[g * nx + x];
-      bufA[lr * pitch + x] = fixed ? (u64)fx_from(d, F) : dbits(d);
+  // f(local row, column) for the cells of local rows [lo, hi), NT at a time:
+  // narrow rows keep as many threads busy as wide ones (one sweep of 16 x 4000
+  // with a loop over rows 100 us, so 24; 256 x 192 26 and 24)
+  auto each_cell = [&](int lo, int hi, auto f) {
+    const int w = (int)nx, dr = NT / w, dc = NT % w;
+    int lr = lo + t / w, x = t % w;
+    while (lr < hi) {
+      f(lr, x);
+      lr += dr;
+      x += dc;
+      if (x >= w) {
+        x -= w;
+        ++lr;
+      }
     }
-  }
+  };
+  // load own rows and the two halo rows inside the grid, converted to the working form
+  const int lr_lo = r0 >= 1 ? 0 : 1, lr_hi = (int)(nr + (r1 < ny ? 2 : 1));
+  each_cell(lr_lo, nr ? lr_hi : 0, [&](int lr, int x) {
+    const double d = a.u[(r0 - 1 + lr) * nx + x];
+    bufA[lr * pitch + x] = fixed ? (u64)fx_from(d, F) : dbits(d);
+  });
   __syncthreads();
 
   int n = a.nsweeps;  // sweeps to run (UNTIL: at most; the count once it is known)
@@ -428,8 +441,9 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
       const int len = min(max(4, min(64, base >> 2)), n - base);
       u64* cur = (base & 1) ? bufB : bufA;
       if (base)  // the chunk's start (the first one's is the input)
-        for (i64 lr = 1; lr <= nr; ++lr)
-          for (i64 x = t; x < nx; x += NT) a.keep[(r0 - 1 + lr) * nx + x] = __longlong_as_double((i64)cur[lr * pitch + x]);
+        each_cell(1, (int)nr + 1, [&](int lr, int x) {
+          a.keep[(r0 - 1 + lr) * nx + x] = __longlong_as_double((i64)cur[lr * pitch + x]);
+        });
       if (hot)
         for (int i = 0; i < len; ++i) hot_sweep(base + i, i, i == len - 1);
       else
@@ -452,14 +466,11 @@ __global__ void __launch_bounds__(NT) jacc_k_jacobi_cluster(JClusterArgs a) {
       n = base + ran;
       cluster_sync();  // every CTA has read the chunk's maxima
       if (ran < len) {  // run the chunk again, up to the input of sweep n - 1
-        for (i64 lr = 0; lr < nr + 2; ++lr) {
-          const i64 g = r0 - 1 + lr;
-          if (g < 0 || g >= ny) continue;
-          for (i64 x = t; x < nx; x += NT) {
-            const double d = base ? __ldcg(a.keep + g * nx + x) : a.u[g * nx + x];
-            cur[lr * pitch + x] = (base == 0 && fixed) ? (u64)fx_from(d, F) : dbits(d);
-          }
-        }
+        each_cell(lr_lo, nr ? lr_hi : 0, [&](int lr, int x) {
+          const i64 at = (r0 - 1 + lr) * nx + x;
+          const double d = base ? __ldcg(a.keep + at) : a.u[at];
+          cur[lr * pitch + x] = (base == 0 && fixed) ? (u64)fx_from(d, F) : dbits(d);
+        });
         cluster_sync();
         if (hot)
           for (int k = base; k < n - 1; ++k) hot_sweep(k, 0, false);
