@@ -379,8 +379,8 @@ jacc_status jacc_sweep_coeffs(jacc_kernel k, void* u0, void* u1, int32_t nsweeps
  * count; §5.2 notes that Himeno reduces its error each iteration): sweeps
  * u0 -> u1 -> u0 ... until a sweep's residual is <= tol or max_sweeps sweeps
  * ran, with the loop and its exit test on the device; the host never waits.
- * FP64 5PT grids of at most 2^17 points that fit one cluster (see
- * JACC_SPEC_CLUSTER) run in one launch of it.  Otherwise it is one CUDA graph
+ * FP64 5PT grids of at most 2^17 points (native arithmetic: 2^15) that fit one
+ * cluster (see JACC_SPEC_CLUSTER) run in one launch of it.  Otherwise it is one CUDA graph
  * (cached per kernel, fields, max_sweeps, tol and output arrays, dropped by
  * jacc_release) whose WHILE conditional nodes run 4 sweeps a turn, 16 from the
  * 18th on (large fields 4 throughout), each followed by a one-thread kernel that

@@ -76,8 +76,13 @@ jacc_status add_child(cudaGraph_t g, cudaGraphNode_t dep, cudaGraph_t child, cud
 // 5-point grid of at most 2^17 points that fits: results are the same bit for
 // bit, and a sweep in the cluster costs 1.0 to 2.4 us (64^2 to 320^2) where
 // one in the graph costs at least two kernel launches.  Larger grids keep the
-// whole GPU: at 400^2 the cluster's 16 SMs are the limit.
+// whole GPU: at 400^2 the cluster's 16 SMs are the limit.  Native arithmetic
+// reaches that limit of its FP64 pipe much sooner (100 sweeps in the cluster
+// and in the graph, us: 160^2 477 and 637, 192^2 680 and 654, 362^2 2123 and
+// 645), whatever the handle.
 static int until_cluster(Kernel& k) {
+  const bool native = k.params.fpath == JACC_FP_NONE;
+  if (native && k.desc.nx * k.desc.ny > (int64_t(1) << 15)) return 0;
   if (k.cluster_nc > 0) return k.cluster_nc;
   if (k.desc.stencil != JACC_STENCIL_5PT || k.desc.dtype != JACC_F64) return 0;
   if (k.desc.nx * k.desc.ny > (int64_t(1) << 17)) return 0;
