@@ -226,17 +226,6 @@ static bool native_fp64(const jacc_kernel_desc& d, int fpath) {
   return d.dtype == 64 && d.stencil != 19 && fpath == JACC_FP_NONE;
 }
 
-// The default tile of native FP64 sweeps, bound by the FP64 pipe.  2D: 16-byte
-// columns and four rows per thread from 2^19 points on, where the grid leaves
-// L2 (4096^2: 259 us a sweep, 288 by strips); below, more and narrower CTAs.
-static int default_tile_native(const jacc_kernel_desc& d) {
-  if (d.stencil == 5) {
-    const int t = d.nx * d.ny < (int64_t(1) << 19) ? 8 : d.nx % 2 ? 16 : 17;
-    if (tile_valid(d, t)) return t;
-  }
-  return default_tile(d);
-}
-
 // CTAs that a grid holds at most in y and in z.
 constexpr int64_t kGridYZ = 65535;
 
@@ -253,10 +242,13 @@ static bool direct_fits(const jacc_kernel_desc& d) {
 // sweep without staging, 22.4 with the ring; 512^3 798 and 480).
 static int table_family(const jacc_kernel_desc& d, int tile, int fpath) {
   const TileCfg& c = kTiles[tile];
-  if (native_fp64(d, fpath)) return JACC_FAM_NATIVE;
-  const bool direct = d.stencil == 7 && JACC_DIRECT_TILE(c.bx, c.by, c.vec16 ? 2 : 1);
-  const bool large = d.dtype == 64 && d.nx * d.ny * d.nz > (int64_t(1) << 20);
-  return direct && (large || !direct_fits(d)) ? JACC_FAM_RING : JACC_FAM_TABLE;
+  const bool direct = d.stencil == 7 && JACC_DIRECT_TILE(c.bx, c.by, c.vec16 ? 2 : 1), fits = direct_fits(d);
+  const int64_t n = d.nx * d.ny * d.nz;
+  // native FP64, us a sweep of tile 4 without staging and with its planes in
+  // registers: 33^3 19 / 22, 101^3 40 / 43, 128^3 52 / 58, 192 x 160 x 144 122 / 109
+  if (native_fp64(d, fpath)) return direct && fits && n <= (int64_t(1) << 21) ? JACC_FAM_TABLE : JACC_FAM_NATIVE;
+  const bool large = d.dtype == 64 && n > (int64_t(1) << 20);
+  return direct && (large || !fits) ? JACC_FAM_RING : JACC_FAM_TABLE;
 }
 
 // Whether the planes per CTA are fitted to the grid: kernels of the library's
@@ -278,18 +270,38 @@ static bool fits_planes(const jacc_kernel_desc& d, int tile, int fam, bool fit) 
 // FP32 768^3 577 / 610, 512^3 195 / 179), of the precompiled ones only the FP32
 // 7-point kernel (512^3 164 / 170); the rest asynchronous copies (precompiled,
 // ring / bulk: 7-point FP64 512^3 396 / 480, 27-point FP32 768^3 604 / 748).
-static int default_family(const jacc_kernel_desc& d, int tile) {
+static int default_family(const jacc_kernel_desc& d, int tile, bool native) {
   if (d.tblock > 1 || d.stencil == 19) return JACC_FAM_TABLE;
   if (d.stencil == 5) return JACC_FAM_STRIP;
   const bool vec = kTiles[tile].vec16, f64 = d.dtype == 64;
   const int64_t n = d.nx * d.ny * d.nz;
   if (d.stencil == 7) {
     const int64_t direct = vec ? (f64 ? int64_t(1) << 21 : int64_t(1) << 22) : (f64 ? int64_t(1) << 20 : int64_t(5) << 17);
-    if (n <= direct && direct_fits(d)) return JACC_FAM_DIRECT;
+    if (n <= (native ? int64_t(1) << 24 : direct) && direct_fits(d)) return JACC_FAM_DIRECT;  // native: see default_tile_native
   }
   const bool bulk = d.stencil == 7 ? n * (f64 ? 8 : 4) >= (int64_t(1) << 28) : !f64 && n * 4 >= (int64_t(1) << 30);
   const bool pays = (d.flags & JACC_SPEC_JIT) || (d.stencil == 7 && !f64);
   return tile == 3 && bulk && pays ? JACC_FAM_BULK : JACC_FAM_RING;
+}
+
+// The library's own choice for native FP64 sweeps: the tile, and whether it is
+// left as it is (JACC_FAM_NATIVE) or given to the family and march of the fixed-
+// point sweeps of the same size (*own).  The latter bring more, shorter CTAs,
+// which small grids need, but more work for the FP64 pipe, which bounds large
+// ones (us a sweep, own / native: 5-point 256^2 3.2 / 5.0, 100 x 6000 14 / 26,
+// 1024^2 23 / 22, 4096^2 288 / 259; 7-point without staging 64^3 9.0 / 22, 128^3
+// 48 / 67, 192 x 160 x 144 96 / 107, 256^3 353 / 370;
+// 27-point 64^3 23 / 27, 97 x 81 x 85 52 / 46).
+static int default_tile_native(const jacc_kernel_desc& d, bool* own) {
+  const int tile = default_tile(d);
+  const int64_t n = d.nx * d.ny * d.nz;
+  if (d.stencil == 5) {
+    *own = n < (int64_t(1) << 20) || d.nx <= 384;  // 256 columns a CTA otherwise
+    const int rows = d.nx % 2 ? 16 : 17;  // 128 x 2 threads, four rows each
+    return !*own && tile_valid(d, rows) ? rows : tile;
+  }
+  *own = d.stencil == 7 ? default_family(d, tile, true) == JACC_FAM_DIRECT : n <= (int64_t(1) << 18);
+  return tile;
 }
 
 // What a CTA of kernel family `fam` covers per plane (columns, rows), and how
@@ -481,7 +493,7 @@ static std::string jit_source(const Kernel& k) {
   };
   std::string src = std::string(device_source()) + fold;
   src += kernel("jacc_jit", k.fam == JACC_FAM_DIRECT ? 256 : c.bx * c.by, bound(k.fam, false), call(k.fam, false, "flags"));
-  if (k.desc.dtype == 64 && k.fam != JACC_FAM_NATIVE) {
+  if (k.desc.dtype == 64 && p.fpath != JACC_FP_NONE) {
     src += kernel("jacc_jit_out", c.bx * c.by, bound(k.fam, true), call(k.fam, true, "flags"));
     src += kernel("jacc_jit_last", c.bx * c.by, bound(k.fam, true), call(k.fam, true, "JFX_OUT_F64"));
   }
@@ -542,8 +554,9 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
         kTiles[tile].by == 4 && desc->nx * desc->ny * desc->nz >= (int64_t(1) << 25) && tile_valid(*desc, tile | 1))
       tile |= 1;
     if (tile < 0 || !tile_valid(*desc, tile)) {
-      tile = native ? default_tile_native(*desc) : default_tile(*desc);
-      fit = desc->stencil != 19 && desc->tblock <= 1 && !native;
+      bool own = true;
+      tile = native ? default_tile_native(*desc, &own) : default_tile(*desc);
+      fit = desc->stencil != 19 && desc->tblock <= 1 && own;
     }
   }
   if (!tile_valid(*desc, tile))
@@ -573,14 +586,14 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   p.c1 = desc->coeffs[1];
   p.c2 = desc->coeffs[2];
   p.c3 = desc->coeffs[3];
-  k->fam = fit ? default_family(*desc, tile) : table_family(*desc, tile, p.fpath);
+  k->fam = fit ? default_family(*desc, tile, native) : table_family(*desc, tile, p.fpath);
   const int fam = k->fam;
   // fixed-point sequences convert in their first and last sweeps, which have a kernel of their own
   const bool edge = desc->dtype == 64 && !native;
   k->block_out = dim3(c.bx, c.by, 1);
   k->block = fam == JACC_FAM_DIRECT ? dim3(32, 8, 1) : k->block_out;
   if (!(desc->flags & JACC_SPEC_JIT) && desc->stencil != 19 && desc->tblock <= 1) {
-    k->func = native ? native_entry(desc->stencil, tile)
+    k->func = fam == JACC_FAM_NATIVE  ? native_entry(desc->stencil, tile)
               : fam == JACC_FAM_TABLE ? table_entry(desc->stencil, desc->dtype, tile, false)
                                       : lib_entry(*desc, p, fit ? fam : 5, k->vec > 1);
     if (fam == JACC_FAM_TABLE && p.fpath == JACC_FP_W32) k->func = jacc_tab_27_64_w32[tile];
