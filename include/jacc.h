@@ -205,12 +205,12 @@ jacc_status jacc_region_boxes_affine(int32_t nloops, const jacc_loop_affine* loo
  *
  * tile_id selects one of JACC_NUM_TILES tile configurations (see
  * jacc_tile_info), or -1 to let the library choose: the autotuner's cached
- * pick for this shape if one exists (large 7PT FP64 grids with JACC_SPEC_JIT:
- * with 16-byte columns where the pick has scalar ones), else a kernel of the library's own for
- * this size, type and row alignment, which may load its input in another way
- * than the tile that jacc_kernel_info names (strips of rows for 5PT, planes
- * staged by asynchronous or bulk copies or not at all for 7PT and 27PT) and
- * marches as many planes or rows per CTA as fill the GPU.
+ * pick for this shape if it was timed ahead of the library's own kernel (by 3 %
+ * or more), else that kernel, made for this size, type and row alignment, which
+ * may load its input in another way than the tile that jacc_kernel_info names
+ * (a cached pick, or the tile the kernel is derived from): strips of rows for
+ * 5PT, planes staged by asynchronous or bulk copies or not at all for 7PT and
+ * 27PT; it marches as many planes or rows per CTA as fill the GPU.
  *
  * flags: JACC_SPEC_JIT compiles a variant with the extents and coefficients
  * folded in as constants (NVRTC, sm_103a; cached in memory and, if the
@@ -470,8 +470,10 @@ jacc_status jacc_sched_release(jacc_sched s);
  * on the caller's fields u0/u1 (their contents change) once to warm up and
  * `reps` more times, timed with CUDA events on `stream`; out->ms[t] is the
  * median time per sweep (infinity and valid[t] = 0 for tiles that do not fit
- * the shape).  The fastest tile is remembered for the shape, so that
- * jacc_specialize with tile_id = -1 uses it.  Synchronises `stream`. */
+ * the shape).  The fastest tile is remembered for the shape, and the library's
+ * own kernel is timed in the same way: jacc_specialize with tile_id = -1 uses
+ * the tile if it is ahead of that kernel by 3 % or more, and otherwise only
+ * names it (jacc_kernel_info).  Synchronises `stream`. */
 typedef struct {
   double ms[JACC_NUM_TILES];    /* median milliseconds per sweep              */
   int32_t valid[JACC_NUM_TILES];
@@ -485,7 +487,7 @@ jacc_status jacc_autotune(const jacc_kernel_desc* desc, void* u0, void* u1, int3
 /* jacc_autotune restricted to the ntiles tile ids in `tiles` (host array,
  * each in [0, JACC_NUM_TILES)): only those are timed (out->valid[t] = 1 for
  * the timed tiles that fit the shape, 0 for all others), and the fastest of
- * them is remembered for the shape.  INVALID_ARG for an empty list or an id
+ * them is remembered for the shape, under the same condition.  INVALID_ARG for an empty list or an id
  * out of range, UNSUPPORTED if none of them fits. */
 jacc_status jacc_autotune_tiles(const jacc_kernel_desc* desc, void* u0, void* u1, int32_t sweeps_per_rep,
                                 int32_t reps, uintptr_t stream, const int32_t* tiles, int32_t ntiles,
@@ -522,7 +524,8 @@ jacc_status jacc_autotune_forget(void);
  * choose      : the model's tile for `desc`; falls back to jacc_autotune on
  *               u0/u1 (needed then) when the side lies outside the range or
  *               the top-2 gap is below the margin.  *used_fallback tells
- *               which.  The chosen tile is remembered for the shape.
+ *               which.  The chosen tile is remembered for the shape; without
+ *               a timing against the library's own kernel it is only named.
  * choose_topk : the model as a filter: the k valid tiles with the lowest
  *               predicted time for `desc` are timed on u0/u1 (required; their
  *               contents change) by jacc_autotune_tiles and the fastest is

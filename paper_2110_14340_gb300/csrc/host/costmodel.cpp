@@ -282,7 +282,10 @@ extern "C" jacc_status jacc_costmodel_choose(jacc_costmodel h, const jacc_kernel
   }
   *tile = pick;
   *used_fallback = 0;
-  remember_tile(*desc, pick);
+  // named by later handles; not timed against the library's own kernel, it does not displace it
+  TunedPick remembered;
+  remembered.tile = pick;
+  remember_pick(*desc, remembered);
   return ok();
 }
 

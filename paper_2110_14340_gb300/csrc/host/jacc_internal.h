@@ -50,6 +50,7 @@ struct Kernel {
   std::string key;
   JParams params{};
   int tile = 0;
+  int named = 0;                // the tile that jacc_kernel_info names (a remembered pick that is not ahead, else `tile`)
   int elem = 8;                 // bytes per element
   int vec = 1;                  // elements per thread in x
   bool jit = false;
@@ -124,10 +125,18 @@ const char* params_source();
 std::mutex& global_mutex();
 
 // Tile validity for a descriptor (vector width and grid limits) and the
-// default tile; the autotuner's remembered pick for a shape (-1 if none).
+// default tile.
 bool tile_valid(const jacc_kernel_desc& d, int t);
 int default_tile(const jacc_kernel_desc& d);
-int tuned_tile(const jacc_kernel_desc& d);
-void remember_tile(const jacc_kernel_desc& d, int tile);
+// What the tuner remembers of a shape: the fastest tile (-1: nothing), and
+// whether it was timed ahead of the library's own kernel.
+struct TunedPick {
+  int tile = -1;
+  bool ahead = false;
+};
+TunedPick tuned_pick(const jacc_kernel_desc& d);
+void remember_pick(const jacc_kernel_desc& d, const TunedPick& p);
+// jacc_specialize with tile_id = -1 as if nothing were remembered.
+jacc_status specialize_own(const jacc_kernel_desc& desc, jacc_kernel* out);
 
 }  // namespace jacc

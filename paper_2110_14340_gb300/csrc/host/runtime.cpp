@@ -350,12 +350,12 @@ bool tile_valid(const jacc_kernel_desc& d, int t) {
   return gx < (1ll << 31) && gy <= kGridYZ && gz <= kGridYZ;
 }
 
-static std::string key_of(const jacc_kernel_desc& d, int tile, bool fit) {
+static std::string key_of(const jacc_kernel_desc& d, int tile, bool fit, int named) {
   jacc_kernel_desc c = d;
   c.tile_id = tile;
   c.reserved = 0;
   if (c.tblock == 0) c.tblock = 1;
-  return std::string(reinterpret_cast<const char*>(&c), sizeof(c)) + (fit ? "f" : "t");
+  return std::string(reinterpret_cast<const char*>(&c), sizeof(c)) + (fit ? "f" : "t") + std::to_string(named);
 }
 
 // Planes per CTA (3D) or rows per warp (2D) of a kernel that takes what fits
@@ -532,36 +532,45 @@ extern "C" jacc_status jacc_tile_info(int32_t tile_id, jacc_tile* out) {
   return ok();
 }
 
+static jacc_status specialize(const jacc_kernel_desc* desc, const TunedPick& pick, jacc_kernel* out);
+
 extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel* out) {
   if (!desc || !out) return fail(JACC_ERR_INVALID_ARG, "NULL descriptor or output");
-  jacc_status st = validate(*desc);
-  if (st) return st;
+  const jacc_status st = validate(*desc);
+  return st ? st : specialize(desc, desc->tile_id < 0 && desc->stencil != 19 ? tuned_pick(*desc) : TunedPick(), out);
+}
+
+jacc_status jacc::specialize_own(const jacc_kernel_desc& desc, jacc_kernel* out) {
+  const jacc_status st = validate(desc);
+  return st ? st : specialize(&desc, TunedPick(), out);
+}
+
+// pick: the autotuner's, where no tile is asked for.
+static jacc_status specialize(const jacc_kernel_desc* desc, const TunedPick& pick, jacc_kernel* out) {
+  jacc_status st = ok();
   JParams plan{};
   plan_fixed(*desc, plan);
   const bool native = native_fp64(*desc, plan.fpath);
   int tile = desc->tile_id;
+  int named = -1;    // the tile that jacc_kernel_info names, if not the kernel's
   bool fit = false;  // the library picks the kernel family and the march along with the tile
   if (desc->stencil == 19) {
     tile = 3;  // the kernel's one configuration: 32 x 4 threads, 16-byte columns, 40-plane march
   } else if (tile < 0) {
-    tile = tuned_tile(*desc);
-    // Picks are timed on precompiled kernels, where the 32 x 4 scalar tile's
-    // asynchronous copies beat the bulk copies of the same tile with 16-byte
-    // columns; folded, the order is the other way round for fields that stream
-    // from HBM (512^3 FP64, us a sweep, scalar and 16-byte: precompiled 385 and
-    // 413, folded 380 and 355).
-    if (tile >= 0 && (desc->flags & JACC_SPEC_JIT) && desc->stencil == 7 && desc->dtype == 64 && kTiles[tile].bx == 32 &&
-        kTiles[tile].by == 4 && desc->nx * desc->ny * desc->nz >= (int64_t(1) << 25) && tile_valid(*desc, tile | 1))
-      tile |= 1;
-    if (tile < 0 || !tile_valid(*desc, tile)) {
+    const bool picked = pick.tile >= 0 && tile_valid(*desc, pick.tile);
+    if (picked && (pick.ahead || desc->tblock > 1)) {
+      tile = pick.tile;
+    } else {
       bool own = true;
       tile = native ? default_tile_native(*desc, &own) : default_tile(*desc);
-      fit = desc->stencil != 19 && desc->tblock <= 1 && own;
+      fit = desc->tblock <= 1 && own;
+      if (picked) named = pick.tile;
     }
   }
   if (!tile_valid(*desc, tile))
     return fail(JACC_ERR_INVALID_ARG, "tile " + std::to_string(tile) + " does not fit this shape (x vector width)");
-  const std::string key = key_of(*desc, tile, fit);
+  if (named < 0) named = tile;
+  const std::string key = key_of(*desc, tile, fit, named);
   std::lock_guard<std::mutex> lock(global_mutex());
   auto it = cache().find(key);
   if (it != cache().end()) {
@@ -574,6 +583,7 @@ extern "C" jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel
   k->desc.tile_id = tile;
   k->key = key;
   k->tile = tile;
+  k->named = named;
   k->elem = desc->dtype / 8;
   const TileCfg& c = kTiles[tile];
   k->vec = c.vec16 ? 16 / k->elem : 1;
@@ -712,7 +722,7 @@ extern "C" jacc_status jacc_kernel_set_wait(jacc_kernel h, int32_t timeout_ms, i
 extern "C" jacc_status jacc_kernel_info(jacc_kernel h, jacc_kernel_info_t* out) {
   if (!h || !out) return fail(JACC_ERR_INVALID_ARG, "NULL handle or output");
   const Kernel& k = *reinterpret_cast<Kernel*>(h);
-  out->tile_id = k.tile;
+  out->tile_id = k.named;
   out->jit = k.jit ? 1 : 0;
   out->fixed_point = k.params.fpath != JACC_FP_NONE ? 1 : 0;
   out->tblock = k.tblock;
