@@ -254,8 +254,9 @@ static int table_family(const jacc_kernel_desc& d, int tile, int fpath) {
 // Whether the planes per CTA are fitted to the grid: kernels of the library's
 // choice, and the FP64 scalar 7-point tiles, whose ring covers four rows per
 // thread: with all of the tile's planes small grids do not fill the GPU (us a
-// sweep, all / fitted: 64 x 60 x 62 tile 10 37.9 / 6.4, 192 x 160 x 144 39.7 /
-// 22.2; large grids take all of them either way).
+// sweep, all / fitted, but with no fewer points per CTA than one row per thread
+// had: 64 x 60 x 62 tile 10 37.9 / 14.9, 192 x 160 x 144 39.7 / 20.6; large
+// grids take all of them either way).
 static bool fits_planes(const jacc_kernel_desc& d, int tile, int fam, bool fit) {
   return fit || (d.stencil == 7 && d.dtype == 64 && !kTiles[tile].vec16 && fam != JACC_FAM_NATIVE);
 }
@@ -615,7 +616,9 @@ static jacc_status specialize(const jacc_kernel_desc* desc, const TunedPick& pic
   p.zc = plane_chunk(*desc, tile, fam);
   k->grid = k->grid_out = cta_grid(*desc, cta_tile(*desc, tile, fam, edge, p.zc));
   if (fits_planes(*desc, tile, fam, fit)) {
-    p.zc = fitted_chunk(*k, p.zc);
+    // a table tile keeps its points per CTA, and with them the tiles their order
+    const int least = fit ? 1 : p.zc / JACC_RING_ROWS(c.bx, c.by);
+    p.zc = std::max(fitted_chunk(*k, p.zc), least);
     if (desc->stencil == 5)
       while ((desc->ny + c.by * p.zc - 1) / (c.by * p.zc) > kGridYZ) p.zc *= 2;  // the grid's limit
   }
