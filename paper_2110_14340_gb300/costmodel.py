@@ -85,8 +85,36 @@ class Buffers:
         return a[:n].view(*s), b[:n].view(*s)
 
 
+def time_sweeps(k, u0, u1, sweeps=4, reps=5):
+    """Milliseconds per sweep on the device: the median of `reps` graph-launched sequences after one to
+    warm up, each queued behind a pause so that the host's launch latency does not count."""
+    import torch
+    ms = []
+    for _ in range(reps + 1):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda._sleep(200000)
+        e0.record()
+        jacc.sweep(k, u0, u1, sweeps)
+        e1.record()
+        e1.synchronize()
+        ms.append(e0.elapsed_time(e1) / sweeps)
+    return float(np.median(ms[1:]))
+
+
+def time_own(stencil, dtype, shape, u0, u1, best_tile, best_ms, reps=5):
+    """Milliseconds per sweep of the kernel that the library chooses by itself: best_ms times its ratio to
+    the best tile, both timed here."""
+    jacc.autotune_forget()
+    args = dict(stencil=stencil, dtype=dtype, nx=shape[0], ny=shape[1], nz=shape[2], coeffs=coeffs_for(stencil))
+    own, tile = jacc.Kernel(**args), jacc.Kernel(tile_id=best_tile, **args)
+    ratio = time_sweeps(own, u0, u1, reps=reps) / time_sweeps(tile, u0, u1, reps=reps)
+    own.release()
+    tile.release()
+    return best_ms * ratio
+
+
 def collect(queries, bufs, reps=5, log=None):
-    """queries: [(stencil, dtype, side)] -> list of dict(stencil, dtype, side, ms[24], valid[24])."""
+    """queries: [(stencil, dtype, side)] -> list of dict(stencil, dtype, side, ms[24], valid[24], own_ms)."""
     table = []
     for i, (st, dt, side) in enumerate(queries):
         nx, ny, nz = shape_for(st, side)
@@ -95,7 +123,8 @@ def collect(queries, bufs, reps=5, log=None):
         # intermediate sweeps that dominate long runs
         r = jacc.autotune(dict(stencil=st, dtype=dt, nx=nx, ny=ny, nz=nz, coeffs=coeffs_for(st)), u0, u1,
                           sweeps_per_rep=4, reps=reps)
-        table.append(dict(stencil=st, dtype=dt, side=side, ms=r["ms"], valid=r["valid"]))
+        own = time_own(st, dt, (nx, ny, nz), u0, u1, r["best_tile"], r["best_ms"], reps)
+        table.append(dict(stencil=st, dtype=dt, side=side, ms=r["ms"], valid=r["valid"], own_ms=own))
         if log:
             log(f"[{i + 1}/{len(queries)}] {st}pt f{dt} side {side}: best tile {r['best_tile']} {r['best_ms']:.4f} ms")
     return table
@@ -107,14 +136,9 @@ def summary(r):
                 max=float(np.max(r)), exact_best=float(np.mean(r == 0.0)))
 
 
-def library_default_tile(q):
-    """The tile jacc_specialize picks with tile_id = -1 and no remembered autotuner pick."""
-    jacc.autotune_forget()
-    nx, ny, nz = shape_for(q["stencil"], q["side"])
-    k = jacc.Kernel(q["stencil"], q["dtype"], nx, ny, nz, coeffs=coeffs_for(q["stencil"]))
-    t = k.info()["tile_id"]
-    k.release()
-    return t
+def own_regret(table):
+    """Per row that has one: time of the library's own kernel / best tile's - 1."""
+    return [q["own_ms"] / min(m for m, v in zip(q["ms"], q["valid"]) if v) - 1.0 for q in table if "own_ms" in q]
 
 
 def search_ms(q):
@@ -125,9 +149,11 @@ def search_ms(q):
 def baselines(train_table, test_table):
     """Regret of the methods without the model on the held-out tables."""
     ft = jacc.fixed_tile(train_table)
-    lib = [library_default_tile(q) for q in test_table]
-    return dict(fixed_tile=dict(tile=ft, **summary(jacc.regret(test_table, [ft] * len(test_table)))),
-                library_default_tile=summary(jacc.regret(test_table, lib)))
+    out = dict(fixed_tile=dict(tile=ft, **summary(jacc.regret(test_table, [ft] * len(test_table)))))
+    own = own_regret(test_table)
+    if own:  # tables of an earlier collection may lack it
+        out["library_own_kernel"] = summary(own)
+    return out
 
 
 def evaluate(model, train_table, test_table, fallback_fraction=0.25):
