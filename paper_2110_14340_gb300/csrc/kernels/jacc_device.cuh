@@ -231,7 +231,6 @@ JD void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 JD bool stopped(const int* stop) {
   return stop && __syncthreads_or(threadIdx.x == 0 && threadIdx.y == 0 && __ldcg(stop) != 0);
 }
-JD double fabs_bits_free(double d) { return __longlong_as_double(__double_as_longlong(d) & 0x7fffffffffffffffLL); }
 
 // FP32 error-free sum (Knuth TwoSum) accumulated as hi + lo.
 JD void two_sum_acc(float& hi, float& lo, float x) {
@@ -769,7 +768,11 @@ template <class T, int BX, int BY, int CH, int V = 1> struct RingG {
   static constexpr int NCH = W / CH, NTOT = NCH * R;        // copies per row, per plane
   static constexpr int PER = (NTOT + NT - 1) / NT;          // copies per thread
   static constexpr int S0 = 46080 / (STAGE * (int)sizeof(T));
-  static constexpr int S = S0 < 3 ? 3 : (S0 > 6 ? 6 : S0);  // stages, at most 45 KB
+  // Stages: what 45 KB hold, but 3 at least (the march needs that many) and 6 at
+  // most.  The widest tiles, FP64 of 64 x 8 and 128 x 4 threads with 16-byte
+  // columns, take 57024 and 62400 bytes so: three CTAs an SM.
+  static constexpr int S = S0 < 3 ? 3 : (S0 > 6 ? 6 : S0);
+  static_assert(S * STAGE * (int)sizeof(T) <= 62400, "static shared memory of a CTA");
 };
 
 template <int BYTES> JD void cpa_copy(void* dst, const void* src) {
@@ -1213,9 +1216,6 @@ JD void box27_tb_entry(const float* __restrict__ u, float* __restrict__ v, const
 
 JD i64 bits_i64(double d) { return (i64)__double_as_longlong(d); }
 JD double i64_bits(i64 q) { return __longlong_as_double(q); }
-
-// Round q * 2^-k to the nearest integer (ties up), k in [0, 62].
-JD i64 fx_round_shift(i64 q, int k) { return k ? ((q + ((i64)1 << (k - 1))) >> k) : q; }
 
 // (x + 2^(k-1)) >> k for a 128-bit x whose result fits in int64, k in [0, 62].
 JD i64 fx128_round_shift(s128 x, int k) {
@@ -2160,8 +2160,8 @@ template <class P> JD i64 box27_weigh(const P& p, i64 c, i64 f, i64 e, i64 g, s1
 // 383, rows of odd length, 447 us a sweep with planes loaded through registers
 // one step ahead, 227 here).
 template <class T, int BX, int BY, int CH, bool EDGE, class P>
-JD void box27r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, const JParams& rt, int F, int flags,
-                    bool want_sum, s128& acc, SumAcc<float>& acc32, T* sm) {
+JD void box27r_body(const T* __restrict__ u, T* __restrict__ v, const P& p, int F, int flags, bool want_sum, s128& acc,
+                    SumAcc<float>& acc32, T* sm) {
   typedef RingG<T, BX, BY, CH> G;
   constexpr bool FX = sizeof(T) == 8;
   typedef typename WT<T, FX ? JM_FIXED : JM_NATIVE>::type W;
@@ -2536,7 +2536,7 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
       s128 acc;
       acc.lo = acc.hi = 0ull;
       SumAcc<float> none;
-      box27r_body<double, BX, BY, V, EDGE>(u, v, p, rt, F, flags, false, acc, none, reinterpret_cast<double*>(raw));
+      box27r_body<double, BX, BY, V, EDGE>(u, v, p, F, flags, false, acc, none, reinterpret_cast<double*>(raw));
       total = fx128_to(acc, F);
     } else {
       SumAcc<T> acc;
@@ -2555,7 +2555,7 @@ JD void box27_entry(const T* __restrict__ u, T* __restrict__ v, const P& p, cons
     __shared__ __align__(16) float sm[G::S * G::STAGE];
     SumAcc<float> acc;
     s128 none;
-    box27r_body<float, BX, BY, V, false>(u, v, p, rt, -1, 0, resid != nullptr, none, acc, sm);
+    box27r_body<float, BX, BY, V, false>(u, v, p, -1, 0, resid != nullptr, none, acc, sm);
     total = acc.total();
   } else {
     __shared__ Plane<T, BX, BY, V> sm;
