@@ -770,7 +770,7 @@ template <class T, int BX, int BY, int CH, int V = 1> struct RingG {
   static constexpr int S0 = 46080 / (STAGE * (int)sizeof(T));
   // Stages: what 45 KB hold, but 3 at least (the march needs that many) and 6 at
   // most.  The widest tiles, FP64 of 64 x 8 and 128 x 4 threads with 16-byte
-  // columns, take 57024 and 62400 bytes so: three CTAs an SM.
+  // columns, take 57024 and 62400 bytes so.
   static constexpr int S = S0 < 3 ? 3 : (S0 > 6 ? 6 : S0);
   static_assert(S * STAGE * (int)sizeof(T) <= 62400, "static shared memory of a CTA");
 };
