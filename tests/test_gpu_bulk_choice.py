@@ -14,7 +14,7 @@ W = tuple(float(w) for w in inputs.box27_weights())
 # from 2^28 bytes a field on (7-point; FP64 folded only), or 2^30 (27-point FP32,
 # folded); chunks of 16 planes (FP32 7-point), 40 and 32
 @pytest.mark.parametrize("stencil,dtype,nx,ny,nz,planes,jit", [
-    (7, 32, 512, 256, 513, 16, False), (7, 32, 512, 256, 513, 16, True), (7, 64, 512, 256, 281, 40, True),
+    (7, 32, 512, 256, 513, 16, False), (7, 32, 512, 256, 513, 16, True), (7, 64, 512, 256, 361, 40, True),
     (27, 32, 1024, 512, 513, 32, True),
 ])
 def test_bulk_copy_choice_equals_tile_3(stencil, dtype, nx, ny, nz, planes, jit):
