@@ -280,11 +280,13 @@ jacc_status jacc_specialize(const jacc_kernel_desc* desc, jacc_kernel* out);
 jacc_status jacc_kernel_info(jacc_kernel k, jacc_kernel_info_t* out);
 jacc_status jacc_release(jacc_kernel k);
 
-/* Device status of a handle's launches (no counterpart in the paper).  The
- * 7PT and 27PT FP32 kernels of explicit tiles with 16-byte columns (and those
- * that the library chooses for fields that stream from HBM) stage their input
- * planes in shared memory with bulk copies and wait for them on mbarriers;
- * each such wait is bounded (default 2 s).  Other kernels have no such waits.  A wait that runs out writes JACC_ERR_TIMEOUT to the
+/* Device status of a handle's launches (no counterpart in the paper).  Kernels
+ * that stage their input planes in shared memory with bulk copies wait for them
+ * on mbarriers, and each such wait is bounded (default 2 s): 7PT (FP32, and FP64
+ * in fixed point) and 27PT FP32 with the 16-byte columns of an explicit tile, and
+ * where the library chooses them for fields that stream from HBM; the 19PT
+ * kernel; and the two-sweep 27PT kernel (tblock = 2).  The other kernels wait on
+ * no mbarrier.  A wait that runs out writes JACC_ERR_TIMEOUT to the
  * handle's device status word and its CTA returns early, so the output of
  * that launch is incomplete.  jacc_kernel_status synchronises the device,
  * stores the word (JACC_OK or JACC_ERR_TIMEOUT) in *status and clears it.
