@@ -122,8 +122,10 @@ static jacc_status autotune_subset(const jacc_kernel_desc* desc, void* u0, void*
     if (!st) {
       st = time_sweeps(k, u0, u1, sweeps_per_rep, reps, stream, e0, e1, &own);
       jacc_release(k);
+      pick.ahead = out->best_ms < kAhead * own;
+    } else if (st == JACC_ERR_INVALID_ARG) {
+      st = ok();  // its tile does not cover this many rows
     }
-    pick.ahead = out->best_ms < kAhead * own;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

@@ -566,6 +566,10 @@ static jacc_status specialize(const jacc_kernel_desc* desc, const TunedPick& pic
       tile = native ? default_tile_native(*desc, &own) : default_tile(*desc);
       fit = desc->tblock <= 1 && own;
       if (picked) named = pick.tile;
+      if (picked && !tile_valid(*desc, tile)) {  // only larger tiles cover so many rows
+        tile = pick.tile;
+        fit = false;
+      }
     }
   }
   if (!tile_valid(*desc, tile))

@@ -74,3 +74,20 @@ def test_a_model_pick_is_named_and_displaces_nothing():
     assert not fallback
     assert jacc.Kernel(**args).info()["tile_id"] == t
     assert geometry(**args) == own
+
+
+# more rows than the own kernel's tile covers in a grid: only the tiles of eight
+# thread rows and the long march do
+def test_a_grid_that_only_large_tiles_cover_is_tuned():
+    args = dict(stencil=5, dtype=32, nx=3, ny=4194305)
+    with pytest.raises(jacc.JaccError):
+        jacc.Kernel(**args)
+    a, b = fields(args)
+    r = jacc.autotune(args, a, b, sweeps_per_rep=1, reps=1)
+    assert r["valid"][6] and not r["valid"][2]
+    assert torch.equal(result(args), result(dict(args, tile_id=6)))
+    jacc.autotune_forget()
+    m = jacc.CostModel(seed=5)
+    m.set_range(1.0, 1e9, 0.0)
+    t, fallback = m.choose(args)
+    assert not fallback and jacc.Kernel(**args).info()["tile_id"] == t
