@@ -268,7 +268,7 @@ static bool fits_planes(const jacc_kernel_desc& d, int tile, int fam, bool fit) 
 // 97^3 5.5 / 4.8, FP64 97^3 8.8 / 9.1, 129^3 16.9 / 12.8).  Folded kernels of
 // fields that stream from HBM stage by bulk copies (bulk / ring: 7-point FP64
 // 512^3 361 / 398, 320^3 98 / 95; FP32 512^3 164 / 189, 400^3 92 / 92; 27-point
-// FP32 768^3 577 / 610, 512^3 195 / 179), of the precompiled ones only the FP32
+// FP32 768^3 573 / 610, 512^3 190 / 179), of the precompiled ones only the FP32
 // 7-point kernel (512^3 164 / 170); the rest asynchronous copies (precompiled,
 // ring / bulk: 7-point FP64 512^3 396 / 480, 27-point FP32 768^3 604 / 748).
 static int default_family(const jacc_kernel_desc& d, int tile, bool native) {
