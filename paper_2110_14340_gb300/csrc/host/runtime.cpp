@@ -245,8 +245,9 @@ static int table_family(const jacc_kernel_desc& d, int tile, int fpath) {
   const bool direct = d.stencil == 7 && JACC_DIRECT_TILE(c.bx, c.by, c.vec16 ? 2 : 1), fits = direct_fits(d);
   const int64_t n = d.nx * d.ny * d.nz;
   // native FP64, us a sweep of tile 4 without staging and with its planes in
-  // registers: 33^3 19 / 22, 101^3 40 / 43, 128^3 52 / 58, 192 x 160 x 144 122 / 109
-  if (native_fp64(d, fpath)) return direct && fits && n <= (int64_t(1) << 21) ? JACC_FAM_TABLE : JACC_FAM_NATIVE;
+  // registers: 33^3 5.4 / 22, 101^3 31 / 43, 128^3 46 / 58, 192 x 160 x 144
+  // 95 / 108
+  if (native_fp64(d, fpath)) return direct && fits && n <= (int64_t(1) << 24) ? JACC_FAM_TABLE : JACC_FAM_NATIVE;
   const bool large = d.dtype == 64 && n > (int64_t(1) << 20);
   return direct && (large || !fits) ? JACC_FAM_RING : JACC_FAM_TABLE;
 }
@@ -360,8 +361,8 @@ static std::string key_of(const jacc_kernel_desc& d, int tile, bool fit, int nam
 }
 
 // Planes per CTA (3D) or rows per warp (2D) of a kernel that takes what fits
-// the grid.  3D: at most the tile's own, and few enough that the grid has at least 2.5 times the
-// CTAs that the device holds at once.  With fewer, the last wave leaves SMs
+// the grid.  3D: at most the tile's own, and few enough that the grid has at
+// least 2.5 times the CTAs that the device holds at once.  With fewer, the last wave leaves SMs
 // idle: 301 x 253 x 199 FP64 at 64 planes (640 CTAs on 152 SMs) 65.2 us a
 // sweep, at 16 planes (2080) 55.7, at 8 (4000) 57.3; 511^3, whose grid is
 // large either way, within 3 % from 8 to 64.
@@ -453,9 +454,9 @@ static int plane_chunk(const jacc_kernel_desc& d, int tile, int fam) {
 
 // The NVRTC source of a folded variant: the device text plus a struct whose
 // static constexpr members replace JParams, and the kernels: jacc_jit for the
-// intermediate (and every FP32 or native) sweeps, and for FP64 jacc_jit_out,
-// in fixed point which converts FP64 on load and store, and jacc_jit_last, only
-// on store.
+// intermediate (and every FP32 or native) sweeps, and in fixed point
+// jacc_jit_out, which converts FP64 on load and store, and jacc_jit_last, only on
+// store.
 static std::string jit_source(const Kernel& k) {
   const JParams& p = k.params;
   const TileCfg& c = kTiles[k.tile];

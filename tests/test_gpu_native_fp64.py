@@ -65,3 +65,21 @@ def test_native_fp64_follows_the_definition(stencil, coeffs, tile, jit, nx, ny, 
     out = torch.zeros_like(u)
     jacc.launch(k, u, out, res)
     assert torch.equal(out, b)
+
+
+# the scalar 32 x 8 tiles stage nothing up to 2^24 points, the library's choice neither
+@pytest.mark.parametrize("nx,ny,nz", [(161, 131, 101), (256, 256, 256), (257, 256, 256)])
+@pytest.mark.parametrize("tile", [-1, 4, 6])
+def test_native_heat3d_of_large_grids_equals_tile_0(tile, nx, ny, nz):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(57)
+    u = torch.rand((nz, ny, nx), generator=g, device="cuda", dtype=torch.float64)
+    out = []
+    for t in (tile, 0):
+        k = jacc.Kernel(7, jacc.F64, nx, ny, nz, coeffs=(0.1,), tile_id=t, arith=jacc.ARITH_NATIVE)
+        a, b = u.clone(), torch.zeros_like(u)
+        res = torch.full((3,), -1.0, dtype=torch.float64, device="cuda")
+        assert jacc.sweep(k, a, b, 3, res) == 1
+        out.append((a, b, res))
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
