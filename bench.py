@@ -239,9 +239,10 @@ def run_gpu(args):
     stream = torch.cuda.current_stream(dev)
     loops, refs, arrays = region_nest()
 
-    # Set-up (untimed): the exhaustive autotuner picks the tile for this shape
-    # (remembered by the library, so tile_id = -1 resolves to it), then the
-    # constant-folded NVRTC variant of that tile is compiled and cached.
+    # Set-up (untimed): the exhaustive autotuner times the tiles and the library's
+    # own kernel for this shape (remembered: tile_id = -1 takes the fastest tile if
+    # it is ahead, and otherwise only names it), then the constant-folded NVRTC
+    # variant of the choice is compiled and cached.
     tune = None
     if args.tile < 0 and not args.no_tune:
         t0 = time.perf_counter()
@@ -492,7 +493,7 @@ def secondary(dev):
         kk.release()
     bt.release()
     del fields
-    # 27-point FP32 1024^3, 100 sweeps, periodic: plain (autotuned tile, precompiled and
+    # 27-point FP32 1024^3, 100 sweeps, periodic: plain (autotuned, precompiled and
     # constant-folded) vs temporal blocking
     n = 1024
     w = tuple(float(x) for x in inputs.box27_weights())
@@ -504,7 +505,7 @@ def secondary(dev):
     c5 = {}
     c5["plain_ms"] = _time_ms(lambda: jacc.sweep(kp, a, b, 100, res), reps=2)
     c5["plain_tile"] = kp.info()["tile_id"]
-    # the same tile with extents and weights folded as constants (NVRTC)
+    # the same with extents and weights folded as constants (NVRTC)
     kj = jacc.Kernel(27, 32, n, n, n, coeffs=w, jit=True)
     c5["jit_ms"] = _time_ms(lambda: jacc.sweep(kj, a, b, 100, res), reps=2)
     for T in (2,):
